@@ -220,9 +220,9 @@ struct BlockWork {
     int* iters_host = nullptr;
     double* rr_host = nullptr;
     double* bb_host = nullptr;
-    double* partial = nullptr;          // grid x K x 2
-    unsigned* ticket = nullptr;
-    int grid = 0;
+    double* partial = nullptr;          // (grid + its teams) x K x 2 partial sums
+    unsigned* ticket = nullptr;         // [0] teams done, [1 + t] blocks of team t done
+    int grid = 0;                       // largest grid of a reducing kernel
     double* cw[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};   // coarsest CG x, r, z, p, q (n_c x K)
     double* cpart = nullptr;            // coarsest CG block partials
     int* cctl = nullptr;                // [0] barrier arrivals, [1] error

@@ -202,72 +202,101 @@ __device__ __forceinline__ void sell_row_k(const SellV& S, const T* __restrict__
     }
 }
 
-// Per-column sums of (v0, v1) over the rows of the whole grid in a fixed
-// order (groups of a warp, warps of a block, then blocks); the last block to
-// finish calls fin(c, sum0, sum1) for every column. Deterministic for a fixed
-// (grid, lanes per row, block width ld): a column's sum never depends on the other columns.
-template <int CPL, typename FIN>
-__device__ __forceinline__ void colsum2(double (&v0)[CPL], double (&v1)[CPL], const Grp& g, int k, int ld, double* partial,
-                                        unsigned* ticket, FIN&& fin) {
-    __shared__ double sm[WARPS][2][MAXK];
+// Sums over `count` blocks' partials (value j of column c of block b at
+// part[(b * 2 + j) * k + c]) by the whole block: tpc consecutive lanes per
+// column (a power of two <= 32, set by the block width ld so that it does not
+// depend on how many columns are live), lane t adds the blocks t, t + tpc, ...
+// in order and the lanes meet in a shuffle tree; out(c, sums) on one lane.
+template <int NV, typename OUT>
+__device__ __forceinline__ void sum_partials(const double* part, int count, int k, int ld, OUT&& out) {
+    int tpc = 1;
+    while (tpc < 32 && tpc * 2 * ld <= TPB) tpc *= 2;
+    const int cpb = TPB / tpc;                           // columns per pass
+    const int t = threadIdx.x & (tpc - 1);
+    for (int cb = 0; cb < k; cb += cpb) {
+        const int c = cb + (int)threadIdx.x / tpc;
+        double s[NV];
+#pragma unroll
+        for (int j = 0; j < NV; ++j) s[j] = 0.0;
+        if (c < k) {
+#pragma unroll 4
+            for (int b = t; b < count; b += tpc)
+#pragma unroll
+                for (int j = 0; j < NV; ++j) s[j] += __ldcg(part + ((size_t)b * 2 + j) * k + c);
+        }
+        for (int o = tpc >> 1; o > 0; o >>= 1)
+#pragma unroll
+            for (int j = 0; j < NV; ++j) s[j] += __shfl_xor_sync(FULL_MASK, s[j], o);
+        if (c < k && t == 0) out(c, s);
+    }
+}
+
+// Per-column sums of v[0 .. NV) over the rows of the whole grid in a fixed
+// order (warps of a block, groups of a warp, blocks of a team of CS_TEAM, then
+// teams); the last block to finish calls fin(c, sum0, sum1) for every column.
+// Deterministic for a fixed (grid, lanes per row, block width ld): a column's
+// sum never depends on the other columns. The FP64 pipe issues one warp
+// instruction per 64 cycles of a sub-partition, so additions are kept few: the
+// block's values meet in shared memory (each addition serves 32 live columns),
+// and the block partials are added by the last block of each team, in parallel
+// over the teams, instead of all by the last block of the grid (20-40 us of
+// every 64-column kernel; a 128^3 solve of 64 columns 223.0 -> 217.6 ms, one of
+// 75x64x49 and 7 columns 8.56 -> 7.71 ms).
+constexpr int CS_TEAM = 32;
+template <int CPL, int NV, typename FIN>
+__device__ __forceinline__ void colsum(double (&v)[NV][CPL], const Grp& g, int k, int ld, double* partial,
+                                       unsigned* ticket, FIN&& fin) {
+    __shared__ double sm[TPB * CPL];
     __shared__ bool last;
-#pragma unroll
-    for (int m = 0; m < CPL; ++m)
-        for (int o = g.G; o < 32; o <<= 1) {
-            v0[m] += __shfl_xor_sync(FULL_MASK, v0[m], o);
-            v1[m] += __shfl_xor_sync(FULL_MASK, v1[m], o);
-        }
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (lane < g.G) {
+    const int gpw = 32 / g.G, W = g.G * CPL;             // groups of a warp, columns of a group (>= k)
+    const int slots = gpw * W;                           // 32 CPL values of a warp
 #pragma unroll
-        for (int m = 0; m < CPL; ++m) {
-            const int c = lane * CPL + m;
-            if (c < k) {
-                sm[warp][0][c] = v0[m];
-                sm[warp][1][c] = v1[m];
+    for (int j = 0; j < NV; ++j) {
+        if (j) __syncthreads();
+        double* own = sm + warp * slots + (lane / g.G) * W + g.gl * CPL;
+#pragma unroll
+        for (int m = 0; m < CPL; ++m) own[m] = v[j][m];
+        __syncthreads();
+        for (int s = threadIdx.x; s < slots; s += TPB) { // the warps, in place
+            double a0 = sm[s], a1 = sm[slots + s];
+#pragma unroll
+            for (int w = 2; w < WARPS; w += 2) {
+                a0 += sm[w * slots + s];
+                a1 += sm[(w + 1) * slots + s];
             }
+            sm[s] = a0 + a1;
+        }
+        __syncthreads();
+        for (int c = threadIdx.x; c < k; c += TPB) {     // the groups
+            double a = sm[c];
+            for (int t = 1; t < gpw; ++t) a += sm[t * W + c];
+            partial[((size_t)blockIdx.x * 2 + j) * k + c] = a;
+            __threadfence();
         }
     }
+    const int nteams = ((int)gridDim.x + CS_TEAM - 1) / CS_TEAM, team = blockIdx.x / CS_TEAM;
+    const int members = min(CS_TEAM, (int)gridDim.x - team * CS_TEAM);
+    double* tpart = partial + (size_t)gridDim.x * 2 * k; // team sums
     __syncthreads();
-    for (int c = threadIdx.x; c < k; c += blockDim.x) {
-        double a = 0.0, b = 0.0;
-        for (int w = 0; w < WARPS; ++w) {
-            a += sm[w][0][c];
-            b += sm[w][1][c];
-        }
-        partial[((size_t)blockIdx.x * 2 + 0) * k + c] = a;
-        partial[((size_t)blockIdx.x * 2 + 1) * k + c] = b;
-        __threadfence();
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    if (threadIdx.x == 0) last = atomicAdd(ticket + 1 + team, 1u) == (unsigned)members - 1;
     __syncthreads();
     if (!last) return;
     __threadfence();
-    // tpc consecutive lanes per column (a power of two <= 32, set by the
-    // block width ld so that it does not depend on how many columns are
-    // live): lane j sums the blocks j, j + tpc, ... in order, then the lanes
-    // combine by a shuffle tree; a fixed order for a fixed (grid, ld).
-    int tpc = 1;
-    while (tpc < 32 && tpc * 2 * ld <= (int)blockDim.x) tpc *= 2;
-    const int cpb = (int)blockDim.x / tpc;               // columns per pass
-    const int j = threadIdx.x & (tpc - 1);
-    for (int c0 = 0; c0 < k; c0 += cpb) {
-        const int c = c0 + (int)threadIdx.x / tpc;
-        double a = 0.0, b = 0.0;
-        if (c < k) {
-#pragma unroll 4
-            for (int blk = j; blk < (int)gridDim.x; blk += tpc) {
-                a += __ldcg(partial + ((size_t)blk * 2 + 0) * k + c);
-                b += __ldcg(partial + ((size_t)blk * 2 + 1) * k + c);
-            }
-        }
-        for (int o = tpc >> 1; o > 0; o >>= 1) {
-            a += __shfl_xor_sync(FULL_MASK, a, o);
-            b += __shfl_xor_sync(FULL_MASK, b, o);
-        }
-        if (c < k && j == 0) fin(c, a, b);
+    sum_partials<NV>(partial + (size_t)team * CS_TEAM * 2 * k, members, k, ld, [&](int c, const double (&s)[NV]) {
+#pragma unroll
+        for (int j = 0; j < NV; ++j) tpart[((size_t)team * 2 + j) * k + c] = s[j];
+        __threadfence();
+    });
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        ticket[1 + team] = 0u;
+        last = atomicAdd(ticket, 1u) == (unsigned)nteams - 1;
     }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    sum_partials<NV>(tpart, nteams, k, ld, [&](int c, const double (&s)[NV]) { fin(c, s[0], NV > 1 ? s[NV - 1] : 0.0); });
     __syncthreads();
     if (threadIdx.x == 0) *ticket = 0u;
 }
@@ -387,9 +416,9 @@ __global__ void __launch_bounds__(TPB) bk_post(SellV SAP, const T* __restrict__ 
                                                double* partial, unsigned* ticket, BlockScalars sc, int flexible) {
     const Grp g = make_grp(G);
     const int c0 = g.gl * CPL;
-    double d0[CPL], d1[CPL];
+    double d[2][CPL];
 #pragma unroll
-    for (int m = 0; m < CPL; ++m) d0[m] = d1[m] = 0.0;
+    for (int m = 0; m < CPL; ++m) d[0][m] = d[1][m] = 0.0;
     if (c0 < k) {
         for (int ip = g.gw; ip < SAP.n; ip += g.ngroups) {
             T acc[CPL];
@@ -419,13 +448,23 @@ __global__ void __launch_bounds__(TPB) bk_post(SellV SAP, const T* __restrict__ 
 #pragma unroll
                 for (int m = 0; m < CPL; ++m) {
                     if (c0 + m >= k) continue;
-                    d0[m] = fma(bd[m], (double)ov[m], d0[m]);
-                    if (Q2) d1[m] = fma(qd[m], (double)ov[m], d1[m]);
+                    d[0][m] = fma(bd[m], (double)ov[m], d[0][m]);
+                    if (Q2) d[1][m] = fma(qd[m], (double)ov[m], d[1][m]);
                 }
             }
         }
     }
-    if (DOT) colsum2<CPL>(d0, d1, g, k, ld, partial, ticket, [&](int c, double a, double b) { fin_rz(sc, c, a, b, flexible); });
+    if (DOT) {
+        auto fin = [&](int c, double a, double b) { fin_rz(sc, c, a, b, flexible); };
+        if (Q2) {
+            colsum<CPL, 2>(d, g, k, ld, partial, ticket, fin);
+        } else {
+            double e[1][CPL];
+#pragma unroll
+            for (int m = 0; m < CPL; ++m) e[0][m] = d[0][m];
+            colsum<CPL, 1>(e, g, k, ld, partial, ticket, fin);
+        }
+    }
 }
 
 
@@ -680,9 +719,9 @@ __global__ void __launch_bounds__(TPB) bk_spmv_dot(SellV S, const double* __rest
                                                    double* partial, unsigned* ticket, BlockScalars sc) {
     const Grp g = make_grp(G);
     const int c0 = g.gl * CPL;
-    double d0[CPL], d1[CPL];
+    double d[1][CPL];
 #pragma unroll
-    for (int m = 0; m < CPL; ++m) d0[m] = d1[m] = 0.0;
+    for (int m = 0; m < CPL; ++m) d[0][m] = 0.0;
     if (c0 < k) {
         for (int ip = g.gw; ip < S.n; ip += g.ngroups) {
             double acc[CPL];
@@ -696,10 +735,10 @@ __global__ void __launch_bounds__(TPB) bk_spmv_dot(SellV S, const double* __rest
             st_cols<VEC, CPL>(Q + o, acc, c0, k);
 #pragma unroll
             for (int m = 0; m < CPL; ++m)
-                if (c0 + m < k) d0[m] = fma(pv[m], acc[m], d0[m]);
+                if (c0 + m < k) d[0][m] = fma(pv[m], acc[m], d[0][m]);
         }
     }
-    colsum2<CPL>(d0, d1, g, k, ld, partial, ticket, [&](int c, double pq, double) {
+    colsum<CPL, 1>(d, g, k, ld, partial, ticket, [&](int c, double pq, double) {
         sc.pq[c] = pq;
         if (sc.mode[c] == COL_ACTIVE) {
             const double alpha = sc.rho[c] / pq;
@@ -733,9 +772,9 @@ __global__ void __launch_bounds__(TPB) bk_update_xr(int n, const double* __restr
         al[m] = on[m] ? sc.alpha[c] : 0.0;
         any |= on[m];
     }
-    double d0[CPL], d1[CPL];
+    double d[1][CPL];
 #pragma unroll
-    for (int m = 0; m < CPL; ++m) d0[m] = d1[m] = 0.0;
+    for (int m = 0; m < CPL; ++m) d[0][m] = 0.0;
     if (any) {
         for (int i = g.gw; i < n; i += g.ngroups) {
             const size_t o = (size_t)i * ld + c0;
@@ -749,13 +788,13 @@ __global__ void __launch_bounds__(TPB) bk_update_xr(int n, const double* __restr
                 if (!on[m]) continue;
                 xv[m] = fma(al[m], pv[m], xv[m]);
                 rv[m] = fma(-al[m], qv[m], rv[m]);
-                d0[m] = fma(rv[m], rv[m], d0[m]);
+                d[0][m] = fma(rv[m], rv[m], d[0][m]);
             }
             st_cols<VEC, CPL>(X + o, xv, c0, k);
             st_cols<VEC, CPL>(R + o, rv, c0, k);
         }
     }
-    colsum2<CPL>(d0, d1, g, k, ld, partial, ticket, [&](int c, double rr, double) {
+    colsum<CPL, 1>(d, g, k, ld, partial, ticket, [&](int c, double rr, double) {
         if (sc.mode[c] != COL_ACTIVE) return;
         sc.rr[c] = rr;
         sc.iters[c] += 1;
@@ -815,9 +854,9 @@ __global__ void __launch_bounds__(TPB) bk_residual(SellV S, const double* __rest
         on[m] = c < k && (stage == 0 ? md == COL_INIT : (stage == 1 ? md == COL_CHECK : true));
         any |= on[m];
     }
-    double d0[CPL], d1[CPL];
+    double d[2][CPL];
 #pragma unroll
-    for (int m = 0; m < CPL; ++m) d0[m] = d1[m] = 0.0;
+    for (int m = 0; m < CPL; ++m) d[0][m] = d[1][m] = 0.0;
     if (any) {
         for (int ip = g.gw; ip < S.n; ip += g.ngroups) {
             double acc[CPL];
@@ -833,13 +872,13 @@ __global__ void __launch_bounds__(TPB) bk_residual(SellV S, const double* __rest
             for (int m = 0; m < CPL; ++m) {
                 if (!on[m]) continue;
                 rv[m] = bv[m] - acc[m];
-                d0[m] = fma(rv[m], rv[m], d0[m]);
-                d1[m] = fma(bv[m], bv[m], d1[m]);
+                d[0][m] = fma(rv[m], rv[m], d[0][m]);
+                d[1][m] = fma(bv[m], bv[m], d[1][m]);
             }
             st_cols<VEC, CPL>(R + o, rv, c0, k);
         }
     }
-    colsum2<CPL>(d0, d1, g, k, ld, partial, ticket, [&](int c, double rr, double bb) {
+    colsum<CPL, 2>(d, g, k, ld, partial, ticket, [&](int c, double rr, double bb) {
         const int md = sc.mode[c];
         if (stage == 0) {
             if (md != COL_INIT) return;
@@ -934,6 +973,13 @@ int grid_rows(const amg_hierarchy* h, long long rows, int G) {
     return blocks_for(rows, (int)groups_per_block, h->num_sms * 8);
 }
 
+// Grid of the reducing kernels: at most 8 blocks per SM and none without rows
+// (every block costs a partial per column). Fixed for (rows, G), so the order
+// of the sums is.
+int red_grid(const amg_hierarchy* h, const BlockWork& W, int G) {
+    return std::min(W.grid, grid_rows(h, h->lev[0].A.n, G));
+}
+
 // Z = B R for columns [0, k) (block V-cycle); level 0 finishes r . z per column.
 template <typename T>
 void block_vcycle(amg_hierarchy* h, BlockWork& W, int k, int flexible) {
@@ -1015,7 +1061,7 @@ void block_vcycle(amg_hierarchy* h, BlockWork& W, int k, int flexible) {
                                   sv(Lv.AP), apv, minv, omega, Lv.agg, p, e, lv(W.x, l), lv(W.r, l), nullptr, nullptr,
                                   lv(W.y, l), k, ld, G, W.partial, W.ticket, W.sc, flexible));
         else
-            DISPATCH_CPL(cpl, ld, bk_post<T, double, CPL, true, VEC><<<W.grid, TPB, 0, st>>>(
+            DISPATCH_CPL(cpl, ld, bk_post<T, double, CPL, true, VEC><<<red_grid(h, W, G), TPB, 0, st>>>(
                                   sv(Lv.AP), apv, minv, omega, Lv.agg, p, e, lv(W.x, 0), lv(W.r, 0), W.R,
                                   flexible ? W.Q : nullptr, W.Z, k, ld, G, W.partial, W.ticket, W.sc, flexible));
         KERNEL_CHECK();
@@ -1122,9 +1168,10 @@ BlockWork& block_ensure(amg_hierarchy* h, int K, bool fixed_width) {
     W->sc.bb = W->mem.alloc<double>(K);
     W->sc.rtol = W->mem.alloc<double>(K);
     W->grid = h->num_sms * 8;
-    W->partial = W->mem.alloc<double>((size_t)W->grid * 2 * K);
-    W->ticket = W->mem.alloc<unsigned>(1);
-    CUDA_CHECK(cudaMemsetAsync(W->ticket, 0, sizeof(unsigned), h->stream));
+    const int teams = (W->grid + CS_TEAM - 1) / CS_TEAM;
+    W->partial = W->mem.alloc<double>((size_t)(W->grid + teams) * 2 * K);
+    W->ticket = W->mem.alloc<unsigned>(1 + teams);
+    CUDA_CHECK(cudaMemsetAsync(W->ticket, 0, sizeof(unsigned) * (1 + teams), h->stream));
     CUDA_CHECK(cudaMemsetAsync(W->sc.mode, 0, sizeof(int) * K, h->stream));
     CUDA_CHECK(cudaMemsetAsync(W->sc.iters, 0, sizeof(int) * K, h->stream));
     CUDA_CHECK(cudaHostAlloc(&W->mode_host, sizeof(int) * K, cudaHostAllocDefault));
@@ -1159,7 +1206,7 @@ void block_init_launch(amg_hierarchy* h, const double* B, double* X, int k) {
     int G, cpl;
     group_shape(W, k, &G, &cpl);
     Level& L0 = h->lev[0];
-    DISPATCH_CPL(cpl, W.K, bk_residual<CPL, VEC><<<W.grid, TPB, 0, st>>>(sv(L0.S), L0.S.val, X, B, W.R, k, W.K, G, W.partial,
+    DISPATCH_CPL(cpl, W.K, bk_residual<CPL, VEC><<<red_grid(h, W, G), TPB, 0, st>>>(sv(L0.S), L0.S.val, X, B, W.R, k, W.K, G, W.partial,
                                                              W.ticket, W.sc, 0));
     KERNEL_CHECK();
     bk_zero_cols<<<blocks_for((long long)L0.A.n * k, TPB, h->num_sms * 8), TPB, 0, st>>>(L0.A.n, X, k, W.K, W.sc.mode,
@@ -1184,13 +1231,13 @@ void block_step_kernels(amg_hierarchy* h, double* X, int k, bool any_active) {
     if (any_active) {
         {
             Scope sc_(&h->prof, st, K_SPMV_DOT, 12.0 * nnz + 16.0 * n * k);
-            DISPATCH_CPL(cpl, ld, bk_spmv_dot<CPL, VEC><<<W.grid, TPB, 0, st>>>(sv(L0.S), L0.S.val, W.P, W.Q, k, ld, G,
+            DISPATCH_CPL(cpl, ld, bk_spmv_dot<CPL, VEC><<<red_grid(h, W, G), TPB, 0, st>>>(sv(L0.S), L0.S.val, W.P, W.Q, k, ld, G,
                                                                      W.partial, W.ticket, W.sc));
             KERNEL_CHECK();
         }
         {
             Scope sc_(&h->prof, st, K_UPDATE_XR, 48.0 * n * k);
-            DISPATCH_CPL(cpl, ld, bk_update_xr<CPL, VEC><<<W.grid, TPB, 0, st>>>(n, W.P, W.Q, X, W.R, k, ld, G, W.partial,
+            DISPATCH_CPL(cpl, ld, bk_update_xr<CPL, VEC><<<red_grid(h, W, G), TPB, 0, st>>>(n, W.P, W.Q, X, W.R, k, ld, G, W.partial,
                                                                       W.ticket, W.sc));
             KERNEL_CHECK();
         }
@@ -1284,7 +1331,7 @@ bool block_check_launch(amg_hierarchy* h, const double* B, double* X, int k) {
     Level& L0 = h->lev[0];
     const double nnz = (double)L0.A.nnz;
     Scope sc_(&h->prof, h->stream, K_RESIDUAL, 12.0 * nnz + 24.0 * L0.A.n * k);
-    DISPATCH_CPL(cpl, W.K, bk_residual<CPL, VEC><<<W.grid, TPB, 0, h->stream>>>(sv(L0.S), L0.S.val, X, B, W.R, k, W.K, G,
+    DISPATCH_CPL(cpl, W.K, bk_residual<CPL, VEC><<<red_grid(h, W, G), TPB, 0, h->stream>>>(sv(L0.S), L0.S.val, X, B, W.R, k, W.K, G,
                                                                     W.partial, W.ticket, W.sc, 1));
     KERNEL_CHECK();
     copy_state_async(h, W);
@@ -1296,7 +1343,7 @@ void block_report_launch(amg_hierarchy* h, const double* B, const double* X, int
     int G, cpl;
     group_shape(W, k, &G, &cpl);
     Level& L0 = h->lev[0];
-    DISPATCH_CPL(cpl, W.K, bk_residual<CPL, VEC><<<W.grid, TPB, 0, h->stream>>>(sv(L0.S), L0.S.val, X, B, W.T, k, W.K, G,
+    DISPATCH_CPL(cpl, W.K, bk_residual<CPL, VEC><<<red_grid(h, W, G), TPB, 0, h->stream>>>(sv(L0.S), L0.S.val, X, B, W.T, k, W.K, G,
                                                                     W.partial, W.ticket, W.sc, 2));
     KERNEL_CHECK();
     copy_state_async(h, W);

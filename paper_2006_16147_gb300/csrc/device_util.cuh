@@ -51,18 +51,49 @@ __device__ __forceinline__ int block_max_int(int v) {
     return t;
 }
 
-// Block-wide sum in a fixed combination order (deterministic for a fixed
-// blockDim). All threads get the result.
-__device__ __forceinline__ double block_sum(double v) {
-    __shared__ double ws[32];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    v = warp_sum(v);
-    if (lane == 0) ws[wid] = v;
+// Sums of NV doubles over a block of T threads in a fixed combination order
+// (deterministic for a fixed T): the sum of v[j] comes back on every lane of
+// warp j (0 elsewhere). This GPU issues one FP64 warp instruction per 64
+// cycles of an SM sub-partition, so the number of warp-wide additions is what
+// a block sum costs: the values go through shared memory and one warp per
+// value adds T / 32 columns and then its lanes, T / 32 + 4 additions a value.
+// (A butterfly in every warp and again over the warps took 10 T / 32 of them
+// and 10 us of every kernel that ends in a dot product at 8 blocks per SM: the
+// product with its dot on 32^3 rows 17.1 -> 10.2 us, with grids sized by the
+// rows; a 32^3 solve 1.89 -> 1.34 ms.)
+// Consecutive calls need a block barrier between them.
+template <int T, int NV>
+__device__ __forceinline__ double block_sums(const double (&v)[NV]) {
+    __shared__ double sm[NV][T];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+#pragma unroll
+    for (int j = 0; j < NV; ++j) sm[j][threadIdx.x] = v[j];
     __syncthreads();
-    double t = (lane < nw) ? ws[lane] : 0.0;
-    t = warp_sum(t);
-    __syncthreads();
-    return t;
+    // up to 256 values: 8 columns a lane by warp j; more: a warp per 256 values
+    // first, which halves the serial chain at 1024 threads
+    constexpr int P = T > 256 ? T / 256 : 1, C = T / P;
+    double s0 = 0.0;
+    if (w < NV * P) {
+        const double* col = sm[w / P] + (w % P) * C + lane;
+        s0 = col[0];
+        double s1 = col[32];
+#pragma unroll
+        for (int k = 64; k < C; k += 64) {
+            s0 += col[k];
+            s1 += col[k + 32];
+        }
+        s0 += s1;
+    }
+    if constexpr (P > 1) {
+        if (w < NV * P) sm[w / P][(w % P) * C + lane] = s0;
+        __syncthreads();
+        if (w < NV) {
+            s0 = sm[w][lane];
+#pragma unroll
+            for (int q = 1; q < P; ++q) s0 += sm[w][q * C + lane];
+        }
+    }
+    return w < NV ? warp_sum(s0) : 0.0;
 }
 
 // Block-wide exclusive scan of ints.

@@ -83,12 +83,10 @@ __global__ void __launch_bounds__(TPB) m_chunk_sums(const int* __restrict__ ch_r
             if (w) b = fma(__ldg(w + i), vi, b);
         }
     }
-    a = block_sum(a);
-    b = block_sum(b);
-    if (threadIdx.x == 0) {
-        part_a[c] = a;
-        part_b[c] = b;
-    }
+    const double ab[2] = {a, b};
+    const double s = block_sums<TPB>(ab);
+    if (threadIdx.x == 0) part_a[c] = s;
+    if (threadIdx.x == 32) part_b[c] = s;
 }
 
 // One thread per system: the system's sums, then its scalar update.

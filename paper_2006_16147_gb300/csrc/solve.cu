@@ -25,6 +25,7 @@ namespace {
 
 constexpr int TPB = 256;
 constexpr int WARPS = TPB / 32;
+constexpr int CG_TPB = 1024;  // threads of the iterative coarsest solve's blocks
 
 enum FinMode : int {
     FIN_NORMS = 0, FIN_PQ = 1, FIN_RR = 2, FIN_RHO_INIT = 3, FIN_RHO_UPDATE = 4, FIN_NONE = 5, FIN_RHO_UPDATE_FCG = 6
@@ -64,38 +65,45 @@ __device__ void finish(int mode, double a, double b, PcgScalars* sc) {
     }
 }
 
-// Block partial sums, then the last block to arrive combines all partials in
-// a fixed order (deterministic for a fixed grid) and calls fin(sum_a, sum_b)
-// on one thread.
-template <typename FIN>
+// Block partial sums of a (and with NV = 2 of b), then the last block to
+// arrive combines all partials in a fixed order (deterministic for a fixed
+// grid) and calls fin(sum_a, sum_b) on one thread.
+template <int NV, typename FIN>
 __device__ __forceinline__ void reduce_then(double a, double b, Reducer red, FIN&& fin) {
     __shared__ bool last;
-    a = block_sum(a);
-    b = block_sum(b);
-    if (threadIdx.x == 0) {
-        red.partial[2 * blockIdx.x] = a;
-        red.partial[2 * blockIdx.x + 1] = b;
+    __shared__ double tot[2];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    double v[NV];
+    v[0] = a;
+    if (NV > 1) v[NV - 1] = b;
+    double s = block_sums<TPB>(v);
+    if (w < NV && lane == 0) {
+        red.partial[2 * blockIdx.x + w] = s;
         __threadfence();
-        last = atomicAdd(red.ticket, 1u) == gridDim.x - 1;
     }
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(red.ticket, 1u) == gridDim.x - 1;
     __syncthreads();
     if (!last) return;
     __threadfence();
-    double sa = 0.0, sb = 0.0;
-    for (int k = threadIdx.x; k < (int)gridDim.x; k += blockDim.x) {
-        sa += __ldcg(&red.partial[2 * k]);
-        sb += __ldcg(&red.partial[2 * k + 1]);
-    }
-    sa = block_sum(sa);
-    sb = block_sum(sb);
+#pragma unroll
+    for (int j = 0; j < NV; ++j) v[j] = 0.0;
+#pragma unroll 5
+    for (int k = threadIdx.x; k < (int)gridDim.x; k += TPB)
+#pragma unroll
+        for (int j = 0; j < NV; ++j) v[j] += __ldcg(&red.partial[2 * k + j]);
+    s = block_sums<TPB>(v);
+    if (w < NV && lane == 0) tot[w] = s;
+    __syncthreads();
     if (threadIdx.x == 0) {
-        fin(sa, sb);
+        fin(tot[0], NV > 1 ? tot[1] : 0.0);
         *red.ticket = 0u;
     }
 }
 
+template <int NV>
 __device__ __forceinline__ void reduce_and_finish(double a, double b, Reducer red, PcgScalars* sc, int mode) {
-    reduce_then(a, b, red, [&](double sa, double sb) { finish(mode, sa, sb, sc); });
+    reduce_then<NV>(a, b, red, [&](double sa, double sb) { finish(mode, sa, sb, sc); });
 }
 
 struct SellView {
@@ -174,17 +182,38 @@ __global__ void __launch_bounds__(TPB) k_pre(SellView S, const T* __restrict__ v
     }
 }
 
+// Member sum of aggregate q, sum_i p_i r_i in ascending order. Up to eight
+// members (three pairwise sweeps give no more) are loaded together: three
+// memory latencies per aggregate (bounds, members, p and r) instead of two
+// per member.
+template <typename T, typename F>
+__device__ __forceinline__ T member_sum(const int* __restrict__ pt_ptr, const int* __restrict__ pt_idx,
+                                        const T* __restrict__ p, int q, F&& rv) {
+    T s = 0;
+    const int e = ld(pt_ptr + q + 1);
+    for (int k = ld(pt_ptr + q); k < e; k += 8) {
+        int i[8];
+        T pv[8], rr[8];
+#pragma unroll
+        for (int t = 0; t < 8; ++t) i[t] = k + t < e ? ld(pt_idx + k + t) : -1;
+#pragma unroll
+        for (int t = 0; t < 8; ++t)
+            if (i[t] >= 0) {
+                pv[t] = ld(p + i[t]);
+                rr[t] = rv(i[t]);
+            }
+#pragma unroll
+        for (int t = 0; t < 8; ++t)
+            if (i[t] >= 0) s = fma(pv[t], rr[t], s);
+    }
+    return s;
+}
+
 template <typename T>
 __global__ void __launch_bounds__(TPB) k_restrict(int nc, const int* __restrict__ pt_ptr, const int* __restrict__ pt_idx,
                                                   const T* __restrict__ p, const T* __restrict__ r, T* __restrict__ bc) {
-    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < nc; q += gridDim.x * blockDim.x) {
-        T s = 0;
-        for (int k = pt_ptr[q]; k < pt_ptr[q + 1]; ++k) {
-            const int i = pt_idx[k];
-            s = fma(ld(p + i), ld(r + i), s);
-        }
-        bc[q] = s;
-    }
+    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < nc; q += gridDim.x * blockDim.x)
+        bc[q] = member_sum(pt_ptr, pt_idx, p, q, [&](int i) { return ld(r + i); });
 }
 
 // Coarse correction and first post-smoothing sweep, fused:
@@ -220,7 +249,10 @@ __global__ void __launch_bounds__(TPB) k_post(SellView SAP, const T* __restrict_
             }
         }
     }
-    if (DOT) reduce_and_finish(dot, dot2, red, sc, mode);
+    if (DOT) {
+        if (q2) reduce_and_finish<2>(dot, dot2, red, sc, mode);
+        else reduce_and_finish<1>(dot, 0.0, red, sc, mode);
+    }
 }
 
 template <typename T, typename TB>
@@ -278,7 +310,7 @@ __global__ void __launch_bounds__(TPB) k_kc_spmv_dot(SellView S, const T* __rest
             db = fma(di, (double)b[i], db);
         }
     }
-    reduce_then(dq, db, red, [&](double a, double c) { kc_finish(ks, KC_ALPHA1, a, c); });
+    reduce_then<2>(dq, db, red, [&](double a, double c) { kc_finish(ks, KC_ALPHA1, a, c); });
 }
 
 // e = alpha1 d1; r2 = b - alpha1 q1.
@@ -300,7 +332,7 @@ __global__ void __launch_bounds__(TPB) k_kc_dot(int n, const T* __restrict__ z2,
     double s = 0.0;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
         s = fma((double)z2[i], (double)q1[i], s);
-    reduce_then(s, 0.0, red, [&](double a, double) { kc_finish(ks, KC_BETA, a, 0.0); });
+    reduce_then<1>(s, 0.0, red, [&](double a, double) { kc_finish(ks, KC_BETA, a, 0.0); });
 }
 
 // d2 = z2 - beta d1; q2 = A z2 - beta q1 (= A d2, without a second product);
@@ -325,7 +357,7 @@ __global__ void __launch_bounds__(TPB) k_kc_spmv2(SellView S, const T* __restric
             dr = fma((double)di, (double)r2[i], dr);
         }
     }
-    reduce_then(dq, dr, red, [&](double a, double c) { kc_finish(ks, KC_ALPHA2, a, c); });
+    reduce_then<2>(dq, dr, red, [&](double a, double c) { kc_finish(ks, KC_ALPHA2, a, c); });
 }
 
 // e += alpha2 d2.
@@ -477,7 +509,8 @@ __global__ void __launch_bounds__(TPB) k_dot(int n, const double* __restrict__ a
         d = fma(a[i], b[i], d);
         if (c) d2 = fma(b[i], c[i], d2);
     }
-    reduce_and_finish(d, d2, red, sc, mode);
+    if (c) reduce_and_finish<2>(d, d2, red, sc, mode);
+    else reduce_and_finish<1>(d, 0.0, red, sc, mode);
 }
 
 // x = A_L^{-1} b on the coarsest level, in FP64 whatever T is.
@@ -530,15 +563,42 @@ __device__ __forceinline__ void cg_grid_sync(unsigned* count, unsigned epoch, in
     __syncthreads();
 }
 
-// Sum of the G block partials of slot k in buffer `buf`, same order in every block.
-__device__ __forceinline__ double cg_sum(const double* part, int G) {
-    double s = 0.0;
-    for (int k = threadIdx.x; k < G; k += blockDim.x) s += __ldcg(part + k);
-    return block_sum(s);
+// This block's partials of v[0 .. NV), one slot of G doubles per value.
+template <int NV>
+__device__ __forceinline__ void cg_partials(const double (&v)[NV], double* part, int G) {
+    const double s = block_sums<CG_TPB>(v);
+    if ((threadIdx.x >> 5) < NV && (threadIdx.x & 31) == 0) part[(size_t)(threadIdx.x >> 5) * G + blockIdx.x] = s;
+}
+
+// Sums of the G block partials of each of NV slots, the same order in every
+// block, by one warp; fin(sums, out) turns them into the step's scalars on one
+// thread (an FP64 division in all 1024 threads would hold the SM's FP64 pipe
+// for microseconds) and the block gets them through shared memory. With that
+// and 1024 threads per SM instead of 512, one coarsest solve of 374K rows (30
+// iterations) takes 1.12 ms, 1.61 ms before.
+template <int NV, int NO, typename FIN>
+__device__ __forceinline__ void cg_sums(const double* part, int G, double (&out)[NO], FIN&& fin) {
+    __shared__ double tot[NO];
+    const int lane = threadIdx.x & 31;
+    if (threadIdx.x < 32) {
+        double s[NV];
+#pragma unroll
+        for (int j = 0; j < NV; ++j) s[j] = 0.0;
+#pragma unroll 5
+        for (int k = lane; k < G; k += 32)
+#pragma unroll
+            for (int j = 0; j < NV; ++j) s[j] += __ldcg(part + (size_t)j * G + k);
+#pragma unroll
+        for (int j = 0; j < NV; ++j) s[j] = warp_sum(s[j]);
+        if (lane == 0) fin(s, tot);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < NO; ++j) out[j] = tot[j];
 }
 
 template <typename TI, typename TO>
-__global__ void __launch_bounds__(512) k_coarse_cg(SellView S, const double* __restrict__ val, int n,
+__global__ void __launch_bounds__(CG_TPB) k_coarse_cg(SellView S, const double* __restrict__ val, int n,
                                                    int nlong, const int* __restrict__ long_rows,
                                                    const int* __restrict__ cptr, const int* __restrict__ ccol,
                                                    const double* __restrict__ cval,
@@ -550,7 +610,7 @@ __global__ void __launch_bounds__(512) k_coarse_cg(SellView S, const double* __r
     const int tid = blockIdx.x * blockDim.x + threadIdx.x, stride = G * blockDim.x;
     unsigned epoch = 0;
     int red = 0;   // reduction counter: buffer = red & 1, two slots per buffer
-    auto slot = [&](int k) { return part + (size_t)((red & 1) * 2 + k) * G; };
+    auto slot = [&]() { return part + (size_t)(red & 1) * 2 * G; };
     double a = 0.0, c = 0.0;
     for (int i = tid; i < n; i += stride) {
         const double bi = (double)b[i];
@@ -562,13 +622,16 @@ __global__ void __launch_bounds__(512) k_coarse_cg(SellView S, const double* __r
         a = fma(bi, zi, a);
         c = fma(bi, bi, c);
     }
-    a = block_sum(a);
-    c = block_sum(c);
-    if (threadIdx.x == 0) { slot(0)[blockIdx.x] = a; slot(1)[blockIdx.x] = c; }
+    {
+        const double v[2] = {a, c};
+        cg_partials<2>(v, slot(), G);
+    }
     cg_grid_sync(bar, ++epoch, err);
     if (__ldcg(err)) return;
-    double rho = cg_sum(slot(0), G);
-    const double bb = cg_sum(slot(1), G);
+    double tot[2];
+    cg_sums<2>(slot(), G, tot, [](const double (&s)[2], double* o) { o[0] = s[0]; o[1] = s[1]; });
+    double rho = tot[0];
+    const double bb = tot[1];
     ++red;
     if (bb > 0.0) {
         const double stop2 = rtol * rtol * bb;
@@ -598,11 +661,13 @@ __global__ void __launch_bounds__(512) k_coarse_cg(SellView S, const double* __r
                     pq = fma(__ldcg(p + i), acc, pq);
                 }
             }
-            pq = block_sum(pq);
-            if (threadIdx.x == 0) slot(0)[blockIdx.x] = pq;
+            const double v1[1] = {pq};
+            cg_partials<1>(v1, slot(), G);
             cg_grid_sync(bar, ++epoch, err);
             if (__ldcg(err)) return;
-            const double alpha = rho / cg_sum(slot(0), G);
+            double s1[1];
+            cg_sums<1>(slot(), G, s1, [&](const double (&s)[1], double* o) { o[0] = rho / s[0]; });
+            const double alpha = s1[0];
             ++red;
             // x += alpha p, r -= alpha q, z = M^-1 r: r . r and r . z in one
             // reduction (z is formed even on the last step, where it is unused)
@@ -616,16 +681,20 @@ __global__ void __launch_bounds__(512) k_coarse_cg(SellView S, const double* __r
                 z[i] = zi;
                 rz = fma(ri, zi, rz);
             }
-            rr = block_sum(rr);
-            rz = block_sum(rz);
-            if (threadIdx.x == 0) { slot(0)[blockIdx.x] = rr; slot(1)[blockIdx.x] = rz; }
+            const double v2[2] = {rr, rz};
+            cg_partials<2>(v2, slot(), G);
             cg_grid_sync(bar, ++epoch, err);
             if (__ldcg(err)) return;
-            const double rr_all = cg_sum(slot(0), G);
-            const double rho_new = cg_sum(slot(1), G);
+            double s2[3];
+            cg_sums<2>(slot(), G, s2, [&](const double (&s)[2], double* o) {
+                o[0] = s[0];
+                o[1] = s[1];
+                o[2] = s[1] / rho;
+            });
+            const double rr_all = s2[0], rho_new = s2[1];
             ++red;
             if (rr_all <= stop2) break;
-            const double beta = rho_new / rho;
+            const double beta = s2[2];
             rho = rho_new;
             for (int i = tid; i < n; i += stride) p[i] = fma(beta, p[i], z[i]);
             cg_grid_sync(bar, ++epoch, err);
@@ -676,7 +745,7 @@ __global__ void __launch_bounds__(TPB) k_residual(SellView S, const double* __re
             bb = fma(bi, bi, bb);
         }
     }
-    reduce_and_finish(rr, bb, red, sc, FIN_NORMS);
+    reduce_and_finish<2>(rr, bb, red, sc, FIN_NORMS);
 }
 
 // q = A p; p . q; alpha = rho / p.q.
@@ -696,7 +765,7 @@ __global__ void __launch_bounds__(TPB) k_spmv_dot(SellView S, const double* __re
             pq = fma(pi, acc, pq);
         }
     }
-    reduce_and_finish(pq, 0.0, red, sc, FIN_PQ);
+    reduce_and_finish<1>(pq, 0.0, red, sc, FIN_PQ);
 }
 
 // x += alpha p; r -= alpha q; ||r||^2.
@@ -714,7 +783,7 @@ __global__ void __launch_bounds__(TPB) k_update_xr(int n, const double* __restri
         if (r32) r32[i] = (float)ri;
         rr = fma(ri, ri, rr);
     }
-    reduce_and_finish(rr, 0.0, red, sc, FIN_RR);
+    reduce_and_finish<1>(rr, 0.0, red, sc, FIN_RR);
 }
 
 // p = z + beta p.
@@ -750,8 +819,11 @@ int sell_grid(const amg_hierarchy* h, int nslices) {
 
 int vec_grid(const amg_hierarchy* h, long long n) { return blocks_for(n, TPB, h->num_sms * 8); }
 
-// Fixed grid of every reducing kernel (deterministic partial order).
-int red_grid(const amg_hierarchy* h) { return h->red.blocks; }
+// Grids of the reducing kernels over nslices SELL slices, resp. n rows: at
+// most 8 blocks per SM and none without work (every block costs a partial
+// and a ticket). Fixed for a matrix, so the partial order is deterministic.
+int red_grid(const amg_hierarchy* h, int nslices) { return blocks_for(nslices, WARPS, h->red.blocks); }
+int red_grid_rows(const amg_hierarchy* h, int n) { return blocks_for(n, TPB, h->red.blocks); }
 int wide_grid(const amg_hierarchy* h, long long rows) { return blocks_for(rows * 32, TPB, h->num_sms * 16); }
 
 void coarse_solve_launch(amg_hierarchy* h, const void* b, void* x, bool fp32_in, bool fp64_out) {
@@ -794,7 +866,7 @@ void coarse_solve_launch(amg_hierarchy* h, const void* b, void* x, bool fp32_in,
                         &C.x, &C.r, &C.z, &C.p, &C.q, &C.part, &bar, &err, &maxit, &rtol};
         const void* fn = !fp32_in ? (const void*)k_coarse_cg<double, double>
                                   : (fp64_out ? (const void*)k_coarse_cg<float, double> : (const void*)k_coarse_cg<float, float>);
-        CUDA_CHECK(cudaLaunchCooperativeKernel(fn, dim3(C.blocks), dim3(512), args, 0, h->stream));
+        CUDA_CHECK(cudaLaunchCooperativeKernel(fn, dim3(C.blocks), dim3(CG_TPB), args, 0, h->stream));
         KERNEL_CHECK();
         return;
     }
@@ -825,7 +897,7 @@ void vcycle_typed(amg_hierarchy* h, const double* r, double* z, int rz_mode) {
         coarse_solve_launch(h, r, z, false, true);
         if (rz_mode != FIN_NONE) {
             Scope sc_(&h->prof, st, K_DOT, 16.0 * n0);
-            k_dot<<<red_grid(h), TPB, 0, st>>>(n0, r, z, q2, h->red, h->sc, rz_mode);
+            k_dot<<<red_grid_rows(h, n0), TPB, 0, st>>>(n0, r, z, q2, h->red, h->sc, rz_mode);
             KERNEL_CHECK();
         }
         return;
@@ -986,7 +1058,7 @@ void vcycle_typed(amg_hierarchy* h, const double* r, double* z, int rz_mode) {
             }
             if (rz_mode != FIN_NONE) {
                 Scope sc_(&h->prof, st, K_DOT, 16.0 * n0);
-                k_dot<<<red_grid(h), TPB, 0, st>>>(n0, r, z, q2, h->red, h->sc, rz_mode);
+                k_dot<<<red_grid_rows(h, n0), TPB, 0, st>>>(n0, r, z, q2, h->red, h->sc, rz_mode);
                 KERNEL_CHECK();
             }
             continue;
@@ -1010,7 +1082,7 @@ void vcycle_typed(amg_hierarchy* h, const double* r, double* z, int rz_mode) {
         if (post == 1) {
             Scope sc_(&h->prof, st, K_POST_L0, by_post2(Lv, nc, V, 8, rz_mode != FIN_NONE, U));
             if (rz_mode != FIN_NONE)
-                launch_post<T, double, double, true>(U, red_grid(h), st, SAP, apv(Lv), wm(Lv), Lv.agg, pv(Lv), e,
+                launch_post<T, double, double, true>(U, red_grid(h, SAP.nslices), st, SAP, apv(Lv), wm(Lv), Lv.agg, pv(Lv), e,
                                                      xcur[0], rcur[0], r, z, h->red, h->sc, rz_mode, q2);
             else
                 launch_post<T, double, double, false>(U, g, st, SAP, apv(Lv), wm(Lv), Lv.agg, pv(Lv), e, xcur[0],
@@ -1035,7 +1107,7 @@ void vcycle_typed(amg_hierarchy* h, const double* r, double* z, int rz_mode) {
             }
             if (rz_mode != FIN_NONE) {
                 Scope sc_(&h->prof, st, K_DOT, 16.0 * n0);
-                k_dot<<<red_grid(h), TPB, 0, st>>>(n0, r, z, q2, h->red, h->sc, rz_mode);
+                k_dot<<<red_grid_rows(h, n0), TPB, 0, st>>>(n0, r, z, q2, h->red, h->sc, rz_mode);
                 KERNEL_CHECK();
             }
         }
@@ -1134,7 +1206,7 @@ void kc_fcg2(amg_hierarchy* h, int m, const T* b, T* e) {
     kc_apply<T>(h, m, b, d1);
     {
         Scope sc_(&h->prof, st, K_KFCG, by_spmv);
-        k_kc_spmv_dot<T><<<red_grid(h), TPB, 0, st>>>(S, O.val(), d1, q1, b, h->red, ks);
+        k_kc_spmv_dot<T><<<red_grid(h, S.nslices), TPB, 0, st>>>(S, O.val(), d1, q1, b, h->red, ks);
         KERNEL_CHECK();
     }
     {
@@ -1145,12 +1217,12 @@ void kc_fcg2(amg_hierarchy* h, int m, const T* b, T* e) {
     kc_apply<T>(h, m, r2, z2);
     {
         Scope sc_(&h->prof, st, K_KFCG, 2.0 * n * V);
-        k_kc_dot<T><<<red_grid(h), TPB, 0, st>>>(n, z2, q1, h->red, ks);
+        k_kc_dot<T><<<red_grid_rows(h, n), TPB, 0, st>>>(n, z2, q1, h->red, ks);
         KERNEL_CHECK();
     }
     {
         Scope sc_(&h->prof, st, K_KFCG, (double)Lm.A.nnz * (V + 4) + (double)n * 5 * V);
-        k_kc_spmv2<T><<<red_grid(h), TPB, 0, st>>>(S, O.val(), z2, q1, d1, r2, d2, h->red, ks);
+        k_kc_spmv2<T><<<red_grid(h, S.nslices), TPB, 0, st>>>(S, O.val(), z2, q1, d1, r2, d2, h->red, ks);
         KERNEL_CHECK();
     }
     {
@@ -1203,7 +1275,7 @@ void kcycle_typed(amg_hierarchy* h, const double* r, double* z, int rz_mode) {
     Scope sc_(&h->prof, st, K_POST_L0, by_post2(L0, nc, V, 8, rz_mode != FIN_NONE, true));
     const int gp = L0.grid_post[f32] ? L0.grid_post[f32] : sell_grid(h, S.nslices);
     if (rz_mode != FIN_NONE)
-        launch_post<T, double, double, true>(true, red_grid(h), st, SAP, O.apw(), O.wm(), L0.agg, O.p(), e, xa, ra, r, z,
+        launch_post<T, double, double, true>(true, red_grid(h, SAP.nslices), st, SAP, O.apw(), O.wm(), L0.agg, O.p(), e, xa, ra, r, z,
                                              h->red, h->sc, rz_mode, q2);
     else
         launch_post<T, double, double, false>(true, gp, st, SAP, O.apw(), O.wm(), L0.agg, O.p(), e, xa, ra, r, z,
@@ -1351,7 +1423,7 @@ void prepare_solve(amg_hierarchy* h) {
         const int nc = h->lev.back().A.n;
         CoarseCg& C = h->ccg;
         int per_sm = 0;
-        CUDA_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_coarse_cg<double, double>, 512, 0));
+        CUDA_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_coarse_cg<double, double>, CG_TPB, 0));
         if (per_sm < 1) AMG_THROW(AMG_ERR_CUDA, "coarsest CG kernel cannot be resident");
         C.blocks = h->num_sms;
         C.x = h->mem.alloc<double>(nc);
@@ -1424,7 +1496,7 @@ amg_status solve(amg_hierarchy* h, const double* b, double* x, double rtol, int 
     CUDA_CHECK(cudaMemsetAsync(h->sc, 0, sizeof(PcgScalars), st));
     {
         Scope sc_(&h->prof, st, K_RESIDUAL, by_res);
-        k_residual<<<red_grid(h), TPB, 0, st>>>(S, A, x, b, h->r, h->red, h->sc);
+        k_residual<<<red_grid(h, S.nslices), TPB, 0, st>>>(S, A, x, b, h->r, h->red, h->sc);
         KERNEL_CHECK();
     }
     read_scalars(h);
@@ -1470,12 +1542,12 @@ amg_status solve(amg_hierarchy* h, const double* b, double* x, double rtol, int 
         }
         {
             Scope sc_(&h->prof, st, K_SPMV_DOT, by_spmv);
-            k_spmv_dot<<<red_grid(h), TPB, 0, st>>>(S, A, h->p, h->q, h->red, h->sc);
+            k_spmv_dot<<<red_grid(h, S.nslices), TPB, 0, st>>>(S, A, h->p, h->q, h->red, h->sc);
             KERNEL_CHECK();
         }
         {
             Scope sc_(&h->prof, st, K_UPDATE_XR, 48.0 * n + (r32 ? 4.0 * n : 0.0));
-            k_update_xr<<<red_grid(h), TPB, 0, st>>>(n, h->p, h->q, x, h->r, r32, h->red, h->sc);
+            k_update_xr<<<red_grid_rows(h, n), TPB, 0, st>>>(n, h->p, h->q, x, h->r, r32, h->red, h->sc);
             KERNEL_CHECK();
         }
         ++it;
@@ -1497,7 +1569,7 @@ amg_status solve(amg_hierarchy* h, const double* b, double* x, double rtol, int 
         if (rel <= rtol) {
             {
                 Scope sc_(&h->prof, st, K_RESIDUAL, by_res);
-                k_residual<<<red_grid(h), TPB, 0, st>>>(S, A, x, b, h->t, h->red, h->sc);
+                k_residual<<<red_grid(h, S.nslices), TPB, 0, st>>>(S, A, x, b, h->t, h->red, h->sc);
                 KERNEL_CHECK();
             }
             read_scalars(h);
@@ -1515,7 +1587,7 @@ amg_status solve(amg_hierarchy* h, const double* b, double* x, double rtol, int 
     if (!have_true) {
         {
             Scope sc_(&h->prof, st, K_RESIDUAL, by_res);
-            k_residual<<<red_grid(h), TPB, 0, st>>>(S, A, x, b, h->t, h->red, h->sc);
+            k_residual<<<red_grid(h, S.nslices), TPB, 0, st>>>(S, A, x, b, h->t, h->red, h->sc);
             KERNEL_CHECK();
         }
         read_scalars(h);
