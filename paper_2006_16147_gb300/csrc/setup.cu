@@ -1501,71 +1501,25 @@ __global__ void k_seg_rows(int m, const int* __restrict__ seg, int* __restrict__
     for (int i = seg[s] + threadIdx.x; i < seg[s + 1]; i += blockDim.x) seg_row[i] = s;
 }
 
-// Dense lower triangle of the diagonal block [r0, r0 + n) (block-diagonal matrix).
-__global__ void k_dense_lower_block(int n, int r0, const int* __restrict__ ptr, const int* __restrict__ col,
-                                    const double* __restrict__ val, double* __restrict__ D) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-        for (int k = ptr[r0 + i]; k < ptr[r0 + i + 1]; ++k) {
-            const int j = col[k] - r0;
-            if (j >= 0 && j <= i) D[(size_t)j * n + i] = val[k];
-        }
-}
-
 // ----------------------------------------------- coarsest: dense Cholesky --
-__global__ void k_dense_lower(int n, const int* __restrict__ ptr, const int* __restrict__ col,
-                              const double* __restrict__ val, double* __restrict__ D) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-        for (int k = ptr[i]; k < ptr[i + 1]; ++k)
-            if (col[k] <= i) D[(size_t)col[k] * n + i] = val[k];
-}
-
-// Left-looking column Cholesky A = L L^T in one block; column-major,
-// sequential sums in k (the textbook order). flag = 1 on a non-positive pivot.
-__global__ void k_cholesky(int n, const double* __restrict__ D, double* __restrict__ L, int* flag) {
-    __shared__ double ljj_s;
-    for (int j = 0; j < n; ++j) {
-        if (threadIdx.x == 0) {
-            double s = D[(size_t)j * n + j];
-            for (int k = 0; k < j; ++k) {
-                const double l = L[(size_t)k * n + j];
-                s = __dsub_rn(s, __dmul_rn(l, l));
-            }
-            if (!(s > 0.0)) { *flag = 1; s = 1.0; }
-            ljj_s = __dsqrt_rn(s);
-            L[(size_t)j * n + j] = ljj_s;
-        }
-        __syncthreads();
-        const double ljj = ljj_s;
-        for (int i = j + 1 + threadIdx.x; i < n; i += blockDim.x) {
-            double t = D[(size_t)j * n + i];
-            for (int k = 0; k < j; ++k) t = __dsub_rn(t, __dmul_rn(L[(size_t)k * n + i], L[(size_t)k * n + j]));
-            L[(size_t)j * n + i] = __ddiv_rn(t, ljj);
-        }
-        __syncthreads();
-    }
-}
-
 // The whole coarsest-level inverse of one diagonal block per CTA: the dense
 // lower triangle from the block's CSR rows, the factor L, Y = L^{-1} and
 // A^{-1} = Y^T Y (row-major, at Ainv + blk[s]); L is also written when Lout
 // is set. Factor and inverse are right-looking: as soon as column j of L (or
-// row k of Y) is final, every entry it touches takes its update at once. Each
-// entry still sees the same operations in the same order as in k_cholesky /
-// k_lower_inverse / k_gram (updates in ascending k, the same roundings), so
-// the bits are the same; the dependent chain is O(n) barrier steps instead of
-// O(n^2) serial operations. A block of n <= SM_DENSE rows works in shared
-// memory, a larger one in gwork + gofs[s] (2 n^2 doubles). segp == nullptr
-// means a single block of rows [0, n0).
+// row k of Y) is final, every entry it touches takes its update at once, in
+// ascending k as in the textbook recurrences; the dependent chain is O(n)
+// barrier steps. A block of n <= SM_DENSE rows works in shared memory, a
+// larger one in gwork + gofs[s] (2 n^2 doubles). Used for a batch of systems,
+// whose blocks fill the chip; one block alone takes k_dense_inverse.
 constexpr int SM_DENSE = 96;
 constexpr int CTA_DENSE = 256;      // largest block one CTA factors (its n^3 FP64 work runs on one SM)
-__global__ void k_coarse_inverse_blocks(int n0, const int* __restrict__ segp, const long long* __restrict__ blk,
+__global__ void k_coarse_inverse_blocks(const int* __restrict__ segp, const long long* __restrict__ blk,
                                         const long long* __restrict__ gofs, const int* __restrict__ ptr,
                                         const int* __restrict__ col, const double* __restrict__ val,
-                                        double* __restrict__ gwork, double* __restrict__ Ainv,
-                                        double* __restrict__ Lout, int* flag) {
+                                        double* __restrict__ gwork, double* __restrict__ Ainv, int* flag) {
     const int sg = blockIdx.x;
-    const int r0 = segp ? segp[sg] : 0;
-    const int n = segp ? segp[sg + 1] - r0 : n0;
+    const int r0 = segp[sg];
+    const int n = segp[sg + 1] - r0;
     if (n <= 0) return;
     extern __shared__ double sm_dense[];
     __shared__ double dg[SM_DENSE];
@@ -1607,37 +1561,178 @@ __global__ void k_coarse_inverse_blocks(int n0, const int* __restrict__ segp, co
         }
         __syncthreads();
     }
-    double* Ai = Ainv + (segp ? blk[sg] : 0);
+    double* Ai = Ainv + blk[sg];
     for (int t = threadIdx.x; t < n * n; t += blockDim.x) {
         const int i = t / n, j = t % n;
         double s = 0.0;
         for (int k = max(i, j); k < n; ++k) s = fma(Ys[i * n + k], Ys[j * n + k], s);
         Ai[t] = s;
-        if (Lout) Lout[t] = j > i ? M[t] : (j == i ? diag[i] : 0.0);   // t = column i, row j
     }
 }
 
-// Y = L^{-1} (column-major, lower), one column per thread.
-__global__ void k_lower_inverse(int n, const double* __restrict__ L, double* __restrict__ Y) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= n) return;
-    for (int i = 0; i < c; ++i) Y[(size_t)c * n + i] = 0.0;
-    Y[(size_t)c * n + c] = 1.0 / L[(size_t)c * n + c];
-    for (int i = c + 1; i < n; ++i) {
-        double t = 0.0;
-        for (int k = c; k < i; ++k) t = fma(L[(size_t)k * n + i], Y[(size_t)c * n + k], t);
-        Y[(size_t)c * n + i] = -t / L[(size_t)i * n + i];
-    }
-}
+// The same inverse of one dense block of rows [r0, r0 + n), in one cooperative
+// launch over many CTAs: panels of DI_NB columns. Every entry takes its updates
+// in ascending k with the same roundings as in k_coarse_inverse_blocks, so the
+// bits are the same.
+//   panel   every CTA factors the DI_NB x DI_NB diagonal block (redundantly:
+//           that saves a grid barrier) and carries one unit of DI_NB vectors
+//           through the same elimination steps: rows of L below the block, or
+//           columns of Y = L^{-1}; n / DI_NB units in all, one per CTA
+//   update  M <- M - L L^T and Y <- Y + L Y behind the panel, tiles of 8 x 32
+//           entries spread over the grid
+// and after the last panel A^{-1} = Y^T Y in the same tiles. What bounds it is
+// the chain of n pivots (a square root, a division and an update each, about
+// 1.2 us at this GPU's FP64 latency); the column that holds the next pivot is
+// updated by the two warps that then divide it, beside the other columns'
+// updates, so a step costs one block barrier and little more than that chain.
+// M and Y are row-major n x n scratch, zero on entry; M takes the lower
+// triangle from the CSR. ctl: [0] barrier arrivals, [1] a wait gave up,
+// [2] non-positive pivot.
+constexpr int DI_NB = 32;
+constexpr int DI_T = 256;
+constexpr int DI_R = DI_T / 32;     // rows of an update tile, one per warp
 
-// Ainv = Y^T Y (row-major).
-__global__ void k_gram(int n, const double* __restrict__ Y, double* __restrict__ Ainv) {
-    const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (t >= (long long)n * n) return;
-    const int i = (int)(t / n), j = (int)(t % n);
-    double s = 0.0;
-    for (int k = max(i, j); k < n; ++k) s = fma(Y[(size_t)i * n + k], Y[(size_t)j * n + k], s);
-    Ainv[(size_t)i * n + j] = s;
+__global__ void __launch_bounds__(DI_T) k_dense_inverse(int n, int r0, const int* __restrict__ ptr,
+                                                        const int* __restrict__ col, const double* __restrict__ val,
+                                                        double* M, double* Y, double* __restrict__ Ainv,
+                                                        double* __restrict__ Lout, int* ctl) {
+    __shared__ double dg[DI_NB][DI_NB + 1];   // diagonal block; operand tile of the updates
+    __shared__ double un[DI_NB][DI_NB + 1];   // unit: vector v, entry k; operand rows of the updates
+    __shared__ double pv[DI_NB];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, G = gridDim.x;
+    unsigned* bar = reinterpret_cast<unsigned*>(ctl);
+    int* err = ctl + 1;
+    unsigned epoch = 0;
+    auto at = [n](int i, int j) { return (size_t)i * n + j; };
+    for (int i = blockIdx.x * DI_R + w; i < n; i += G * DI_R)
+        for (int k = ptr[r0 + i] + lane; k < ptr[r0 + i + 1]; k += 32) {
+            const int j = col[k] - r0;
+            if (j >= 0 && j <= i) M[at(i, j)] = val[k];
+        }
+    grid_sync(bar, ++epoch, err);
+    if (__ldcg(err)) return;
+    for (int j0 = 0; j0 < n; j0 += DI_NB) {
+        const int nb = min(DI_NB, n - j0), j1 = j0 + nb;
+        const int um = (n - j1 + DI_NB - 1) / DI_NB, units = um + (j1 + DI_NB - 1) / DI_NB;
+        for (int u = blockIdx.x; u < units; u += G) {
+            const bool isL = u < um;                              // rows of L, else columns of Y
+            const int v0 = isL ? j1 + u * DI_NB : (u - um) * DI_NB;
+            const int nv = isL ? min(DI_NB, n - v0) : min(DI_NB, j1 - v0);
+            for (int t = w; t < DI_NB; t += DI_R) {
+                dg[t][lane] = t < nb && lane <= t ? __ldcg(M + at(j0 + t, j0 + lane)) : 0.0;
+                if (isL) un[t][lane] = t < nv && lane < nb ? __ldcg(M + at(v0 + t, j0 + lane)) : 0.0;
+                else un[lane][t] = lane < nv && t < nb ? __ldcg(Y + at(j0 + t, v0 + lane)) : 0.0;
+            }
+            __syncthreads();
+            // one more update and the division of column j (warp 0: the
+            // diagonal block, warp 1: the unit); the pivot entry itself stays
+            // for the other warp to read
+            auto column = [&](int j) {
+                double s = dg[j][j];
+                double x = w == 0 ? dg[lane][j] : un[lane][j];
+                if (j > 0) {
+                    const double l = dg[j][j - 1];
+                    const double y = w == 0 ? dg[lane][j - 1] : un[lane][j - 1];
+                    s = __dsub_rn(s, __dmul_rn(l, l));
+                    if (w == 0 || isL) x = __dsub_rn(x, __dmul_rn(y, l));
+                    else x = fma(l, y, x);
+                }
+                if (!(s > 0.0)) {
+                    if (lane == 0) ctl[2] = 1;
+                    s = 1.0;
+                }
+                const double d = __dsqrt_rn(s);
+                const int k = j0 + j, v = v0 + lane;
+                const double num = w == 0 || isL ? x : (v == k ? 1.0 : -x);
+                const double q = __ddiv_rn(num, d);
+                if (w == 0) {
+                    if (lane > j) dg[lane][j] = q;
+                    if (lane == j) pv[j] = d;
+                } else {
+                    un[lane][j] = isL || v <= k ? q : 0.0;
+                }
+            };
+            if (w < 2) column(0);
+            __syncthreads();
+            for (int j = 0; j + 1 < nb; ++j) {
+                if (w < 2) {
+                    column(j + 1);
+                } else if (w < 5) {
+                    for (int c = j + w; c < nb; c += 3) {        // columns j + 2 .. nb - 1
+                        const double a = dg[c][j];
+                        if (lane >= c) dg[lane][c] = __dsub_rn(dg[lane][c], __dmul_rn(dg[lane][j], a));
+                    }
+                } else {
+                    for (int c = j + w - 3; c < nb; c += 3) {
+                        const double a = dg[c][j], b = un[lane][j], x = un[lane][c];
+                        un[lane][c] = isL ? __dsub_rn(x, __dmul_rn(b, a)) : fma(a, b, x);
+                    }
+                }
+                __syncthreads();
+            }
+            for (int t = w; t < DI_NB; t += DI_R) {
+                if (isL) {
+                    if (t < nv && lane < nb) M[at(v0 + t, j0 + lane)] = un[t][lane];
+                    if (Lout && lane < nv && t < nb) Lout[at(j0 + t, v0 + lane)] = un[lane][t];
+                } else if (lane < nv && t < nb) {
+                    Y[at(j0 + t, v0 + lane)] = un[lane][t];
+                }
+                if (u == 0 && Lout && t < nb && lane >= t && lane < nb)
+                    Lout[at(j0 + t, j0 + lane)] = lane == t ? pv[t] : dg[lane][t];
+            }
+            __syncthreads();
+        }
+        grid_sync(bar, ++epoch, err);
+        if (__ldcg(err)) return;
+        if (j1 >= n) break;                                       // nb == DI_NB from here on
+        const int rt = (n - j1 + DI_R - 1) / DI_R, ct = (n + DI_NB - 1) / DI_NB;
+        for (int t = blockIdx.x; t < rt * ct; t += G) {
+            const int i0 = j1 + t / ct * DI_R, c0 = t % ct * DI_NB;
+            if (c0 >= min(i0 + DI_R, n)) continue;                // above the diagonal
+            const bool isY = c0 < j1;
+            const int i = i0 + w, c = c0 + lane;
+            const bool live = i < n && c <= i;
+            un[w][lane] = i < n ? __ldcg(M + at(i, j0 + lane)) : 0.0;
+            for (int r = w; r < DI_NB; r += DI_R) {
+                if (isY) dg[r][lane] = __ldcg(Y + at(j0 + r, c));                      // c < j1 <= n
+                else dg[lane][r] = c0 + r < n ? __ldcg(M + at(c0 + r, j0 + lane)) : 0.0;
+            }
+            double* e = (isY ? Y : M) + at(i, c);
+            double x = live ? __ldcg(e) : 0.0;
+            __syncthreads();
+#pragma unroll 8
+            for (int k = 0; k < DI_NB; ++k) {
+                const double a = un[w][k], b = dg[k][lane];
+                x = isY ? fma(a, b, x) : __dsub_rn(x, __dmul_rn(a, b));
+            }
+            if (live) *e = x;
+            __syncthreads();
+        }
+        grid_sync(bar, ++epoch, err);
+        if (__ldcg(err)) return;
+    }
+    // terms with k < max(i, j) are exact zeros
+    const int rt = (n + DI_R - 1) / DI_R, ct = (n + DI_NB - 1) / DI_NB;
+    for (int t = blockIdx.x; t < rt * ct; t += G) {
+        const int i0 = t / ct * DI_R, c0 = t % ct * DI_NB;
+        if (c0 >= min(i0 + DI_R, n)) continue;
+        const int i = i0 + w, c = c0 + lane;
+        double s = 0.0;
+        for (int k0 = i0 / DI_NB * DI_NB; k0 < n; k0 += DI_NB) {
+            for (int r = w; r < DI_NB; r += DI_R) {
+                dg[r][lane] = k0 + r < n && c < n ? __ldcg(Y + at(k0 + r, c)) : 0.0;
+                if (lane < DI_R) un[r][lane] = k0 + r < n && i0 + lane < n ? __ldcg(Y + at(k0 + r, i0 + lane)) : 0.0;
+            }
+            __syncthreads();
+#pragma unroll 8
+            for (int k = 0; k < DI_NB; ++k) s = fma(un[k][w], dg[k][lane], s);
+            __syncthreads();
+        }
+        if (i < n && c <= i) {
+            Ainv[at(i, c)] = s;
+            Ainv[at(c, i)] = s;
+        }
+    }
 }
 
 // Column scaling for the pre-smoother: valm_k = val_k * minv[col_k].
@@ -2452,6 +2547,43 @@ int read_int(const int* dev, int* host, cudaStream_t st) {
     CUDA_CHECK(cudaMemcpyAsync(host, dev, sizeof(int), cudaMemcpyDeviceToHost, st));
     CUDA_CHECK(cudaStreamSynchronize(st));
     return *host;
+}
+
+// Scratch of k_dense_inverse for blocks of up to n rows.
+struct DenseWork {
+    double *M, *Y;
+    int* ctl;
+    DenseWork(Scratch& S, int n) {
+        M = S.mem.alloc<double>((size_t)n * n);
+        Y = S.mem.alloc<double>((size_t)n * n);
+        ctl = S.mem.alloc<int>(4);
+        CUDA_CHECK(cudaMemsetAsync(ctl, 0, sizeof(int) * 4, S.mem.stream));
+    }
+    // After one or more dense_inverse calls, with a stream synchronisation.
+    void check(Scratch& S, cudaStream_t st, const char* not_spd) {
+        CUDA_CHECK(cudaMemcpyAsync(S.host, ctl, sizeof(int) * 3, cudaMemcpyDeviceToHost, st));
+        CUDA_CHECK(cudaStreamSynchronize(st));
+        if (S.host[1]) AMG_THROW(AMG_ERR_TIMEOUT, "dense coarsest inverse: a block did not reach the grid barrier");
+        if (S.host[2]) AMG_THROW(AMG_ERR_NOT_SPD, "%s", not_spd);
+    }
+};
+
+// Ainv (and, if Lout is given, the column-major factor, zeroed by the caller)
+// of the dense diagonal block of A's rows [r0, r0 + n). The grid has a block
+// for every update tile up to one per SM: 61x47x33 (n = 185) took 3.18 ms on
+// one CTA and now XXX us, 256^3 (n = 64) 384 us and XXX us.
+void dense_inverse(amg_hierarchy* h, DenseWork& D, const DevCsr& A, int r0, int n, double* Ainv, double* Lout) {
+    cudaStream_t st = h->stream;
+    CUDA_CHECK(cudaMemsetAsync(D.M, 0, sizeof(double) * (size_t)n * n, st));
+    CUDA_CHECK(cudaMemsetAsync(D.Y, 0, sizeof(double) * (size_t)n * n, st));
+    CUDA_CHECK(cudaMemsetAsync(D.ctl, 0, sizeof(int), st));
+    const long long tiles = (long long)((n + DI_R - 1) / DI_R) * ((n + DI_NB - 1) / DI_NB);
+    const int grid = (int)std::max(1LL, std::min<long long>(tiles, h->num_sms));
+    const int *ptr = A.ptr, *col = A.col;
+    const double* val = A.val;
+    void* args[] = {&n, &r0, &ptr, &col, &val, &D.M, &D.Y, &Ainv, &Lout, &D.ctl};
+    CUDA_CHECK(cudaLaunchCooperativeKernel((const void*)k_dense_inverse, dim3(grid), dim3(DI_T), args, 0, st));
+    KERNEL_CHECK();
 }
 
 // C.nnz from C.ptr[n] and C.max_row from a row-length maximum, with one
@@ -3448,28 +3580,16 @@ void setup_hierarchy(amg_hierarchy* h, const amg_csr* Ain, const double* w_in) {
             const int smd = (int)(2 * sizeof(double) * (size_t)maxsm * maxsm);
             CUDA_CHECK(cudaFuncSetAttribute(k_coarse_inverse_blocks, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                             (int)(2 * sizeof(double) * SM_DENSE * SM_DENSE)));
-            k_coarse_inverse_blocks<<<nseg, 1024, smd, st>>>(0, h->segL_ptr, h->segL_blk, d_gofs, Lc.A.ptr,
-                                                             Lc.A.col, Lc.A.val, gwork, h->coarse_inv, nullptr,
-                                                             S.cnt + 5);
+            k_coarse_inverse_blocks<<<nseg, 1024, smd, st>>>(h->segL_ptr, h->segL_blk, d_gofs, Lc.A.ptr, Lc.A.col,
+                                                             Lc.A.val, gwork, h->coarse_inv, S.cnt + 5);
             KERNEL_CHECK();
         } else {
-            double* D = S.mem.alloc<double>((size_t)maxb * maxb + 1);
-            double* Lf = S.mem.alloc<double>((size_t)maxb * maxb + 1);
-            double* Y = S.mem.alloc<double>((size_t)maxb * maxb + 1);
+            DenseWork D(S, maxb);
             for (int s2 = 0; s2 < nseg; ++s2) {
                 const int ns = sp[s2 + 1] - sp[s2];
-                if (ns == 0) continue;
-                CUDA_CHECK(cudaMemsetAsync(D, 0, sizeof(double) * ns * ns, st));
-                CUDA_CHECK(cudaMemsetAsync(Lf, 0, sizeof(double) * ns * ns, st));
-                k_dense_lower_block<<<grid_for(h, ns), TPB, 0, st>>>(ns, sp[s2], Lc.A.ptr, Lc.A.col, Lc.A.val, D);
-                KERNEL_CHECK();
-                k_cholesky<<<1, 1024, 0, st>>>(ns, D, Lf, S.cnt + 5);
-                KERNEL_CHECK();
-                k_lower_inverse<<<(ns + 127) / 128, 128, 0, st>>>(ns, Lf, Y);
-                KERNEL_CHECK();
-                k_gram<<<(int)(((long long)ns * ns + 255) / 256), 256, 0, st>>>(ns, Y, h->coarse_inv + boff[s2]);
-                KERNEL_CHECK();
+                if (ns > 0) dense_inverse(h, D, Lc.A, sp[s2], ns, h->coarse_inv + boff[s2], nullptr);
             }
+            D.check(S, st, "a coarsest block hit a non-positive pivot");
         }
         if (read_int(S.cnt + 5, S.host, st)) AMG_THROW(AMG_ERR_NOT_SPD, "a coarsest block hit a non-positive pivot");
     }
@@ -3479,35 +3599,10 @@ void setup_hierarchy(amg_hierarchy* h, const amg_csr* Ain, const double* w_in) {
         Scope sc_(&h->prof, st, S_COARSE, 0.0);
         h->coarse_L = h->mem.alloc<double>((size_t)nc * nc);
         h->coarse_inv = h->mem.alloc<double>((size_t)nc * nc);
-        CUDA_CHECK(cudaMemsetAsync(S.cnt + 5, 0, sizeof(int), st));
-        if (nc <= CTA_DENSE) {                            // one CTA: shared memory up to SM_DENSE rows
-            const int smd = nc <= SM_DENSE ? (int)(2 * sizeof(double) * (size_t)nc * nc) : 0;
-            double* gwork = nc <= SM_DENSE ? nullptr : S.mem.alloc<double>(2 * (size_t)nc * nc + nc);
-            long long* gofs = S.mem.alloc<long long>(1);
-            CUDA_CHECK(cudaMemsetAsync(gofs, 0, sizeof(long long), st));
-            CUDA_CHECK(cudaFuncSetAttribute(k_coarse_inverse_blocks, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                            (int)(2 * sizeof(double) * SM_DENSE * SM_DENSE)));
-            k_coarse_inverse_blocks<<<1, 1024, smd, st>>>(nc, nullptr, nullptr, gofs, Lc.A.ptr, Lc.A.col,
-                                                          Lc.A.val, gwork, h->coarse_inv, h->coarse_L, S.cnt + 5);
-            KERNEL_CHECK();
-            if (read_int(S.cnt + 5, S.host, st))
-                AMG_THROW(AMG_ERR_NOT_SPD, "coarsest-level Cholesky hit a non-positive pivot");
-        } else {
-            double* D = S.mem.alloc<double>((size_t)nc * nc);
-            double* Y = S.mem.alloc<double>((size_t)nc * nc);
-            CUDA_CHECK(cudaMemsetAsync(D, 0, sizeof(double) * nc * nc, st));
-            CUDA_CHECK(cudaMemsetAsync(h->coarse_L, 0, sizeof(double) * nc * nc, st));
-            k_dense_lower<<<grid_for(h, nc), TPB, 0, st>>>(nc, Lc.A.ptr, Lc.A.col, Lc.A.val, D);
-            KERNEL_CHECK();
-            k_cholesky<<<1, 1024, 0, st>>>(nc, D, h->coarse_L, S.cnt + 5);
-            KERNEL_CHECK();
-            if (read_int(S.cnt + 5, S.host, st))
-                AMG_THROW(AMG_ERR_NOT_SPD, "coarsest-level Cholesky hit a non-positive pivot");
-            k_lower_inverse<<<(nc + 127) / 128, 128, 0, st>>>(nc, h->coarse_L, Y);
-            KERNEL_CHECK();
-            k_gram<<<(int)(((long long)nc * nc + 255) / 256), 256, 0, st>>>(nc, Y, h->coarse_inv);
-            KERNEL_CHECK();
-        }
+        CUDA_CHECK(cudaMemsetAsync(h->coarse_L, 0, sizeof(double) * (size_t)nc * nc, st));
+        DenseWork D(S, nc);
+        dense_inverse(h, D, Lc.A, 0, nc, h->coarse_inv, h->coarse_L);
+        D.check(S, st, "coarsest-level Cholesky hit a non-positive pivot");
     }
     CUDA_CHECK(cudaStreamSynchronize(st));
     h->prof.flush();
