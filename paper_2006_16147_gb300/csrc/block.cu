@@ -38,6 +38,7 @@ namespace {
 constexpr int TPB = 256;
 constexpr int WARPS = TPB / 32;
 constexpr int MAXK = 256;
+constexpr int CC_TPB = 512;   // threads of the iterative coarsest solve's blocks, one block per SM
 
 struct SellV {
     int n, nslices;
@@ -67,30 +68,31 @@ __device__ __forceinline__ Grp make_grp(int G) {
 // The CPL consecutive values at p (a lane's columns of one row; lim of them
 // are live columns). With VEC the row stride is a multiple of CPL, so the
 // address is aligned to CPL values and all CPL lie inside the row: the loads
-// are vectors. Without VEC only the live columns are read. CG reads through
-// L2 only (values other blocks write during the launch).
+// are vectors. Without VEC only the live columns are read. CG reads with plain
+// loads (values that other blocks write during the launch and a grid barrier
+// publishes; its fences order them).
 template <bool VEC, bool CG, int CPL, typename T>
 __device__ __forceinline__ void ld_cols(const T* p, T (&v)[CPL], int lim) {
     if constexpr (VEC && std::is_same<T, float>::value && CPL >= 4) {
 #pragma unroll
         for (int q = 0; q < CPL / 4; ++q) {
-            const float4 f = CG ? __ldcg(reinterpret_cast<const float4*>(p) + q)
+            const float4 f = CG ? reinterpret_cast<const float4*>(p)[q]
                                 : __ldg(reinterpret_cast<const float4*>(p) + q);
             v[4 * q] = f.x; v[4 * q + 1] = f.y; v[4 * q + 2] = f.z; v[4 * q + 3] = f.w;
         }
     } else if constexpr (VEC && std::is_same<T, float>::value && CPL == 2) {
-        const float2 f = CG ? __ldcg(reinterpret_cast<const float2*>(p)) : __ldg(reinterpret_cast<const float2*>(p));
+        const float2 f = CG ? *reinterpret_cast<const float2*>(p) : __ldg(reinterpret_cast<const float2*>(p));
         v[0] = f.x; v[1] = f.y;
     } else if constexpr (VEC && std::is_same<T, double>::value && CPL >= 2) {
 #pragma unroll
         for (int q = 0; q < CPL / 2; ++q) {
-            const double2 f = CG ? __ldcg(reinterpret_cast<const double2*>(p) + q)
+            const double2 f = CG ? reinterpret_cast<const double2*>(p)[q]
                                  : __ldg(reinterpret_cast<const double2*>(p) + q);
             v[2 * q] = f.x; v[2 * q + 1] = f.y;
         }
     } else {
 #pragma unroll
-        for (int m = 0; m < CPL; ++m) v[m] = m < lim ? (CG ? __ldcg(p + m) : __ldg(p + m)) : T(0);
+        for (int m = 0; m < CPL; ++m) v[m] = m < lim ? (CG ? p[m] : __ldg(p + m)) : T(0);
     }
 }
 
@@ -501,214 +503,257 @@ __device__ __forceinline__ void bk_grid_sync(unsigned* count, unsigned epoch, in
     __syncthreads();
 }
 
-// Block partial of one value per column into out[blockIdx.x * k + c].
-template <int CPL>
-__device__ __forceinline__ void bk_colpart(double (&v)[CPL], const Grp& g, int k, double* out) {
-    __shared__ double sm[WARPS][MAXK];
-#pragma unroll
-    for (int m = 0; m < CPL; ++m)
-        for (int o = g.G; o < 32; o <<= 1) v[m] += __shfl_xor_sync(FULL_MASK, v[m], o);
+// Sums over the grid of v[0 .. NV) per column: this block's partials go to
+// part[(blockIdx.x * NV + j) * k + c], and after the grid barrier every block
+// adds them in the same order into dst[j * k + c]. As few FP64 additions as
+// there are partials: lanes of a warp add different columns, through shared
+// memory (butterflies in every warp, 152 serial loads per column and a
+// division per thread made a reduction of 16 columns cost 14 us, four of them
+// an iteration).
+template <int CPL, int NV>
+__device__ __forceinline__ void cc_partials(double (&v)[NV][CPL], const Grp& g, int k, double* part, double* sm) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (lane < g.G) {
+    const int gpw = 32 / g.G, W = g.G * CPL;             // groups of a warp, columns of a group (>= k)
+    constexpr int SLOTS = 32 * CPL;                      // gpw * W: values of a warp
 #pragma unroll
-        for (int m = 0; m < CPL; ++m) {
-            const int c = lane * CPL + m;
-            if (c < k) sm[warp][c] = v[m];
+    for (int j = 0; j < NV; ++j) {
+        __syncthreads();
+        double* own = sm + warp * SLOTS + (lane / g.G) * W + g.gl * CPL;
+#pragma unroll
+        for (int m = 0; m < CPL; ++m) own[m] = v[j][m];
+        __syncthreads();
+        for (int s = threadIdx.x; s < SLOTS; s += CC_TPB) {
+            double a0 = sm[s], a1 = sm[SLOTS + s];
+#pragma unroll
+            for (int w = 2; w < CC_TPB / 32; w += 2) {
+                a0 += sm[w * SLOTS + s];
+                a1 += sm[(w + 1) * SLOTS + s];
+            }
+            sm[s] = a0 + a1;
+        }
+        __syncthreads();
+        for (int c = threadIdx.x; c < k; c += CC_TPB) {
+            double a = sm[c];
+            for (int t = 1; t < gpw; ++t) a += sm[t * W + c];
+            part[((size_t)blockIdx.x * NV + j) * k + c] = a;
         }
     }
-    __syncthreads();
-    for (int c = threadIdx.x; c < k; c += blockDim.x) {
-        double a = 0.0;
-        for (int w = 0; w < WARPS; ++w) a += sm[w][c];
-        out[(size_t)blockIdx.x * k + c] = a;
+}
+template <int NV>
+__device__ __forceinline__ void cc_sums(const double* part, int k, int ld, double* dst, double* sm) {
+    const int nv = NV * k;                               // values; R threads share one (R from the block width ld:
+    int R = 1;                                           // the order does not depend on the columns in flight)
+    while (R < 32 && 2 * R * NV * ld <= CC_TPB) R *= 2;
+    for (int v0 = 0; v0 < nv; v0 += CC_TPB / R) {
+        const int cnt = min(nv - v0, CC_TPB / R);
+        __syncthreads();
+        for (int t = threadIdx.x; t < cnt * R; t += CC_TPB) {
+            const int v = v0 + t % cnt;
+            double a = 0.0;
+#pragma unroll 5
+            for (int b = t / cnt; b < (int)gridDim.x; b += R) a += __ldcg(part + (size_t)b * nv + v);
+            sm[t] = a;
+        }
+        __syncthreads();
+        for (int half = R >> 1; half > 0; half >>= 1) {  // a tree over the R partial sums of every value
+            for (int t = threadIdx.x; t < cnt * half; t += CC_TPB) sm[t] += sm[t + cnt * half];
+            __syncthreads();
+        }
+        for (int t = threadIdx.x; t < cnt; t += CC_TPB) dst[v0 + t] = sm[t];
     }
     __syncthreads();
 }
 
-// dst[c] = sum over blocks of part[blk * k + c], same order in every block.
-__device__ __forceinline__ void bk_colsum(const double* part, int k, double* dst) {
-    for (int c = threadIdx.x; c < k; c += blockDim.x) {
-        double a = 0.0;
-        for (int b = 0; b < (int)gridDim.x; ++b) a += __ldcg(part + (size_t)b * k + c);
-        dst[c] = a;
-    }
-    __syncthreads();
-}
-
-template <typename TI, typename TO, int CPL>
-__global__ void __launch_bounds__(TPB) bk_coarse_cg(SellV S, const double* __restrict__ sval, int n, int nlong,
-                                                    const int* __restrict__ long_rows, const int* __restrict__ cptr,
-                                                    const int* __restrict__ ccol, const double* __restrict__ cval,
-                                                    const double* __restrict__ minv, const TI* __restrict__ B,
-                                                    TO* __restrict__ Xo, int k, int ld, int G, double* x, double* r,
-                                                    double* z, double* p, double* q, double* part, unsigned* bar,
-                                                    int* err, int maxit, double rtol) {
-    __shared__ double s_rho[MAXK], s_bb[MAXK], s_t[MAXK];
+// One iteration is two grid barriers: the product q = A z + beta q (= A p)
+// with p = z + beta p, then x, r and z = M^-1 r with r.r and r.z. 64^3 jump
+// coefficients, 16 columns, 30 iterations: 1.69 ms before (four barriers, a
+// block of 256 threads per SM), 0.74 ms now.
+template <typename TI, typename TO, int CPL, bool VEC>
+__global__ void __launch_bounds__(CC_TPB) bk_coarse_cg(SellV S, const double* __restrict__ sval, int n, int nlong,
+                                                       const int* __restrict__ long_rows, const int* __restrict__ cptr,
+                                                       const int* __restrict__ ccol, const double* __restrict__ cval,
+                                                       const double* __restrict__ minv, const TI* __restrict__ B,
+                                                       TO* __restrict__ Xo, int k, int ld, int G, double* x, double* r,
+                                                       double* z, double* p, double* q, double* part, unsigned* bar,
+                                                       int* err, int maxit, double rtol) {
+    __shared__ double s_rho[MAXK], s_stop[MAXK], s_t[2 * MAXK], s_al[MAXK];   // s_al: alpha, then beta
     __shared__ int s_live[MAXK];
-    __shared__ int s_any;
+    extern __shared__ double cc_sm[];                    // CC_TPB * CPL
     const Grp g = make_grp(G);
+    const int c0 = g.gl * CPL;
     const int lane = threadIdx.x & 31;
     const int gwarp = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     const int nwarps = (int)((gridDim.x * blockDim.x) >> 5);
-    const size_t PK = (size_t)gridDim.x * k;
     unsigned epoch = 0;
-    int red = 0;
-    auto slot = [&]() { return part + (size_t)(red & 1) * PK; };
-    double d0[CPL];
-    // x = 0, r = b, z = M^-1 r, p = z; rho = r.z and bb = b.b per column
+    int red = 0;                                         // reduction counter: two buffers of two values
+    auto slot = [&]() { return part + (size_t)(red & 1) * 2 * gridDim.x * k; };
+    double d2[2][CPL];
 #pragma unroll
-    for (int m = 0; m < CPL; ++m) d0[m] = 0.0;
-    double d1[CPL];
+    for (int m = 0; m < CPL; ++m) d2[0][m] = d2[1][m] = 0.0;
+    // x = 0, r = b, z = M^-1 r; b.b and rho = r.z per column
+    if (c0 < k)
+        for (int i = g.gw; i < n; i += g.ngroups) {
+            const double mi = minv[i];
+            const size_t o = (size_t)i * ld + c0;
+            TI bt[CPL];
+            double bi[CPL], zi[CPL], zero[CPL];
+            ld_cols<VEC, false, CPL>(B + o, bt, k - c0);
 #pragma unroll
-    for (int m = 0; m < CPL; ++m) d1[m] = 0.0;
-    for (int i = g.gw; i < n; i += g.ngroups) {
-        const double mi = minv[i];
-#pragma unroll
-        for (int m = 0; m < CPL; ++m) {
-            const int c = g.gl * CPL + m;
-            if (c >= k) continue;
-            const size_t o = (size_t)i * ld + c;
-            const double bi = (double)B[o];
-            x[o] = 0.0;
-            r[o] = bi;
-            const double zi = mi * bi;
-            z[o] = zi;
-            p[o] = zi;
-            d0[m] = fma(bi, zi, d0[m]);
-            d1[m] = fma(bi, bi, d1[m]);
+            for (int m = 0; m < CPL; ++m) {
+                bi[m] = (double)bt[m];
+                zi[m] = mi * bi[m];
+                zero[m] = 0.0;
+                if (c0 + m >= k) continue;
+                d2[0][m] = fma(bi[m], bi[m], d2[0][m]);
+                d2[1][m] = fma(bi[m], zi[m], d2[1][m]);
+            }
+            st_cols<VEC, CPL>(x + o, zero, c0, k);
+            st_cols<VEC, CPL>(r + o, bi, c0, k);
+            st_cols<VEC, CPL>(z + o, zi, c0, k);
         }
-    }
-    bk_colpart<CPL>(d0, g, k, slot());
-    bk_colpart<CPL>(d1, g, k, slot() + PK * 2);
+    cc_partials<CPL, 2>(d2, g, k, slot(), cc_sm);
     bk_grid_sync(bar, ++epoch, err);
     if (__ldcg(err)) return;
-    bk_colsum(slot(), k, s_rho);
-    bk_colsum(slot() + PK * 2, k, s_bb);
-    for (int c = threadIdx.x; c < k; c += blockDim.x) s_live[c] = s_bb[c] > 0.0;
-    __syncthreads();
+    cc_sums<2>(slot(), k, ld, s_t, cc_sm);
     ++red;
+    for (int c = threadIdx.x; c < k; c += blockDim.x) {
+        const double bb = s_t[c];
+        s_live[c] = bb > 0.0;
+        s_stop[c] = rtol * rtol * bb;
+        s_rho[c] = s_t[k + c];
+        s_al[c] = 0.0;
+    }
+    __syncthreads();
     for (int it = 0; it < maxit; ++it) {
-        if (threadIdx.x == 0) {
-            int a = 0;
-            for (int c = 0; c < k; ++c) a |= s_live[c];
-            s_any = a;
-        }
-        __syncthreads();
-        if (!s_any) break;
-        // q = A p, p . q
+        int alive = 0;
+        for (int c = threadIdx.x; c < k; c += blockDim.x) alive |= s_live[c];
+        if (!__syncthreads_or(alive)) break;
+        double be[CPL], d1[1][CPL];
+        bool on[CPL], any = false;
 #pragma unroll
-        for (int m = 0; m < CPL; ++m) d0[m] = 0.0;
-        for (int ip = g.gw; ip < S.n; ip += g.ngroups) {
+        for (int m = 0; m < CPL; ++m) {
+            on[m] = c0 + m < k && s_live[c0 + m];
+            be[m] = on[m] ? s_al[c0 + m] : 0.0;
+            any |= on[m];
+            d1[0][m] = 0.0;
+        }
+        // p = z + beta p, q = A z + beta q of one row (it = 0: p and q are not
+        // read), p . q; the row's own p, q and z are loaded before its product
+        double pv[CPL], qv[CPL], zv[CPL];
+        auto own_row = [&](int i) {
+            const size_t o = (size_t)i * ld + c0;
+            ld_cols<VEC, true, CPL>(z + o, zv, k - c0);
+            if (it > 0) {
+                ld_cols<VEC, true, CPL>(p + o, pv, k - c0);
+                ld_cols<VEC, true, CPL>(q + o, qv, k - c0);
+            }
+        };
+        auto finish_row = [&](int i, const double (&acc)[CPL]) {
+            const size_t o = (size_t)i * ld + c0;
+#pragma unroll
+            for (int m = 0; m < CPL; ++m) {
+                pv[m] = it > 0 ? fma(be[m], pv[m], zv[m]) : zv[m];
+                qv[m] = it > 0 ? fma(be[m], qv[m], acc[m]) : acc[m];
+                if (on[m]) d1[0][m] = fma(pv[m], qv[m], d1[0][m]);
+            }
+            st_cols<VEC, CPL>(p + o, pv, c0, k);
+            st_cols<VEC, CPL>(q + o, qv, c0, k);
+        };
+        if (any)
+            for (int ip = g.gw; ip < S.n; ip += g.ngroups) {
+                double acc[CPL];
+#pragma unroll
+                for (int m = 0; m < CPL; ++m) acc[m] = 0.0;
+                const int i = rowid(S, ip);
+                own_row(i);
+                sell_row_k<VEC, true, CPL>(S, sval, ip, c0, k, (const double*)z, ld, acc);
+                finish_row(i, acc);
+            }
+        // long rows: a warp per row, its lane groups take the entries in turn
+        for (int lr = gwarp; lr < nlong; lr += nwarps) {
+            const int i = __ldg(long_rows + lr);
+            const int e1 = __ldg(cptr + i + 1);
             double acc[CPL];
 #pragma unroll
             for (int m = 0; m < CPL; ++m) acc[m] = 0.0;
-            sell_row_k<false, true, CPL>(S, sval, ip, g.gl * CPL, k, (const double*)p, ld, acc);
-            const int i = rowid(S, ip);
+            if (any)
+#pragma unroll 4
+                for (int e = __ldg(cptr + i) + lane / G; e < e1; e += 32 / G) {
+                    const double a = __ldg(cval + e);
+                    double ze[CPL];
+                    ld_cols<VEC, true, CPL>((const double*)z + (size_t)__ldg(ccol + e) * ld + c0, ze, k - c0);
 #pragma unroll
-            for (int m = 0; m < CPL; ++m) {
-                const int c = g.gl * CPL + m;
-                if (c >= k) continue;
-                const size_t o = (size_t)i * ld + c;
-                q[o] = acc[m];
-                d0[m] = fma(__ldcg(p + o), acc[m], d0[m]);
+                    for (int m = 0; m < CPL; ++m) acc[m] = fma(a, ze[m], acc[m]);
+                }
+            for (int o = 16; o >= G; o >>= 1)
+#pragma unroll
+                for (int m = 0; m < CPL; ++m) acc[m] += __shfl_xor_sync(FULL_MASK, acc[m], o);
+            if (any && lane < G) {
+                own_row(i);
+                finish_row(i, acc);
             }
         }
-        for (int lr = gwarp; lr < nlong; lr += nwarps) {
-            const int i = __ldg(long_rows + lr);
-            const int e0 = __ldg(cptr + i), e1 = __ldg(cptr + i + 1);
-            for (int c = 0; c < k; ++c) {
-                double a = 0.0;
-                for (int e = e0 + lane; e < e1; e += 32) a = fma(__ldg(cval + e), __ldcg(p + (size_t)__ldg(ccol + e) * ld + c), a);
-                a = warp_sum(a);
-                const size_t o = (size_t)i * ld + c;
-                if (lane == 0) q[o] = a;
-                // the first group of the warp carries the long rows' share of p . q
-#pragma unroll
-                for (int m = 0; m < CPL; ++m)
-                    if (lane < G && lane * CPL + m == c) d0[m] = fma(__ldcg(p + o), a, d0[m]);
-            }
-        }
-        bk_colpart<CPL>(d0, g, k, slot());
+        cc_partials<CPL, 1>(d1, g, k, slot(), cc_sm);
         bk_grid_sync(bar, ++epoch, err);
         if (__ldcg(err)) return;
-        bk_colsum(slot(), k, s_t);
+        cc_sums<1>(slot(), k, ld, s_t, cc_sm);
         ++red;
-        // alpha per live column; x += alpha p, r -= alpha q; r.r
+        for (int c = threadIdx.x; c < k; c += blockDim.x) s_al[c] = s_live[c] ? s_rho[c] / s_t[c] : 0.0;
+        __syncthreads();
+        // x += alpha p, r -= alpha q, z = M^-1 r; r.r and r.z (columns that
+        // are not live keep their values: alpha = 0)
         double al[CPL];
 #pragma unroll
         for (int m = 0; m < CPL; ++m) {
-            const int c = g.gl * CPL + m;
-            al[m] = (c < k && s_live[c]) ? s_rho[c] / s_t[c] : 0.0;
-            d0[m] = 0.0;
+            al[m] = on[m] ? s_al[c0 + m] : 0.0;
+            d2[0][m] = d2[1][m] = 0.0;
         }
-        for (int i = g.gw; i < n; i += g.ngroups) {
+        if (any)
+            for (int i = g.gw; i < n; i += g.ngroups) {
+                const double mi = minv[i];
+                const size_t o = (size_t)i * ld + c0;
+                double pv[CPL], qv[CPL], xv[CPL], rv[CPL], zv[CPL];
+                ld_cols<VEC, true, CPL>(p + o, pv, k - c0);
+                ld_cols<VEC, true, CPL>(q + o, qv, k - c0);
+                ld_own<VEC, CPL>(x + o, xv, k - c0);
+                ld_own<VEC, CPL>(r + o, rv, k - c0);
 #pragma unroll
-            for (int m = 0; m < CPL; ++m) {
-                const int c = g.gl * CPL + m;
-                if (c >= k || al[m] == 0.0) continue;
-                const size_t o = (size_t)i * ld + c;
-                x[o] = fma(al[m], __ldcg(p + o), x[o]);
-                const double ri = fma(-al[m], __ldcg(q + o), r[o]);
-                r[o] = ri;
-                d0[m] = fma(ri, ri, d0[m]);
+                for (int m = 0; m < CPL; ++m) {
+                    if (al[m] != 0.0) {
+                        xv[m] = fma(al[m], pv[m], xv[m]);
+                        rv[m] = fma(-al[m], qv[m], rv[m]);
+                    }
+                    zv[m] = mi * rv[m];
+                    d2[0][m] = fma(rv[m], rv[m], d2[0][m]);
+                    d2[1][m] = fma(rv[m], zv[m], d2[1][m]);
+                }
+                st_cols<VEC, CPL>(x + o, xv, c0, k);
+                st_cols<VEC, CPL>(r + o, rv, c0, k);
+                st_cols<VEC, CPL>(z + o, zv, c0, k);
             }
-        }
-        bk_colpart<CPL>(d0, g, k, slot());
+        cc_partials<CPL, 2>(d2, g, k, slot(), cc_sm);
         bk_grid_sync(bar, ++epoch, err);
         if (__ldcg(err)) return;
-        bk_colsum(slot(), k, s_t);
+        cc_sums<2>(slot(), k, ld, s_t, cc_sm);
         ++red;
-        for (int c = threadIdx.x; c < k; c += blockDim.x)
-            if (s_live[c] && s_t[c] <= rtol * rtol * s_bb[c]) s_live[c] = 0;
-        __syncthreads();
-        // z = M^-1 r; r.z; beta; p = z + beta p
-#pragma unroll
-        for (int m = 0; m < CPL; ++m) d0[m] = 0.0;
-        for (int i = g.gw; i < n; i += g.ngroups) {
-            const double mi = minv[i];
-#pragma unroll
-            for (int m = 0; m < CPL; ++m) {
-                const int c = g.gl * CPL + m;
-                if (c >= k || !s_live[c]) continue;
-                const size_t o = (size_t)i * ld + c;
-                const double zi = mi * r[o];
-                z[o] = zi;
-                d0[m] = fma(r[o], zi, d0[m]);
-            }
-        }
-        bk_colpart<CPL>(d0, g, k, slot());
-        bk_grid_sync(bar, ++epoch, err);
-        if (__ldcg(err)) return;
-        bk_colsum(slot(), k, s_t);
-        ++red;
-        double be[CPL];
-#pragma unroll
-        for (int m = 0; m < CPL; ++m) {
-            const int c = g.gl * CPL + m;
-            be[m] = (c < k && s_live[c]) ? s_t[c] / s_rho[c] : 0.0;
+        for (int c = threadIdx.x; c < k; c += blockDim.x) {
+            if (!s_live[c]) continue;
+            if (s_t[c] <= s_stop[c]) s_live[c] = 0;
+            s_al[c] = s_t[k + c] / s_rho[c];
+            s_rho[c] = s_t[k + c];
         }
         __syncthreads();
-        for (int c = threadIdx.x; c < k; c += blockDim.x)
-            if (s_live[c]) s_rho[c] = s_t[c];
+    }
+    if (c0 < k)
         for (int i = g.gw; i < n; i += g.ngroups) {
+            const size_t o = (size_t)i * ld + c0;
+            double xv[CPL];
+            TO xo[CPL];
+            ld_own<VEC, CPL>(x + o, xv, k - c0);
 #pragma unroll
-            for (int m = 0; m < CPL; ++m) {
-                const int c = g.gl * CPL + m;
-                if (c >= k || !s_live[c]) continue;
-                const size_t o = (size_t)i * ld + c;
-                p[o] = fma(be[m], p[o], z[o]);
-            }
+            for (int m = 0; m < CPL; ++m) xo[m] = (TO)xv[m];
+            st_cols<VEC, CPL>(Xo + o, xo, c0, k);
         }
-        bk_grid_sync(bar, ++epoch, err);
-        if (__ldcg(err)) return;
-    }
-    for (int i = g.gw; i < n; i += g.ngroups) {
-#pragma unroll
-        for (int m = 0; m < CPL; ++m) {
-            const int c = g.gl * CPL + m;
-            if (c < k) Xo[(size_t)i * ld + c] = (TO)x[(size_t)i * ld + c];
-        }
-    }
 }
 
 // ------------------------------------------------------------- CG ----------
@@ -1042,8 +1087,9 @@ void block_vcycle(amg_hierarchy* h, BlockWork& W, int k, int flexible) {
                             (void*)&cval, (void*)&cminv, (void*)&bin, (void*)&xout, &kk, &ldd, &GG, &W.cw[0],
                             &W.cw[1], &W.cw[2], &W.cw[3], &W.cw[4], &W.cpart, &bar, &err, &maxit, &rtol};
             const void* fn = nullptr;
-            DISPATCH_CPL(cpl, ld, fn = (const void*)bk_coarse_cg<T, T, CPL>);
-            CUDA_CHECK(cudaLaunchCooperativeKernel(fn, dim3(h->num_sms), dim3(TPB), args, 0, st));
+            DISPATCH_CPL(cpl, ld, fn = (const void*)bk_coarse_cg<T, T, CPL, VEC>);
+            CUDA_CHECK(cudaLaunchCooperativeKernel(fn, dim3(h->num_sms), dim3(CC_TPB), args,
+                                                   sizeof(double) * CC_TPB * cpl, st));
             KERNEL_CHECK();
         }
     }
@@ -1184,7 +1230,8 @@ BlockWork& block_ensure(amg_hierarchy* h, int K, bool fixed_width) {
         W->cpart = W->mem.alloc<double>((size_t)h->num_sms * K * 4);
         W->cctl = W->mem.alloc<int>(4);
         int per_sm = 0;
-        CUDA_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, bk_coarse_cg<double, double, 8>, TPB, 0));
+        CUDA_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, bk_coarse_cg<double, double, 8, true>, CC_TPB,
+                                                                 sizeof(double) * CC_TPB * 8));
         if (per_sm < 1) AMG_THROW(AMG_ERR_CUDA, "multi-column coarsest CG kernel cannot be resident");
     }
     if (h->opt.autotune && !fixed_width) block_autotune(h, *W);

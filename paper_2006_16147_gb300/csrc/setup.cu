@@ -2570,8 +2570,9 @@ struct DenseWork {
 
 // Ainv (and, if Lout is given, the column-major factor, zeroed by the caller)
 // of the dense diagonal block of A's rows [r0, r0 + n). The grid has a block
-// for every update tile up to one per SM: 61x47x33 (n = 185) took 3.18 ms on
-// one CTA and now XXX us, 256^3 (n = 64) 384 us and XXX us.
+// for every update tile up to one per SM: 61x47x33 (n = 192) took 3.18 ms on
+// one CTA and now 0.47 ms (a step 7.04 -> 4.27 ms); the blocks of 64 rows of
+// 128^3 to 256^3 are a 0.4 ms chain in one CTA, two panels here.
 void dense_inverse(amg_hierarchy* h, DenseWork& D, const DevCsr& A, int r0, int n, double* Ainv, double* Lout) {
     cudaStream_t st = h->stream;
     CUDA_CHECK(cudaMemsetAsync(D.M, 0, sizeof(double) * (size_t)n * n, st));
@@ -2907,14 +2908,23 @@ void build_sell(amg_hierarchy* h, DevCsr A, DevSell& E, Scratch& S, bool fp32, c
 // Hybrid layout for the iterative coarsest solve: rows with at most lmax
 // entries in SELL-C-sigma (positions map to rows through perm), longer rows
 // listed in long_rows and read straight from the CSR by one warp each, so a
-// few long rows cannot hold up a whole slice.
-void build_sell_hybrid(amg_hierarchy* h, const DevCsr& A, DevSell& E, Scratch& S, int lmax) {
+// few long rows cannot hold up a whole slice. A stalled coarsest level has rows
+// of a few entries and hubs of a hundred and next to nothing between (374K rows
+// of 256^3 jump coefficients: 2% above 8, 1.9% above 32); with lmax = 8 a slice
+// is one batch of loads, not up to four in series. Where more than 1/16 of the
+// rows are longer, lmax = 32: a warp per row spends six FP64 instructions on
+// it, a slice at most lmax on 32 rows.
+void build_sell_hybrid(amg_hierarchy* h, const DevCsr& A, DevSell& E, Scratch& S) {
     cudaStream_t st = h->stream;
     const int n = A.n;
-    k_long_flags<<<grid_for(h, n), TPB, 0, st>>>(n, A.ptr, lmax, S.flag);
-    KERNEL_CHECK();
-    scan_exclusive(S.flag, S.qid, n, S.cnt + 6, st, S.scan_tmp);
-    const int nlong = read_int(S.cnt + 6, S.host, st);
+    int nlong = 0;
+    for (int lmax : {8, 32}) {
+        k_long_flags<<<grid_for(h, n), TPB, 0, st>>>(n, A.ptr, lmax, S.flag);
+        KERNEL_CHECK();
+        scan_exclusive(S.flag, S.qid, n, S.cnt + 6, st, S.scan_tmp);
+        nlong = read_int(S.cnt + 6, S.host, st);
+        if (nlong <= n / 16) break;
+    }
     const int nshort = n - nlong;
     E.nlong = nlong;
     E.long_rows = h->mem.alloc<int>(nlong > 0 ? nlong : 1);
@@ -3517,7 +3527,7 @@ void setup_hierarchy(amg_hierarchy* h, const amg_csr* Ain, const double* w_in) {
         }
         Scope sc_(&h->prof, st, S_FORMAT, 24.0 * L.A.nnz);
         const bool coarsest_cg = l == nlev - 1 && L.A.n > o.max_dense;
-        if (coarsest_cg && l > 0) build_sell_hybrid(h, L.A, L.S, S, 32);
+        if (coarsest_cg && l > 0) build_sell_hybrid(h, L.A, L.S, S);
         else if (l == 0 || l < nlev - 1 || coarsest_cg) build_sell(h, L.A, L.S, S, fp32);
         if (l == nlev - 1) break;
         build_scaled(h, L, fp32);

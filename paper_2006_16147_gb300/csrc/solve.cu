@@ -537,7 +537,10 @@ __global__ void k_coarse_solve(int n, const double* __restrict__ Ainv, const T* 
 // maxit iterations, all in FP64 and in one cooperative launch. Scalars are
 // block partials written to a double buffer; after each grid barrier every
 // block sums the partials in the same order, so all blocks hold identical
-// scalars without a broadcast step. Waits are bounded (2 s).
+// scalars without a broadcast step. Waits are bounded (2 s). What a barrier
+// publishes is read with plain loads: the barrier's fences order them, and the
+// gathers of z find neighbouring rows in L1 (never with ld.nc, whose lines a
+// fence does not drop).
 __device__ __forceinline__ unsigned long long cg_global_ns() {
     unsigned long long t;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
@@ -575,7 +578,9 @@ __device__ __forceinline__ void cg_partials(const double (&v)[NV], double* part,
 // thread (an FP64 division in all 1024 threads would hold the SM's FP64 pipe
 // for microseconds) and the block gets them through shared memory. With that
 // and 1024 threads per SM instead of 512, one coarsest solve of 374K rows (30
-// iterations) takes 1.12 ms, 1.61 ms before.
+// iterations) takes 1.10 ms, 1.61 ms before; with two barriers an iteration
+// (the direction update inside the product), a row's loads together and hubs
+// kept out of the slices 1.01 ms. A third of that is the FP64 pipe.
 template <int NV, int NO, typename FIN>
 __device__ __forceinline__ void cg_sums(const double* part, int G, double (&out)[NO], FIN&& fin) {
     __shared__ double tot[NO];
@@ -598,7 +603,7 @@ __device__ __forceinline__ void cg_sums(const double* part, int G, double (&out)
 }
 
 template <typename TI, typename TO>
-__global__ void __launch_bounds__(CG_TPB) k_coarse_cg(SellView S, const double* __restrict__ val, int n,
+__global__ void __launch_bounds__(CG_TPB, 1) k_coarse_cg(SellView S, const double* __restrict__ val, int n,
                                                    int nlong, const int* __restrict__ long_rows,
                                                    const int* __restrict__ cptr, const int* __restrict__ ccol,
                                                    const double* __restrict__ cval,
@@ -618,7 +623,6 @@ __global__ void __launch_bounds__(CG_TPB) k_coarse_cg(SellView S, const double* 
         r[i] = bi;
         const double zi = minv[i] * bi;
         z[i] = zi;
-        p[i] = zi;
         a = fma(bi, zi, a);
         c = fma(bi, bi, c);
     }
@@ -630,36 +634,84 @@ __global__ void __launch_bounds__(CG_TPB) k_coarse_cg(SellView S, const double* 
     if (__ldcg(err)) return;
     double tot[2];
     cg_sums<2>(slot(), G, tot, [](const double (&s)[2], double* o) { o[0] = s[0]; o[1] = s[1]; });
-    double rho = tot[0];
+    double rho = tot[0], beta = 0.0;
     const double bb = tot[1];
     ++red;
     if (bb > 0.0) {
         const double stop2 = rtol * rtol * bb;
         for (int it = 0; it < maxit; ++it) {
-            // q = A p, p . q
+            // q = A z + beta q (= A p), p = z + beta p, p . q; a row's own
+            // z, p and q are loaded before its product, beside the gathers
             double pq = 0.0;
-            const int lane = threadIdx.x & 31, nw = G * (blockDim.x >> 5);
-            for (int sl = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); sl < S.nslices; sl += nw) {
-                const double acc = sell_row(S.col, val, (long long)S.sptr[sl] * 32 + lane, S.sptr[sl + 1] - S.sptr[sl],
-                                            [&](int j) { return __ldcg(p + j); });
-                const int ip = sl * 32 + lane;
-                if (ip < S.n) {
-                    const int i = sell_rowid(S, ip);
-                    q[i] = acc;
-                    pq = fma(__ldcg(p + i), acc, pq);
+            struct Own { double z, p, q; };
+            auto own = [&](int i) {
+                Own o{z[i], 0.0, 0.0};
+                if (it > 0) {
+                    o.p = p[i];
+                    o.q = q[i];
                 }
-            }
+                return o;
+            };
+            auto finish_row = [&](int i, const Own& o, double acc) {
+                double pi = o.z;
+                if (it > 0) {
+                    pi = fma(beta, o.p, pi);
+                    acc = fma(beta, o.q, acc);
+                }
+                p[i] = pi;
+                q[i] = acc;
+                pq = fma(pi, acc, pq);
+            };
+            const int lane = threadIdx.x & 31, nw = G * (blockDim.x >> 5);
             // long rows: one warp per row, straight from the CSR
             for (int lr = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); lr < nlong; lr += nw) {
                 const int i = __ldg(long_rows + lr);
+                const Own o = own(i);
+                const int e = __ldg(cptr + i + 1);
                 double acc = 0.0;
-                for (int k = __ldg(cptr + i) + lane; k < __ldg(cptr + i + 1); k += 32)
-                    acc = fma(__ldg(cval + k), __ldcg(p + __ldg(ccol + k)), acc);
-                acc = warp_sum(acc);
-                if (lane == 0) {
-                    q[i] = acc;
-                    pq = fma(__ldcg(p + i), acc, pq);
+                for (int k = __ldg(cptr + i) + lane; k < e; k += 128) {
+                    int j[4];
+                    double v[4], zv[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const bool ok = k + 32 * u < e;
+                        j[u] = ok ? __ldg(ccol + k + 32 * u) : -1;
+                        v[u] = ok ? __ldg(cval + k + 32 * u) : 0.0;
+                    }
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) zv[u] = j[u] >= 0 ? z[j[u]] : 0.0;
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+                        if (j[u] >= 0) acc = fma(v[u], zv[u], acc);
                 }
+                acc = warp_sum(acc);
+                if (lane == 0) finish_row(i, o, acc);
+            }
+            for (int sl = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); sl < S.nslices; sl += nw) {
+                const int ip = sl * 32 + lane;
+                const int i = ip < S.n ? sell_rowid(S, ip) : -1;
+                const int s0 = __ldg(S.sptr + sl), w = __ldg(S.sptr + sl + 1) - s0;
+                const long long base = (long long)s0 * 32 + lane;
+                Own o{};
+                if (i >= 0) o = own(i);
+                double acc = 0.0;
+                for (int k = 0; k < w; k += 4) {           // mean width 3 in the hybrid layout
+                    int j[4];
+                    double v[4], zv[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+                        if (k + u < w) {
+                            j[u] = __ldg(S.col + base + 32 * (k + u));
+                            v[u] = __ldg(val + base + 32 * (k + u));
+                        }
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+                        if (k + u < w) zv[u] = z[j[u]];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+                        if (k + u < w) acc = fma(v[u], zv[u], acc);
+                }
+                if (i >= 0) finish_row(i, o, acc);
             }
             const double v1[1] = {pq};
             cg_partials<1>(v1, slot(), G);
@@ -672,14 +724,32 @@ __global__ void __launch_bounds__(CG_TPB) k_coarse_cg(SellView S, const double* 
             // x += alpha p, r -= alpha q, z = M^-1 r: r . r and r . z in one
             // reduction (z is formed even on the last step, where it is unused)
             double rr = 0.0, rz = 0.0;
-            for (int i = tid; i < n; i += stride) {
-                x[i] = fma(alpha, __ldcg(p + i), x[i]);
-                const double ri = fma(-alpha, __ldcg(q + i), r[i]);
-                r[i] = ri;
-                rr = fma(ri, ri, rr);
-                const double zi = minv[i] * ri;
-                z[i] = zi;
-                rz = fma(ri, zi, rz);
+            for (int i0 = tid; i0 < n; i0 += 2 * stride) {
+                double xv[2], rv[2], pv[2], qv[2], mv[2];
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    const int i = i0 + u * stride;
+                    if (i < n) {
+                        pv[u] = p[i];
+                        qv[u] = q[i];
+                        xv[u] = x[i];
+                        rv[u] = r[i];
+                        mv[u] = minv[i];
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    const int i = i0 + u * stride;
+                    if (i < n) {
+                        x[i] = fma(alpha, pv[u], xv[u]);
+                        const double ri = fma(-alpha, qv[u], rv[u]);
+                        r[i] = ri;
+                        rr = fma(ri, ri, rr);
+                        const double zi = mv[u] * ri;
+                        z[i] = zi;
+                        rz = fma(ri, zi, rz);
+                    }
+                }
             }
             const double v2[2] = {rr, rz};
             cg_partials<2>(v2, slot(), G);
@@ -691,14 +761,10 @@ __global__ void __launch_bounds__(CG_TPB) k_coarse_cg(SellView S, const double* 
                 o[1] = s[1];
                 o[2] = s[1] / rho;
             });
-            const double rr_all = s2[0], rho_new = s2[1];
             ++red;
-            if (rr_all <= stop2) break;
-            const double beta = s2[2];
-            rho = rho_new;
-            for (int i = tid; i < n; i += stride) p[i] = fma(beta, p[i], z[i]);
-            cg_grid_sync(bar, ++epoch, err);
-            if (__ldcg(err)) return;
+            if (s2[0] <= stop2) break;
+            rho = s2[1];
+            beta = s2[2];
         }
     }
     for (int i = tid; i < n; i += stride) xout[i] = (TO)x[i];
