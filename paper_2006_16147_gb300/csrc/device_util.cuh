@@ -96,6 +96,103 @@ __device__ __forceinline__ double block_sums(const double (&v)[NV]) {
     return w < NV ? warp_sum(s0) : 0.0;
 }
 
+// Programmatic dependent launch: a kernel started with launch_dep (below, host
+// side) may begin while the kernel before it on the stream still runs. It does
+// what needs only the hierarchy's arrays, then dep_wait() returns when that
+// kernel is done and its writes are visible; and only then may the next one
+// begin, so at most two kernels overlap. Vectors that an earlier kernel wrote
+// are read after the wait and with ldv: an ordinary load, never ld.nc, which
+// the compiler picks for const __restrict__ pointers and which the wait does
+// not order.
+__device__ __forceinline__ void dep_wait() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+template <typename T>
+__device__ __forceinline__ T ldv(const T* p) { return __ldca(p); }
+
+// ----------------------------------------- FP64 beside a slow FP64 pipe ----
+// Conversions and adds of doubles cost 64 issue cycles per warp here, FP32 and
+// integer instructions one or two. The conversions below are the same values
+// from the IEEE formats' fields; the rare cases that are not a matter of moving
+// fields (subnormal results and inputs, infinities, NaN) take the conversion
+// instruction.
+__device__ __forceinline__ double f2d(float f) {
+    const unsigned u = __float_as_uint(f), a = u & 0x7fffffffu;
+    if (a - 0x00800000u >= 0x7f000000u && a != 0u) return (double)f;
+    return __hiloint2double((int)((a ? (a >> 3) + 0x38000000u : 0u) | (u & 0x80000000u)), (int)(u << 29));
+}
+
+__device__ __forceinline__ float d2f(double d) {
+    const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
+    const unsigned e = (hi >> 20) & 0x7ffu;
+    if (e - 897u >= 253u && ((hi << 1) | lo)) return (float)d;    // results from 2^-126 below 2^127: never overflows
+    unsigned t = (__funnelshift_l(lo, hi, 3) - (896u << 23)) & 0x7fffffffu;
+    const unsigned rest = lo << 3;                                // the 29 bits below the result's last
+    t += rest > 0x80000000u || (rest == 0x80000000u && (t & 1u));
+    return __uint_as_float((e ? t : 0u) | (hi & 0x80000000u));
+}
+
+// A double of magnitude 2^-80 .. 2^127 as three floats, exactly: 24, 23 and 6
+// bits of its mantissa. Anything else but zero gives NaN.
+struct Split3 {
+    float h, m, l;
+    bool one;         // the double is a float: m = l = 0
+};
+__device__ __forceinline__ Split3 split3(double a) {
+    const unsigned hi = (unsigned)__double2hiint(a), lo = (unsigned)__double2loint(a);
+    const unsigned sgn = hi & 0x80000000u, t = (__funnelshift_l(lo, hi, 3) - (896u << 23)) & 0x7fffffffu;
+    const unsigned rest = lo & 0x1fffffffu;
+    Split3 s{__uint_as_float(t | sgn), 0.0f, 0.0f, rest == 0u};
+    if (rest) {
+        const unsigned e = (t & 0x7f800000u) | sgn, em = e - (23u << 23), el = e - (46u << 23);
+        s.m = __uint_as_float(em | (rest >> 6)) - __uint_as_float(em);
+        s.l = __uint_as_float(el | ((rest & 63u) << 17)) - __uint_as_float(el);
+    }
+    if (((hi >> 20) & 0x7ffu) - 943u > 207u) s.h = ((hi << 1) | lo) ? __uint_as_float(0x7fc00000u) : 0.0f;
+    return s;
+}
+
+// Sum of products a z of doubles a (split) and floats z without the FP64 pipe:
+// the products' high parts summed exactly into s1 + s2 (an error-free product
+// by fma, Knuth's two-sum), what those leave, 2^-46 of the largest product and
+// below, into s3. value() rounds twice in FP64, so the sum is nearer than a
+// chain of FP64 FMAs, as long as ok(): the largest product lies in
+// 2^-60 .. 2^120 and nothing was infinite or NaN (else the caller takes the
+// FP64 chain).
+struct SplitSum {
+    float s1 = 0.0f, s2 = 0.0f, s3 = 0.0f, big = 0.0f;
+    static __device__ __forceinline__ float two_sum(float& s, float x) {
+        const float t = __fadd_rn(s, x), b = __fadd_rn(t, -s);
+        const float e = __fadd_rn(__fadd_rn(s, -__fadd_rn(t, -b)), __fadd_rn(x, -b));
+        s = t;
+        return e;
+    }
+    __device__ __forceinline__ void add(const Split3& a, float z) {
+        const float h = __fmul_rn(a.h, z), e = __fmaf_rn(a.h, z, -h);
+        big = fmaxf(big, fabsf(h));
+        const float t = two_sum(s1, h);
+        s3 = __fadd_rn(s3, two_sum(s2, t));
+        s3 = __fadd_rn(s3, two_sum(s2, e));
+        if (!a.one) {
+            const float g = __fmul_rn(a.m, z);
+            s3 = __fadd_rn(s3, two_sum(s2, g));
+            s3 = __fadd_rn(s3, __fmaf_rn(a.m, z, -g));
+            s3 = __fmaf_rn(a.l, z, s3);
+        }
+    }
+    __device__ __forceinline__ bool ok() const {
+        return big >= 0x1p-60f && big <= 0x1p120f && fabsf(s1) <= 0x1p126f;   // false for NaN
+    }
+    // as f2d, with magnitudes below 2^-126 (2^-66 of the largest product) taken as zero
+    static __device__ __forceinline__ double wide(float f) {
+        const unsigned u = __float_as_uint(f), a = u & 0x7fffffffu;
+        return a < 0x00800000u ? 0.0
+                               : __hiloint2double((int)((a >> 3) + 0x38000000u | (u & 0x80000000u)), (int)(u << 29));
+    }
+    __device__ __forceinline__ double value() const { return wide(s1) + (wide(s2) + wide(s3)); }
+};
+
 // Block-wide exclusive scan of ints.
 __device__ __forceinline__ int block_exclusive_scan_int(int v) {
     __shared__ int ws[32];

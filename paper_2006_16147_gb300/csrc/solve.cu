@@ -42,7 +42,7 @@ __device__ void finish(int mode, double a, double b, PcgScalars* sc) {
             break;
         }
         case FIN_RR: sc->rr = a; break;
-        case FIN_RHO_INIT: sc->rho = a; if (!isfinite(a)) sc->breakdown = 1; break;
+        case FIN_RHO_INIT: sc->rho = a; sc->beta = 0.0; if (!isfinite(a)) sc->breakdown = 1; break;
         case FIN_RHO_UPDATE: {
             const double beta = a / sc->rho;
             sc->rho_new = a;
@@ -119,43 +119,99 @@ __device__ __forceinline__ int sell_rowid(const SellView& S, int ip) { return S.
 template <typename T>
 __device__ __forceinline__ T ld(const T* p) { return __ldg(p); }
 
-// Row dot product of one SELL slice lane: sum_k val[k] * xv(col[k]). The
-// loop is unrolled by four so that the column, value and gather loads of four
-// entries are in flight together. Two accumulators shorten the FMA chain
-// (latency-bound kernels); one accumulator saves the final add, which pays in
-// the fused smoothers, where the FP64 pipe (this GPU's FP64 rate is 1/64 of
-// its FP32 rate) is the bound.
-template <typename T, int NACC = 2, typename F>
-__device__ __forceinline__ T sell_row(const int* __restrict__ col, const T* __restrict__ val, long long base, int w,
-                                      F&& xv) {
-    T a0 = 0, a1 = 0;
-    int k = 0;
-    for (; k + 4 <= w; k += 4, base += 128) {
-        const int j0 = ld(col + base), j1 = ld(col + base + 32), j2 = ld(col + base + 64), j3 = ld(col + base + 96);
-        const T v0 = ld(val + base), v1 = ld(val + base + 32), v2 = ld(val + base + 64), v3 = ld(val + base + 96);
-        const T x0 = xv(j0), x1 = xv(j1), x2 = xv(j2), x3 = xv(j3);
-        if (NACC == 1) {
-            a0 = fma(v0, x0, a0);
-            a0 = fma(v1, x1, a0);
-            a0 = fma(v2, x2, a0);
-            a0 = fma(v3, x3, a0);
-        } else {
-            a0 = fma(v0, x0, a0);
-            a1 = fma(v1, x1, a1);
-            a0 = fma(v2, x2, a0);
-            a1 = fma(v3, x3, a1);
-        }
+// Row dot product of one SELL slice lane: sum_k val[k] * xv(col[k]), entries
+// taken RB at a time: a batch's columns and values are in flight together, then
+// its gathers. load() fetches the first batch, which needs only the matrix,
+// ahead of the wait for the kernel before. Two sizes (sell_small):
+//   RB = 8  the slices of a small matrix, all resident at once: a row of up to
+//           eight entries costs two memory latencies, not the eight of four and
+//           then one by one, which were most of a 5-7 us kernel
+//   RB = 4  the others, in 32 registers: with all 64 warps of an SM the FP64
+//           pipe and the memory work side by side; at half of them they take
+//           turns (256^3 level 0 with RB = 8: k_post 262 -> 452 us)
+// Two accumulators shorten the FMA chain (latency-bound kernels); one saves the
+// final add, which pays in the fused smoothers, where the FP64 pipe (this GPU's
+// FP64 rate is 1/64 of its FP32 rate) is the bound.
+template <int RB, typename T>
+struct RowBatch {
+    int w;
+    long long base;
+    int j[RB];
+    T v[RB];
+    __device__ __forceinline__ void fetch(const int* __restrict__ col, const T* __restrict__ val, int k) {
+#pragma unroll
+        for (int u = 0; u < RB; ++u)
+            if (k + u < w) {
+                j[u] = ld(col + base + 32 * (k + u));
+                v[u] = ld(val + base + 32 * (k + u));
+            }
     }
-    for (; k < w; ++k, base += 32) a0 = fma(ld(val + base), xv(ld(col + base)), a0);
-    return NACC == 1 ? a0 : a0 + a1;
-}
+    __device__ __forceinline__ void load(const SellView& S, const T* __restrict__ val, int s) {
+        const int s0 = ld(S.sptr + s);
+        w = ld(S.sptr + s + 1) - s0;
+        base = (long long)s0 * 32 + (threadIdx.x & 31);
+        if (RB == 8) fetch(S.col, val, 0);
+    }
+    template <int NACC = 2, typename F>
+    __device__ __forceinline__ T dot(const SellView& S, const T* __restrict__ val, F&& xv) {
+        T a0 = 0, a1 = 0;
+        if constexpr (RB == 4) {
+            const int* c = S.col + base;
+            const T* a = val + base;
+            int k = 0;
+            for (; k + 4 <= w; k += 4, c += 128, a += 128) {
+                const int j0 = ld(c), j1 = ld(c + 32), j2 = ld(c + 64), j3 = ld(c + 96);
+                const T v0 = ld(a), v1 = ld(a + 32), v2 = ld(a + 64), v3 = ld(a + 96);
+                const T x0 = xv(j0), x1 = xv(j1), x2 = xv(j2), x3 = xv(j3);
+                a0 = fma(v0, x0, a0);
+                if (NACC == 1) a0 = fma(v1, x1, a0);
+                else a1 = fma(v1, x1, a1);
+                a0 = fma(v2, x2, a0);
+                if (NACC == 1) a0 = fma(v3, x3, a0);
+                else a1 = fma(v3, x3, a1);
+            }
+            for (; k < w; ++k, c += 32, a += 32) a0 = fma(ld(a), xv(ld(c)), a0);
+            return NACC == 1 ? a0 : a0 + a1;
+        }
+        for (int k = 0;;) {
+            T x[RB];
+#pragma unroll
+            for (int u = 0; u < RB; ++u)
+                if (k + u < w) x[u] = xv(j[u]);
+#pragma unroll
+            for (int u = 0; u < RB; ++u)
+                if (k + u < w) {
+                    if (NACC == 1 || u % 2 == 0) a0 = fma(v[u], x[u], a0);
+                    else a1 = fma(v[u], x[u], a1);
+                }
+            k += RB;
+            if (k >= w) break;
+            fetch(S.col, val, k);
+        }
+        return NACC == 1 ? a0 : a0 + a1;
+    }
+};
+// A vector that an earlier kernel wrote: RB = 8 kernels start before that one
+// ends, RB = 4 kernels after it.
+template <int RB, typename T>
+__device__ __forceinline__ T ldx(const T* p) { return RB == 8 ? ldv(p) : ld(p); }
+// resident blocks per SM that the register budget of a batch size allows
+#define SELL_BOUNDS __launch_bounds__(TPB, RB == 4 ? 8 : 4)
 
-#define SELL_LOOP(S)                                                                 \
-    const int lane = threadIdx.x & 31;                                               \
-    const int nw_ = gridDim.x * WARPS;                                               \
-    for (int s = blockIdx.x * WARPS + (threadIdx.x >> 5); s < (S).nslices; s += nw_)
+__device__ __forceinline__ double to_d(double v) { return v; }
+__device__ __forceinline__ double to_d(float v) { return f2d(v); }
 
-#define SELL_ROW_ARGS(S) (S).col, (long long)(S).sptr[s] * 32 + lane, (S).sptr[s + 1] - (S).sptr[s]
+// Slices of this warp: `s`, with the first batch of its row in `row`. With
+// RB = 8 waits for the kernel before (after the first batch's loads) and lets
+// the next one start.
+#define SELL_LOOP(S, T, val)                                                               \
+    const int lane = threadIdx.x & 31;                                                     \
+    const int nw_ = gridDim.x * WARPS;                                                     \
+    RowBatch<RB, T> row;                                                                   \
+    int s = blockIdx.x * WARPS + (threadIdx.x >> 5);                                       \
+    if (s < (S).nslices) row.load(S, val, s);                                              \
+    if (RB == 8) dep_wait();                                                               \
+    for (; s < (S).nslices; s += nw_, s < (S).nslices ? row.load(S, val, s) : (void)0)
 
 // --------------------------------------------------------- V-cycle ---------
 // First pre-smoothing sweep from a zero guess, fused with the residual:
@@ -164,17 +220,16 @@ __device__ __forceinline__ T sell_row(const int* __restrict__ col, const T* __re
 // wm = omega M^-1. With U (one pre-smoothing sweep), x is not stored but
 // u = x + omega M^-1 r = omega M^-1 (b + r), the part of the post-smoother
 // that does not depend on the coarse correction.
-template <typename T, typename TB, bool U>
-__global__ void __launch_bounds__(TPB) k_pre(SellView S, const T* __restrict__ valm, const T* __restrict__ wm,
+template <int RB, typename T, typename TB, bool U>
+__global__ void SELL_BOUNDS k_pre(SellView S, const T* __restrict__ valm, const T* __restrict__ wm,
                                              T omega, const TB* __restrict__ b, T* __restrict__ x,
                                              T* __restrict__ r) {
-    SELL_LOOP(S) {
-        const T acc = sell_row<T, 1>(S.col, valm, (long long)S.sptr[s] * 32 + lane, S.sptr[s + 1] - S.sptr[s],
-                               [&](int j) { return (T)ld(b + j); });
+    SELL_LOOP(S, T, valm) {
+        const T acc = row.template dot<1>(S, valm, [&](int j) { return (T)ldx<RB>(b + j); });
         const int ip = s * 32 + lane;
         if (ip < S.n) {
             const int i = sell_rowid(S, ip);
-            const T bi = (T)b[i];
+            const T bi = (T)ldx<RB>(b + i);
             const T ri = fma(-omega, acc, bi);
             r[i] = ri;
             x[i] = U ? wm[i] * (bi + ri) : wm[i] * bi;
@@ -182,38 +237,48 @@ __global__ void __launch_bounds__(TPB) k_pre(SellView S, const T* __restrict__ v
     }
 }
 
-// Member sum of aggregate q, sum_i p_i r_i in ascending order. Up to eight
-// members (three pairwise sweeps give no more) are loaded together: three
-// memory latencies per aggregate (bounds, members, p and r) instead of two
-// per member.
-template <typename T, typename F>
-__device__ __forceinline__ T member_sum(const int* __restrict__ pt_ptr, const int* __restrict__ pt_idx,
-                                        const T* __restrict__ p, int q, F&& rv) {
-    T s = 0;
-    const int e = ld(pt_ptr + q + 1);
-    for (int k = ld(pt_ptr + q); k < e; k += 8) {
-        int i[8];
-        T pv[8], rr[8];
+// Restriction: bc_q = sum_i p_i r_i over the members of aggregate q in
+// ascending order. Up to eight members (three pairwise sweeps give no more) are
+// loaded together; bounds, members and p come from the hierarchy and are there
+// before the wait for the kernel that writes r.
+template <typename T>
+__global__ void __launch_bounds__(TPB) k_restrict(int nc, const int* __restrict__ pt_ptr, const int* __restrict__ pt_idx,
+                                                  const T* __restrict__ p, const T* __restrict__ r, T* __restrict__ bc) {
+    int q = blockIdx.x * blockDim.x + threadIdx.x;
+    int k = 0, e = 0, i[8];
+    T pv[8];
+    auto fetch = [&]() {
 #pragma unroll
         for (int t = 0; t < 8; ++t) i[t] = k + t < e ? ld(pt_idx + k + t) : -1;
 #pragma unroll
         for (int t = 0; t < 8; ++t)
-            if (i[t] >= 0) {
-                pv[t] = ld(p + i[t]);
-                rr[t] = rv(i[t]);
-            }
+            if (i[t] >= 0) pv[t] = ld(p + i[t]);
+    };
+    auto open = [&]() {
+        k = ld(pt_ptr + q);
+        e = ld(pt_ptr + q + 1);
+        fetch();
+    };
+    if (q < nc) open();
+    dep_wait();
+    while (q < nc) {
+        T s = 0;
+        for (;;) {
+            T rv[8];
 #pragma unroll
-        for (int t = 0; t < 8; ++t)
-            if (i[t] >= 0) s = fma(pv[t], rr[t], s);
+            for (int t = 0; t < 8; ++t)
+                if (i[t] >= 0) rv[t] = ldv(r + i[t]);
+#pragma unroll
+            for (int t = 0; t < 8; ++t)
+                if (i[t] >= 0) s = fma(pv[t], rv[t], s);
+            k += 8;
+            if (k >= e) break;
+            fetch();
+        }
+        bc[q] = s;
+        q += gridDim.x * blockDim.x;
+        if (q < nc) open();
     }
-    return s;
-}
-
-template <typename T>
-__global__ void __launch_bounds__(TPB) k_restrict(int nc, const int* __restrict__ pt_ptr, const int* __restrict__ pt_idx,
-                                                  const T* __restrict__ p, const T* __restrict__ r, T* __restrict__ bc) {
-    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < nc; q += gridDim.x * blockDim.x)
-        bc[q] = member_sum(pt_ptr, pt_idx, p, q, [&](int i) { return ld(r + i); });
 }
 
 // Coarse correction and first post-smoothing sweep, fused:
@@ -226,26 +291,26 @@ __global__ void __launch_bounds__(TPB) k_restrict(int nc, const int* __restrict_
 // wm = omega M^-1. With DOT, also bdot . out (r . z of CG on level 0),
 // finished into the CG scalars. FP64 work per row: one FMA per entry of
 // apw, two more, and the dot.
-template <typename T, typename TB, typename TO, bool DOT, bool U>
-__global__ void __launch_bounds__(TPB) k_post(SellView SAP, const T* __restrict__ apw, const T* __restrict__ wm,
+template <int RB, typename T, typename TB, typename TO, bool DOT, bool U>
+__global__ void SELL_BOUNDS k_post(SellView SAP, const T* __restrict__ apw, const T* __restrict__ wm,
                                               const int* __restrict__ agg, const T* __restrict__ p,
                                               const T* __restrict__ e, const T* __restrict__ x,
                                               const T* __restrict__ r, const TB* __restrict__ bdot,
                                               TO* __restrict__ out, Reducer red, PcgScalars* sc, int mode,
                                               const double* __restrict__ q2) {
     double dot = 0.0, dot2 = 0.0;
-    SELL_LOOP(SAP) {
-        const T acc = sell_row<T, 1>(SAP.col, apw, (long long)SAP.sptr[s] * 32 + lane, SAP.sptr[s + 1] - SAP.sptr[s],
-                               [&](int q) { return ld(e + q); });
+    SELL_LOOP(SAP, T, apw) {
+        const T acc = row.template dot<1>(SAP, apw, [&](int q) { return ldx<RB>(e + q); });
         const int ip = s * 32 + lane;
         if (ip < SAP.n) {
             const int i = sell_rowid(SAP, ip);
-            const T ui = U ? x[i] : fma(wm[i], r[i], x[i]);
-            const T o = fma(p[i], e[agg[i]], ui) - acc;
+            const T ui = U ? ldx<RB>(x + i) : fma(wm[i], ldx<RB>(r + i), ldx<RB>(x + i));
+            const T o = fma(p[i], ldx<RB>(e + agg[i]), ui) - acc;
             out[i] = (TO)o;
             if (DOT) {
-                dot = fma((double)bdot[i], (double)(TO)o, dot);
-                if (q2) dot2 = fma(q2[i], (double)(TO)o, dot2);
+                const double od = to_d((TO)o);
+                dot = fma((double)ldx<RB>(bdot + i), od, dot);
+                if (q2) dot2 = fma(ldx<RB>(q2 + i), od, dot2);
             }
         }
     }
@@ -255,20 +320,38 @@ __global__ void __launch_bounds__(TPB) k_post(SellView SAP, const T* __restrict_
     }
 }
 
+// Whether all slices are resident at once with four blocks of the RB = 8
+// kernels per SM.
+bool sell_small(const amg_hierarchy* h, const SellView& S) { return S.nslices <= h->num_sms * 4 * WARPS; }
+// RB = 8 kernels begin beside the kernel before; for a large matrix that gains
+// nothing, and the compiler keeps its freedom with ld.nc.
+template <int RB, typename... P, typename... A>
+void launch_sell(void (*kernel)(P...), int grid, cudaStream_t st, A&&... args) {
+    if (RB == 8) launch_dep(kernel, grid, TPB, 0, st, std::forward<A>(args)...);
+    else kernel<<<grid, TPB, 0, st>>>(std::forward<A>(args)...);
+}
+#define SELL_DISPATCH(h, S, ...)                                    \
+    do {                                                            \
+        if (sell_small(h, S)) { constexpr int RB = 8; __VA_ARGS__; } \
+        else { constexpr int RB = 4; __VA_ARGS__; }                 \
+    } while (0)
+
 template <typename T, typename TB>
-void launch_pre(bool u, int grid, cudaStream_t st, SellView S, const T* valm, const T* wm, T omega, const TB* b, T* x,
+void launch_pre(const amg_hierarchy* h, bool u, int grid, cudaStream_t st, SellView S, const T* valm, const T* wm, T omega, const TB* b, T* x,
                 T* r) {
-    if (u) k_pre<T, TB, true><<<grid, TPB, 0, st>>>(S, valm, wm, omega, b, x, r);
-    else k_pre<T, TB, false><<<grid, TPB, 0, st>>>(S, valm, wm, omega, b, x, r);
+    SELL_DISPATCH(h, S, if (u) launch_sell<RB>(k_pre<RB, T, TB, true>, grid, st, S, valm, wm, omega, b, x, r);
+                  else launch_sell<RB>(k_pre<RB, T, TB, false>, grid, st, S, valm, wm, omega, b, x, r));
     KERNEL_CHECK();
 }
 
 template <typename T, typename TB, typename TO, bool DOT>
-void launch_post(bool u, int grid, cudaStream_t st, SellView SAP, const T* apw, const T* wm, const int* agg,
+void launch_post(const amg_hierarchy* h, bool u, int grid, cudaStream_t st, SellView SAP, const T* apw, const T* wm, const int* agg,
                  const T* p, const T* e, const T* x, const T* r, const TB* bdot, TO* out, Reducer red, PcgScalars* sc,
                  int mode, const double* q2) {
-    if (u) k_post<T, TB, TO, DOT, true><<<grid, TPB, 0, st>>>(SAP, apw, wm, agg, p, e, x, r, bdot, out, red, sc, mode, q2);
-    else k_post<T, TB, TO, DOT, false><<<grid, TPB, 0, st>>>(SAP, apw, wm, agg, p, e, x, r, bdot, out, red, sc, mode, q2);
+    SELL_DISPATCH(h, SAP, if (u) launch_sell<RB>(k_post<RB, T, TB, TO, DOT, true>, grid, st, SAP, apw, wm, agg, p, e, x,
+                                            r, bdot, out, red, sc, mode, q2);
+                  else launch_sell<RB>(k_post<RB, T, TB, TO, DOT, false>, grid, st, SAP, apw, wm, agg, p, e, x, r,
+                                  bdot, out, red, sc, mode, q2));
     KERNEL_CHECK();
 }
 
@@ -293,21 +376,20 @@ __device__ __forceinline__ void kc_finish(KcScalars* ks, int mode, double a, dou
 }
 
 // q1 = A d1; d1.q1 and d1.b -> rho1, alpha1.
-template <typename T>
-__global__ void __launch_bounds__(TPB) k_kc_spmv_dot(SellView S, const T* __restrict__ val, const T* __restrict__ d1,
+template <int RB, typename T>
+__global__ void SELL_BOUNDS k_kc_spmv_dot(SellView S, const T* __restrict__ val, const T* __restrict__ d1,
                                                      T* __restrict__ q1, const T* __restrict__ b, Reducer red,
                                                      KcScalars* ks) {
     double dq = 0.0, db = 0.0;
-    SELL_LOOP(S) {
-        const T acc = sell_row(S.col, val, (long long)S.sptr[s] * 32 + lane, S.sptr[s + 1] - S.sptr[s],
-                               [&](int j) { return ld(d1 + j); });
+    SELL_LOOP(S, T, val) {
+        const T acc = row.dot(S, val, [&](int j) { return ldx<RB>(d1 + j); });
         const int ip = s * 32 + lane;
         if (ip < S.n) {
             const int i = sell_rowid(S, ip);
             q1[i] = acc;
-            const double di = (double)d1[i];
+            const double di = (double)ldx<RB>(d1 + i);
             dq = fma(di, (double)acc, dq);
-            db = fma(di, (double)b[i], db);
+            db = fma(di, (double)ldx<RB>(b + i), db);
         }
     }
     reduce_then<2>(dq, db, red, [&](double a, double c) { kc_finish(ks, KC_ALPHA1, a, c); });
@@ -318,10 +400,11 @@ template <typename T>
 __global__ void __launch_bounds__(TPB) k_kc_update1(int n, const T* __restrict__ d1, const T* __restrict__ q1,
                                                     const T* __restrict__ b, T* __restrict__ e, T* __restrict__ r2,
                                                     const KcScalars* ks) {
+    dep_wait();
     const T a = (T)ks->alpha1;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        e[i] = a * d1[i];
-        r2[i] = fma(-a, q1[i], b[i]);
+        e[i] = a * ldv(d1 + i);
+        r2[i] = fma(-a, ldv(q1 + i), ldv(b + i));
     }
 }
 
@@ -330,31 +413,31 @@ template <typename T>
 __global__ void __launch_bounds__(TPB) k_kc_dot(int n, const T* __restrict__ z2, const T* __restrict__ q1, Reducer red,
                                                 KcScalars* ks) {
     double s = 0.0;
+    dep_wait();
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-        s = fma((double)z2[i], (double)q1[i], s);
+        s = fma((double)ldv(z2 + i), (double)ldv(q1 + i), s);
     reduce_then<1>(s, 0.0, red, [&](double a, double) { kc_finish(ks, KC_BETA, a, 0.0); });
 }
 
 // d2 = z2 - beta d1; q2 = A z2 - beta q1 (= A d2, without a second product);
 // d2.q2 and d2.r2 -> alpha2.
-template <typename T>
-__global__ void __launch_bounds__(TPB) k_kc_spmv2(SellView S, const T* __restrict__ val, const T* __restrict__ z2,
+template <int RB, typename T>
+__global__ void SELL_BOUNDS k_kc_spmv2(SellView S, const T* __restrict__ val, const T* __restrict__ z2,
                                                   const T* __restrict__ q1, const T* __restrict__ d1,
                                                   const T* __restrict__ r2, T* __restrict__ d2, Reducer red,
                                                   KcScalars* ks) {
-    const T be = (T)ks->beta;
     double dq = 0.0, dr = 0.0;
-    SELL_LOOP(S) {
-        const T acc = sell_row(S.col, val, (long long)S.sptr[s] * 32 + lane, S.sptr[s + 1] - S.sptr[s],
-                               [&](int j) { return ld(z2 + j); });
+    SELL_LOOP(S, T, val) {
+        const T be = (T)ks->beta;
+        const T acc = row.dot(S, val, [&](int j) { return ldx<RB>(z2 + j); });
         const int ip = s * 32 + lane;
         if (ip < S.n) {
             const int i = sell_rowid(S, ip);
-            const T q2 = fma(-be, q1[i], acc);
-            const T di = fma(-be, d1[i], z2[i]);
+            const T q2 = fma(-be, ldx<RB>(q1 + i), acc);
+            const T di = fma(-be, ldx<RB>(d1 + i), ldx<RB>(z2 + i));
             d2[i] = di;
             dq = fma((double)di, (double)q2, dq);
-            dr = fma((double)di, (double)r2[i], dr);
+            dr = fma((double)di, (double)ldx<RB>(r2 + i), dr);
         }
     }
     reduce_then<2>(dq, dr, red, [&](double a, double c) { kc_finish(ks, KC_ALPHA2, a, c); });
@@ -364,18 +447,19 @@ __global__ void __launch_bounds__(TPB) k_kc_spmv2(SellView S, const T* __restric
 template <typename T>
 __global__ void __launch_bounds__(TPB) k_kc_update2(int n, const T* __restrict__ d2, T* __restrict__ e,
                                                     const KcScalars* ks) {
+    dep_wait();
     const T a = (T)ks->alpha2;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) e[i] = fma(a, d2[i], e[i]);
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
+        e[i] = fma(a, ldv(d2 + i), e[i]);
 }
 
 // ------------------------------------------- smoothed prolongator (SA) ----
 // Restriction b_c = Pbar^T r (rows of Pbar^T in SELL).
-template <typename T>
-__global__ void __launch_bounds__(TPB) k_sell_spmv(SellView S, const T* __restrict__ val, const T* __restrict__ x,
+template <int RB, typename T>
+__global__ void SELL_BOUNDS k_sell_spmv(SellView S, const T* __restrict__ val, const T* __restrict__ x,
                                                    T* __restrict__ y) {
-    SELL_LOOP(S) {
-        const T acc = sell_row(S.col, val, (long long)S.sptr[s] * 32 + lane, S.sptr[s + 1] - S.sptr[s],
-                               [&](int j) { return ld(x + j); });
+    SELL_LOOP(S, T, val) {
+        const T acc = row.dot(S, val, [&](int j) { return ldx<RB>(x + j); });
         const int ip = s * 32 + lane;
         if (ip < S.n) y[sell_rowid(S, ip)] = acc;
     }
@@ -402,11 +486,12 @@ __global__ void __launch_bounds__(TPB) k_wide(int n, const int* __restrict__ ptr
                                               double* __restrict__ xo) {
     const int lane = threadIdx.x & 31;
     const int nw = (gridDim.x * blockDim.x) >> 5;
+    dep_wait();
     for (int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n; i += nw) {
         const int kb = ptr[i], ke = ptr[i + 1];
         double acc0 = 0.0, acc1 = 0.0;
         int k = kb + lane;
-        auto xv = [&](int j) { return ld(x + j); };
+        auto xv = [&](int j) { return ldv(x + j); };
         for (; k + 32 < ke; k += 64) {
             const int j0 = col[k], j1 = col[k + 32];
             const double v0 = OP == W_PRE ? val[k] * minv[j0] : val[k];
@@ -426,12 +511,12 @@ __global__ void __launch_bounds__(TPB) k_wide(int n, const int* __restrict__ ptr
             if (OP == W_SPMV) y[i] = acc;
             if (OP == W_ADD) y[i] = y[i] + acc;
             if (OP == W_PRE) {
-                const double bi = b[i];
+                const double bi = ldv(b + i);
                 y[i] = fma(-omega, acc, bi);
                 xo[i] = wm[i] * bi;
             }
-            if (OP == W_SMOOTH) y[i] = fma(omega * minv[i], b[i] - acc, x[i]);
-            if (OP == W_RES) y[i] = b[i] - acc;
+            if (OP == W_SMOOTH) y[i] = fma(omega * minv[i], ldv(b + i) - acc, ldv(x + i));
+            if (OP == W_RES) y[i] = ldv(b + i) - acc;
         }
     }
 }
@@ -439,12 +524,11 @@ __global__ void __launch_bounds__(TPB) k_wide(int n, const int* __restrict__ ptr
 bool wide(const DevCsr& M, int min_mean) { return M.n > 0 && (long long)M.nnz >= (long long)min_mean * M.n; }
 
 // Prolongation x <- x + Pbar e (rows of Pbar in SELL).
-template <typename T>
-__global__ void __launch_bounds__(TPB) k_prolong(SellView S, const T* __restrict__ val, const T* __restrict__ e,
+template <int RB, typename T>
+__global__ void SELL_BOUNDS k_prolong(SellView S, const T* __restrict__ val, const T* __restrict__ e,
                                                  T* __restrict__ x) {
-    SELL_LOOP(S) {
-        const T acc = sell_row(S.col, val, (long long)S.sptr[s] * 32 + lane, S.sptr[s + 1] - S.sptr[s],
-                               [&](int q) { return ld(e + q); });
+    SELL_LOOP(S, T, val) {
+        const T acc = row.dot(S, val, [&](int q) { return ldx<RB>(e + q); });
         const int ip = s * 32 + lane;
         if (ip < S.n) {
             const int i = sell_rowid(S, ip);
@@ -459,55 +543,57 @@ __global__ void __launch_bounds__(TPB) k_prolong(SellView S, const T* __restrict
 __global__ void __launch_bounds__(TPB) k_to_f32(int n, const double* __restrict__ a, float* __restrict__ b) {
     const int stride = gridDim.x * blockDim.x;
     int i = blockIdx.x * blockDim.x + threadIdx.x;
+    dep_wait();
     for (; i + stride < n; i += 2 * stride) {
-        const double a0 = a[i], a1 = a[i + stride];
-        b[i] = (float)a0;
-        b[i + stride] = (float)a1;
+        const double a0 = ldv(a + i), a1 = ldv(a + i + stride);
+        b[i] = d2f(a0);
+        b[i + stride] = d2f(a1);
     }
-    if (i < n) b[i] = (float)a[i];
+    if (i < n) b[i] = d2f(ldv(a + i));
 }
 
 // Residual after the last of several pre-smoothing sweeps: r = b - A x.
 // (Sweeps between the first and the last are k_smooth, the first is k_pre
 // storing x + omega M^-1 r; each reads one gathered vector, one FMA per
 // stored entry.)
-template <typename T, typename TB>
-__global__ void __launch_bounds__(TPB) k_resid(SellView S, const T* __restrict__ val, const TB* __restrict__ b,
+template <int RB, typename T, typename TB>
+__global__ void SELL_BOUNDS k_resid(SellView S, const T* __restrict__ val, const TB* __restrict__ b,
                                                const T* __restrict__ x, T* __restrict__ r) {
-    SELL_LOOP(S) {
-        const T acc = sell_row(S.col, val, (long long)S.sptr[s] * 32 + lane, S.sptr[s + 1] - S.sptr[s],
-                               [&](int j) { return ld(x + j); });
+    SELL_LOOP(S, T, val) {
+        const T acc = row.dot(S, val, [&](int j) { return ldx<RB>(x + j); });
         const int ip = s * 32 + lane;
         if (ip < S.n) {
             const int i = sell_rowid(S, ip);
-            r[i] = (T)b[i] - acc;
+            r[i] = (T)ldx<RB>(b + i) - acc;
         }
     }
 }
 
 // Extra post-smoothing sweep: y' = y + omega M^-1 (b - A y).
-template <typename T, typename TB, typename TO>
-__global__ void __launch_bounds__(TPB) k_smooth(SellView S, const T* __restrict__ val, const T* __restrict__ minv,
+template <int RB, typename T, typename TB, typename TO>
+__global__ void SELL_BOUNDS k_smooth(SellView S, const T* __restrict__ val, const T* __restrict__ minv,
                                                 T omega, const TB* __restrict__ b, const T* __restrict__ yin,
                                                 TO* __restrict__ yout) {
-    SELL_LOOP(S) {
-        const T acc = sell_row(S.col, val, (long long)S.sptr[s] * 32 + lane, S.sptr[s + 1] - S.sptr[s],
-                               [&](int j) { return ld(yin + j); });
+    SELL_LOOP(S, T, val) {
+        const T acc = row.dot(S, val, [&](int j) { return ldx<RB>(yin + j); });
         const int ip = s * 32 + lane;
         if (ip < S.n) {
             const int i = sell_rowid(S, ip);
-            yout[i] = (TO)fma(omega * minv[i], (T)b[i] - acc, yin[i]);
+            yout[i] = (TO)fma(omega * minv[i], (T)ldx<RB>(b + i) - acc, ldx<RB>(yin + i));
         }
     }
 }
 
 // a . b and, if c is given, b . c.
-__global__ void __launch_bounds__(TPB) k_dot(int n, const double* __restrict__ a, const double* __restrict__ b,
+template <typename TZ>
+__global__ void __launch_bounds__(TPB) k_dot(int n, const double* __restrict__ a, const TZ* __restrict__ b,
                                              const double* __restrict__ c, Reducer red, PcgScalars* sc, int mode) {
     double d = 0.0, d2 = 0.0;
+    dep_wait();
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        d = fma(a[i], b[i], d);
-        if (c) d2 = fma(b[i], c[i], d2);
+        const double bi = to_d(ldv(b + i));
+        d = fma(ldv(a + i), bi, d);
+        if (c) d2 = fma(bi, ldv(c + i), d2);
     }
     if (c) reduce_and_finish<2>(d, d2, red, sc, mode);
     else reduce_and_finish<1>(d, 0.0, red, sc, mode);
@@ -517,7 +603,8 @@ __global__ void __launch_bounds__(TPB) k_dot(int n, const double* __restrict__ a
 template <typename T, typename TO>
 __global__ void k_coarse_solve(int n, const double* __restrict__ Ainv, const T* __restrict__ b, TO* __restrict__ x) {
     extern __shared__ double bs[];
-    for (int j = threadIdx.x; j < n; j += blockDim.x) bs[j] = (double)b[j];
+    dep_wait();
+    for (int j = threadIdx.x; j < n; j += blockDim.x) bs[j] = (double)ldv(b + j);
     __syncthreads();
     const int lane = threadIdx.x & 31;
     const int warps = blockDim.x >> 5;
@@ -777,6 +864,7 @@ __global__ void k_coarse_solve_seg(int n, int m, const int* __restrict__ segp, c
                                    const double* __restrict__ Ainv, const T* __restrict__ b, TO* __restrict__ x) {
     const int lane = threadIdx.x & 31;
     const int nw = (gridDim.x * blockDim.x) >> 5;
+    dep_wait();
     for (int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n; i += nw) {
         int lo = 0, hi = m;
         while (hi - lo > 1) {
@@ -786,7 +874,7 @@ __global__ void k_coarse_solve_seg(int n, int m, const int* __restrict__ segp, c
         const int r0 = segp[lo], ns = segp[lo + 1] - r0;
         const double* row = Ainv + blk[lo] + (long long)(i - r0) * ns;
         double acc = 0.0;
-        for (int j = lane; j < ns; j += 32) acc = fma(row[j], (double)b[r0 + j], acc);
+        for (int j = lane; j < ns; j += 32) acc = fma(row[j], (double)ldv(b + r0 + j), acc);
         acc = warp_sum(acc);
         if (lane == 0) x[i] = (TO)acc;
     }
@@ -794,17 +882,17 @@ __global__ void k_coarse_solve_seg(int n, int m, const int* __restrict__ segp, c
 
 // ------------------------------------------------------------- PCG ---------
 // r = b - A x; ||r||^2 and ||b||^2.
-__global__ void __launch_bounds__(TPB) k_residual(SellView S, const double* __restrict__ val,
+template <int RB>
+__global__ void SELL_BOUNDS k_residual(SellView S, const double* __restrict__ val,
                                                   const double* __restrict__ x, const double* __restrict__ b,
                                                   double* __restrict__ r, Reducer red, PcgScalars* sc) {
     double rr = 0.0, bb = 0.0;
-    SELL_LOOP(S) {
-        const double acc = sell_row(S.col, val, (long long)S.sptr[s] * 32 + lane, S.sptr[s + 1] - S.sptr[s],
-                                    [&](int j) { return ld(x + j); });
+    SELL_LOOP(S, double, val) {
+        const double acc = row.dot(S, val, [&](int j) { return ldx<RB>(x + j); });
         const int ip = s * 32 + lane;
         if (ip < S.n) {
             const int i = sell_rowid(S, ip);
-            const double bi = b[i];
+            const double bi = ldx<RB>(b + i);
             const double ri = bi - acc;
             r[i] = ri;
             rr = fma(ri, ri, rr);
@@ -814,24 +902,78 @@ __global__ void __launch_bounds__(TPB) k_residual(SellView S, const double* __re
     reduce_and_finish<2>(rr, bb, red, sc, FIN_NORMS);
 }
 
-// q = A p; p . q; alpha = rho / p.q.
-__global__ void __launch_bounds__(TPB) k_spmv_dot(SellView S, const double* __restrict__ val,
-                                                  const double* __restrict__ p, double* __restrict__ q, Reducer red,
-                                                  PcgScalars* sc) {
+// p = z + beta p; q = A z + beta q (= A p); p . q; alpha = rho / p.q: the
+// direction update inside the product, for small matrices, where a launch
+// counts (a solve on 32^3 rows 1297 -> 1255 us). After a restart beta = 0 and p
+// and q are not read. Large ones take k_update_p and k_spmv_dot: here the four
+// vector streams cost the registers of half the warps, and 256^3 took 564 us
+// instead of 361.
+template <int RB, typename TZ>
+__global__ void SELL_BOUNDS k_direction(SellView S, const double* __restrict__ val, const TZ* __restrict__ z,
+                                        double* __restrict__ p, double* __restrict__ q, Reducer red, PcgScalars* sc) {
     double pq = 0.0;
-    SELL_LOOP(S) {
+    SELL_LOOP(S, double, val) {
+        const double beta = sc->beta;
+        const bool first = beta == 0.0;
         const int ip = s * 32 + lane;
         const bool live = ip < S.n;
         const int i = live ? sell_rowid(S, ip) : 0;
-        const double pi = live ? ld(p + i) : 0.0;
-        const double acc = sell_row(S.col, val, (long long)S.sptr[s] * 32 + lane, S.sptr[s + 1] - S.sptr[s],
-                                    [&](int j) { return ld(p + j); });
+        double pi = 0.0, qi = 0.0;
+        if (live && !first) {
+            pi = p[i];
+            qi = q[i];
+        }
+        const double acc = row.dot(S, val, [&](int j) { return to_d(ldx<RB>(z + j)); });
         if (live) {
-            q[i] = acc;
-            pq = fma(pi, acc, pq);
+            const double zd = to_d(ldx<RB>(z + i));
+            pi = first ? zd : fma(beta, pi, zd);
+            qi = first ? acc : fma(beta, qi, acc);
+            p[i] = pi;
+            q[i] = qi;
+            pq = fma(pi, qi, pq);
         }
     }
     reduce_and_finish<1>(pq, 0.0, red, sc, FIN_PQ);
+}
+
+// q = A p; p . q; alpha = rho / p.q.
+template <int RB>
+__global__ void SELL_BOUNDS k_spmv_dot(SellView S, const double* __restrict__ val, const double* __restrict__ p,
+                                       double* __restrict__ q, Reducer red, PcgScalars* sc) {
+    double pq = 0.0;
+    SELL_LOOP(S, double, val) {
+        const int ip = s * 32 + lane;
+        const bool live = ip < S.n;
+        const int i = live ? sell_rowid(S, ip) : 0;
+        const double acc = row.dot(S, val, [&](int j) { return ldx<RB>(p + j); });
+        if (live) {
+            q[i] = acc;
+            pq = fma(ldx<RB>(p + i), acc, pq);
+        }
+    }
+    reduce_and_finish<1>(pq, 0.0, red, sc, FIN_PQ);
+}
+
+// p = z + beta p (p = z after a restart).
+template <typename TZ>
+__global__ void __launch_bounds__(TPB) k_update_p(int n, const TZ* __restrict__ z, double* __restrict__ p,
+                                                  const PcgScalars* sc) {
+    dep_wait();
+    const double beta = sc->beta;
+    const int stride = gridDim.x * blockDim.x;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += 4 * stride) {
+        TZ zv[4];
+        double pv[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (i + u * stride < n) {
+                zv[u] = ldv(z + i + u * stride);
+                pv[u] = p[i + u * stride];
+            }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (i + u * stride < n) p[i + u * stride] = beta == 0.0 ? to_d(zv[u]) : fma(beta, pv[u], to_d(zv[u]));
+    }
 }
 
 // x += alpha p; r -= alpha q; ||r||^2.
@@ -840,23 +982,17 @@ __global__ void __launch_bounds__(TPB) k_spmv_dot(SellView S, const double* __re
 __global__ void __launch_bounds__(TPB) k_update_xr(int n, const double* __restrict__ p, const double* __restrict__ q,
                                                    double* __restrict__ x, double* __restrict__ r,
                                                    float* __restrict__ r32, Reducer red, PcgScalars* sc) {
+    dep_wait();
     const double alpha = sc->alpha;
     double rr = 0.0;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        x[i] = fma(alpha, p[i], x[i]);
-        const double ri = fma(-alpha, q[i], r[i]);
+        x[i] = fma(alpha, ldv(p + i), x[i]);
+        const double ri = fma(-alpha, ldv(q + i), r[i]);
         r[i] = ri;
-        if (r32) r32[i] = (float)ri;
+        if (r32) r32[i] = d2f(ri);
         rr = fma(ri, ri, rr);
     }
     reduce_and_finish<1>(rr, 0.0, red, sc, FIN_RR);
-}
-
-// p = z + beta p.
-__global__ void __launch_bounds__(TPB) k_update_p(int n, const double* __restrict__ z, double* __restrict__ p,
-                                                  const PcgScalars* sc) {
-    const double beta = sc->beta;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) p[i] = fma(beta, p[i], z[i]);
 }
 
 // ------------------------------------------------------------ host ---------
@@ -899,13 +1035,13 @@ void coarse_solve_launch(amg_hierarchy* h, const void* b, void* x, bool fp32_in,
         const int grid = blocks_for((long long)n * 32, 256, h->num_sms * 8);
         Scope sc_(&h->prof, h->stream, K_COARSE, 16.0 * n);
         if (!fp32_in)
-            k_coarse_solve_seg<double, double><<<grid, 256, 0, h->stream>>>(n, m, h->segL_ptr, h->segL_blk,
+            launch_dep(k_coarse_solve_seg<double, double>, grid, 256, 0, h->stream, n, m, h->segL_ptr, h->segL_blk,
                                                                             h->coarse_inv, (const double*)b, (double*)x);
         else if (fp64_out)
-            k_coarse_solve_seg<float, double><<<grid, 256, 0, h->stream>>>(n, m, h->segL_ptr, h->segL_blk,
+            launch_dep(k_coarse_solve_seg<float, double>, grid, 256, 0, h->stream, n, m, h->segL_ptr, h->segL_blk,
                                                                            h->coarse_inv, (const float*)b, (double*)x);
         else
-            k_coarse_solve_seg<float, float><<<grid, 256, 0, h->stream>>>(n, m, h->segL_ptr, h->segL_blk,
+            launch_dep(k_coarse_solve_seg<float, float>, grid, 256, 0, h->stream, n, m, h->segL_ptr, h->segL_blk,
                                                                           h->coarse_inv, (const float*)b, (float*)x);
         KERNEL_CHECK();
         return;
@@ -942,17 +1078,19 @@ void coarse_solve_launch(amg_hierarchy* h, const void* b, void* x, bool fp32_in,
     const size_t sh = sizeof(double) * (size_t)n;
     Scope sc_(&h->prof, h->stream, K_COARSE, by_coarse(n, fp32_in ? 4 : 8, fp64_out ? 8 : 4));
     if (!fp32_in)
-        k_coarse_solve<double, double><<<grid, threads, sh, h->stream>>>(n, h->coarse_inv, (const double*)b, (double*)x);
+        launch_dep(k_coarse_solve<double, double>, grid, threads, sh, h->stream, n, h->coarse_inv, (const double*)b, (double*)x);
     else if (fp64_out)
-        k_coarse_solve<float, double><<<grid, threads, sh, h->stream>>>(n, h->coarse_inv, (const float*)b, (double*)x);
+        launch_dep(k_coarse_solve<float, double>, grid, threads, sh, h->stream, n, h->coarse_inv, (const float*)b, (double*)x);
     else
-        k_coarse_solve<float, float><<<grid, threads, sh, h->stream>>>(n, h->coarse_inv, (const float*)b, (float*)x);
+        launch_dep(k_coarse_solve<float, float>, grid, threads, sh, h->stream, n, h->coarse_inv, (const float*)b, (float*)x);
     KERNEL_CHECK();
 }
 
-// z = B r on level 0. With rz_mode != FIN_NONE, also finishes r . z.
-template <typename T>
-void vcycle_typed(amg_hierarchy* h, const double* r, double* z, int rz_mode) {
+// z = B r on level 0, z in the V-cycle's type or FP64. With rz_mode !=
+// FIN_NONE, also finishes r . z. A single level (the coarsest solve alone) has
+// an FP64 z.
+template <typename T, typename TZ>
+void vcycle_typed(amg_hierarchy* h, const double* r, TZ* z, int rz_mode) {
     cudaStream_t st = h->stream;
     const double* q2 = rz_mode == FIN_RHO_UPDATE_FCG ? h->q : nullptr;
     const int L = (int)h->lev.size() - 1;
@@ -962,8 +1100,8 @@ void vcycle_typed(amg_hierarchy* h, const double* r, double* z, int rz_mode) {
     if (L == 0) {
         coarse_solve_launch(h, r, z, false, true);
         if (rz_mode != FIN_NONE) {
-            Scope sc_(&h->prof, st, K_DOT, 16.0 * n0);
-            k_dot<<<red_grid_rows(h, n0), TPB, 0, st>>>(n0, r, z, q2, h->red, h->sc, rz_mode);
+            Scope sc_(&h->prof, st, K_DOT, (8.0 + sizeof(TZ)) * n0);
+            launch_dep(k_dot<TZ>, red_grid_rows(h, n0), TPB, 0, st, n0, r, z, q2, h->red, h->sc, rz_mode);
             KERNEL_CHECK();
         }
         return;
@@ -999,7 +1137,7 @@ void vcycle_typed(amg_hierarchy* h, const double* r, double* z, int rz_mode) {
         const int Vb = l == 0 ? 8 : V;
         if (l == 0 && f32 && !h->r32_ready) {           // else the CG update already wrote it
             Scope sc_(&h->prof, st, K_CONVERT, 12.0 * Lv.A.n);
-            k_to_f32<<<vec_grid(h, Lv.A.n), TPB, 0, st>>>(Lv.A.n, r, (float*)vec(Lv, VB));
+            launch_dep(k_to_f32, vec_grid(h, Lv.A.n), TPB, 0, st, Lv.A.n, r, (float*)vec(Lv, VB));
             KERNEL_CHECK();
         }
         const bool wideA = SA && !f32 && wide(Lv.A, WIDE_MIN_A);       // dense coarse level of a smoothed hierarchy
@@ -1011,35 +1149,35 @@ void vcycle_typed(amg_hierarchy* h, const double* r, double* z, int rz_mode) {
         if (wideA) {
             Scope sc_(&h->prof, st, l == 0 ? K_PRE_L0 : K_PRE, by_pre(Lv, V, l == 0 ? 8 : V));
             const double* bl = l == 0 ? r : (const double*)vec(Lv, VB);
-            k_wide<W_PRE><<<wide_grid(h, Lv.A.n), TPB, 0, st>>>(Lv.A.n, Lv.A.ptr, Lv.A.col, Lv.A.val, bl, Lv.minv,
+            launch_dep(k_wide<W_PRE>, wide_grid(h, Lv.A.n), TPB, 0, st, Lv.A.n, Lv.A.ptr, Lv.A.col, Lv.A.val, bl, Lv.minv,
                                                                 Lv.wminv, (double)omega, bl, (double*)ra,
                                                                 (double*)xa);
             KERNEL_CHECK();
         } else {
             Scope sc_(&h->prof, st, l == 0 ? K_PRE_L0 : K_PRE, by_pre(Lv, V, l == 0 && !f32 ? 8 : V));
-            if (l == 0 && !f32) launch_pre<T, double>(U || more, g, st, S, valm(Lv), wm(Lv), omega, r, xa, ra);
-            else launch_pre<T, T>(U || more, g, st, S, valm(Lv), wm(Lv), omega, vec(Lv, VB), xa, ra);
+            if (l == 0 && !f32) launch_pre<T, double>(h, U || more, g, st, S, valm(Lv), wm(Lv), omega, r, xa, ra);
+            else launch_pre<T, T>(h, U || more, g, st, S, valm(Lv), wm(Lv), omega, vec(Lv, VB), xa, ra);
         }
         // the dense-level path stored x_1: it takes one sweep more here
         for (int k = wideA ? 1 : 2; k < pre; ++k) {
             Scope sc_(&h->prof, st, K_PRE_STEP, by_smooth(Lv, V, Vb, V));
             if (wideA)
-                k_wide<W_SMOOTH><<<wide_grid(h, Lv.A.n), TPB, 0, st>>>(
+                launch_dep(k_wide<W_SMOOTH>, wide_grid(h, Lv.A.n), TPB, 0, st, 
                     Lv.A.n, Lv.A.ptr, Lv.A.col, Lv.A.val, (const double*)xa, Lv.minv, nullptr, (double)omega,
                     l == 0 ? r : (const double*)vec(Lv, VB), (double*)xb, nullptr);
-            else if (l == 0) k_smooth<T, double, T><<<g, TPB, 0, st>>>(S, val(Lv), minv(Lv), omega, r, xa, xb);
-            else k_smooth<T, T, T><<<g, TPB, 0, st>>>(S, val(Lv), minv(Lv), omega, vec(Lv, VB), xa, xb);
+            else if (l == 0) SELL_DISPATCH(h, S, launch_sell<RB>(k_smooth<RB, T, double, T>, g, st, S, val(Lv), minv(Lv), omega, r, xa, xb));
+            else SELL_DISPATCH(h, S, launch_sell<RB>(k_smooth<RB, T, T, T>, g, st, S, val(Lv), minv(Lv), omega, vec(Lv, VB), xa, xb));
             KERNEL_CHECK();
             std::swap(xa, xb);
         }
         if (more) {
             Scope sc_(&h->prof, st, K_PRE_STEP, by_resid(Lv, V, Vb));
             if (wideA)
-                k_wide<W_RES><<<wide_grid(h, Lv.A.n), TPB, 0, st>>>(
+                launch_dep(k_wide<W_RES>, wide_grid(h, Lv.A.n), TPB, 0, st, 
                     Lv.A.n, Lv.A.ptr, Lv.A.col, Lv.A.val, (const double*)xa, nullptr, nullptr, 0.0,
                     l == 0 ? r : (const double*)vec(Lv, VB), (double*)ra, nullptr);
-            else if (l == 0) k_resid<T, double><<<g, TPB, 0, st>>>(S, val(Lv), r, xa, ra);
-            else k_resid<T, T><<<g, TPB, 0, st>>>(S, val(Lv), vec(Lv, VB), xa, ra);
+            else if (l == 0) SELL_DISPATCH(h, S, launch_sell<RB>(k_resid<RB, T, double>, g, st, S, val(Lv), r, xa, ra));
+            else SELL_DISPATCH(h, S, launch_sell<RB>(k_resid<RB, T, T>, g, st, S, val(Lv), vec(Lv, VB), xa, ra));
             KERNEL_CHECK();
         }
         xcur[l] = xa;
@@ -1050,17 +1188,17 @@ void vcycle_typed(amg_hierarchy* h, const double* r, double* z, int rz_mode) {
             const SellView SPT{Lv.PBT.n, Lv.PBT.nslices, Lv.PBT.sptr, Lv.PBT.col, Lv.PBT.perm};
             Scope sc_(&h->prof, st, K_RESTRICT, (double)Lv.pbar_t.nnz * (V + 4) + (double)(Lv.A.n + nc) * V);
             if (!f32 && wide(Lv.pbar_t, WIDE_MIN_P))
-                k_wide<W_SPMV><<<wide_grid(h, nc), TPB, 0, st>>>(nc, Lv.pbar_t.ptr, Lv.pbar_t.col, Lv.pbar_t.val,
+                launch_dep(k_wide<W_SPMV>, wide_grid(h, nc), TPB, 0, st, nc, Lv.pbar_t.ptr, Lv.pbar_t.col, Lv.pbar_t.val,
                                                                  (const double*)ra, nullptr, nullptr, 0.0, nullptr,
                                                                  (double*)vec(h->lev[l + 1], VB), nullptr);
             else
-                k_sell_spmv<T><<<sell_grid(h, SPT.nslices), TPB, 0, st>>>(
-                    SPT, f32 ? (const T*)Lv.PBT.val32 : (const T*)Lv.PBT.val, ra, vec(h->lev[l + 1], VB));
+                SELL_DISPATCH(h, SPT, launch_sell<RB>(k_sell_spmv<RB, T>, sell_grid(h, SPT.nslices), st, 
+                    SPT, f32 ? (const T*)Lv.PBT.val32 : (const T*)Lv.PBT.val, ra, vec(h->lev[l + 1], VB)));
             KERNEL_CHECK();
             continue;
         }
         Scope sc_(&h->prof, st, K_RESTRICT, by_restrict(Lv.A.n, nc, V));
-        k_restrict<T><<<Lv.grid_restrict[f32] ? Lv.grid_restrict[f32] : vec_grid(h, nc), TPB, 0, st>>>(
+        launch_dep(k_restrict<T>, Lv.grid_restrict[f32] ? Lv.grid_restrict[f32] : vec_grid(h, nc), TPB, 0, st, 
             nc, Lv.pt_ptr, Lv.pt_idx, pv(Lv), ra, vec(h->lev[l + 1], VB));
         KERNEL_CHECK();
     }
@@ -1082,13 +1220,13 @@ void vcycle_typed(amg_hierarchy* h, const double* r, double* z, int rz_mode) {
                 Scope sc_(&h->prof, st, l == 0 ? K_POST_L0 : K_POST,
                           (double)Lv.pbar.nnz * (V + 4) + 2.0 * Lv.A.n * V + (double)nc * V);
                 if (!f32 && wide(Lv.pbar, WIDE_MIN_P))
-                    k_wide<W_ADD><<<wide_grid(h, Lv.A.n), TPB, 0, st>>>(Lv.A.n, Lv.pbar.ptr, Lv.pbar.col,
+                    launch_dep(k_wide<W_ADD>, wide_grid(h, Lv.A.n), TPB, 0, st, Lv.A.n, Lv.pbar.ptr, Lv.pbar.col,
                                                                        Lv.pbar.val, (const double*)e, nullptr,
                                                                        nullptr, 0.0, nullptr, (double*)xcur[l],
                                                                        nullptr);
                 else
-                    k_prolong<T><<<sell_grid(h, SPB.nslices), TPB, 0, st>>>(
-                        SPB, f32 ? (const T*)Lv.PB.val32 : (const T*)Lv.PB.val, e, xcur[l]);
+                    SELL_DISPATCH(h, SPB, launch_sell<RB>(k_prolong<RB, T>, sell_grid(h, SPB.nslices), st, 
+                        SPB, f32 ? (const T*)Lv.PB.val32 : (const T*)Lv.PB.val, e, xcur[l]));
                 KERNEL_CHECK();
             }
             // post sweeps alternate between y and the x buffer the pre-smoother left free
@@ -1099,11 +1237,11 @@ void vcycle_typed(amg_hierarchy* h, const double* r, double* z, int rz_mode) {
                     T* dst = bufs[k & 1];
                     Scope sc_(&h->prof, st, K_SMOOTH, by_smooth(Lv, V, V, V));
                     if (!f32 && wide(Lv.A, WIDE_MIN_A))
-                        k_wide<W_SMOOTH><<<wide_grid(h, Lv.A.n), TPB, 0, st>>>(
+                        launch_dep(k_wide<W_SMOOTH>, wide_grid(h, Lv.A.n), TPB, 0, st, 
                             Lv.A.n, Lv.A.ptr, Lv.A.col, Lv.A.val, (const double*)cur, Lv.minv, nullptr,
                             (double)omega, (const double*)vec(Lv, VB), (double*)dst, nullptr);
                     else
-                        k_smooth<T, T, T><<<g, TPB, 0, st>>>(S, val(Lv), minv(Lv), omega, vec(Lv, VB), cur, dst);
+                        SELL_DISPATCH(h, S, launch_sell<RB>(k_smooth<RB, T, T, T>, g, st, S, val(Lv), minv(Lv), omega, vec(Lv, VB), cur, dst));
                     KERNEL_CHECK();
                     cur = dst;
                 }
@@ -1113,18 +1251,18 @@ void vcycle_typed(amg_hierarchy* h, const double* r, double* z, int rz_mode) {
             for (int k = 0; k + 1 < post; ++k) {
                 T* dst = bufs[k & 1];
                 Scope sc_(&h->prof, st, K_SMOOTH, by_smooth(Lv, V, 8, V));
-                k_smooth<T, double, T><<<g, TPB, 0, st>>>(S, val(Lv), minv(Lv), omega, r, cur, dst);
+                SELL_DISPATCH(h, S, launch_sell<RB>(k_smooth<RB, T, double, T>, g, st, S, val(Lv), minv(Lv), omega, r, cur, dst));
                 KERNEL_CHECK();
                 cur = dst;
             }
             {
-                Scope sc_(&h->prof, st, K_SMOOTH, by_smooth(Lv, V, 8, 8));
-                k_smooth<T, double, double><<<g, TPB, 0, st>>>(S, val(Lv), minv(Lv), omega, r, cur, z);
+                Scope sc_(&h->prof, st, K_SMOOTH, by_smooth(Lv, V, 8, sizeof(TZ)));
+                SELL_DISPATCH(h, S, launch_sell<RB>(k_smooth<RB, T, double, TZ>, g, st, S, val(Lv), minv(Lv), omega, r, cur, z));
                 KERNEL_CHECK();
             }
             if (rz_mode != FIN_NONE) {
-                Scope sc_(&h->prof, st, K_DOT, 16.0 * n0);
-                k_dot<<<red_grid_rows(h, n0), TPB, 0, st>>>(n0, r, z, q2, h->red, h->sc, rz_mode);
+                Scope sc_(&h->prof, st, K_DOT, (8.0 + sizeof(TZ)) * n0);
+                launch_dep(k_dot<TZ>, red_grid_rows(h, n0), TPB, 0, st, n0, r, z, q2, h->red, h->sc, rz_mode);
                 KERNEL_CHECK();
             }
             continue;
@@ -1133,12 +1271,12 @@ void vcycle_typed(amg_hierarchy* h, const double* r, double* z, int rz_mode) {
             T *ya = vec(Lv, VY), *yb = spare[l];
             {
                 Scope sc_(&h->prof, st, K_POST, by_post2(Lv, nc, V, V, false, U));
-                launch_post<T, T, T, false>(U, g, st, SAP, apv(Lv), wm(Lv), Lv.agg, pv(Lv), e, xcur[l], rcur[l],
+                launch_post<T, T, T, false>(h, U, g, st, SAP, apv(Lv), wm(Lv), Lv.agg, pv(Lv), e, xcur[l], rcur[l],
                                             (const T*)nullptr, ya, h->red, h->sc, FIN_NONE, nullptr);
             }
             for (int k = 1; k < post; ++k) {
                 Scope sc_(&h->prof, st, K_SMOOTH, by_smooth(Lv, V, V, V));
-                k_smooth<T, T, T><<<g, TPB, 0, st>>>(S, val(Lv), minv(Lv), omega, vec(Lv, VB), ya, yb);
+                SELL_DISPATCH(h, S, launch_sell<RB>(k_smooth<RB, T, T, T>, g, st, S, val(Lv), minv(Lv), omega, vec(Lv, VB), ya, yb));
                 KERNEL_CHECK();
                 std::swap(ya, yb);
             }
@@ -1146,34 +1284,34 @@ void vcycle_typed(amg_hierarchy* h, const double* r, double* z, int rz_mode) {
             continue;
         }
         if (post == 1) {
-            Scope sc_(&h->prof, st, K_POST_L0, by_post2(Lv, nc, V, 8, rz_mode != FIN_NONE, U));
+            Scope sc_(&h->prof, st, K_POST_L0, by_post2(Lv, nc, V, sizeof(TZ), rz_mode != FIN_NONE, U));
             if (rz_mode != FIN_NONE)
-                launch_post<T, double, double, true>(U, red_grid(h, SAP.nslices), st, SAP, apv(Lv), wm(Lv), Lv.agg, pv(Lv), e,
+                launch_post<T, double, TZ, true>(h, U, red_grid(h, SAP.nslices), st, SAP, apv(Lv), wm(Lv), Lv.agg, pv(Lv), e,
                                                      xcur[0], rcur[0], r, z, h->red, h->sc, rz_mode, q2);
             else
-                launch_post<T, double, double, false>(U, g, st, SAP, apv(Lv), wm(Lv), Lv.agg, pv(Lv), e, xcur[0],
-                                                      rcur[0], r, z, h->red, h->sc, FIN_NONE, nullptr);
+                launch_post<T, double, TZ, false>(h, U, g, st, SAP, apv(Lv), wm(Lv), Lv.agg, pv(Lv), e, xcur[0],
+                                                  rcur[0], r, z, h->red, h->sc, FIN_NONE, nullptr);
         } else {
             T *ya = vec(Lv, VY), *yb = spare[0];
             {
                 Scope sc_(&h->prof, st, K_POST_L0, by_post2(Lv, nc, V, V, false, U));
-                launch_post<T, double, T, false>(U, g, st, SAP, apv(Lv), wm(Lv), Lv.agg, pv(Lv), e, xcur[0], rcur[0],
+                launch_post<T, double, T, false>(h, U, g, st, SAP, apv(Lv), wm(Lv), Lv.agg, pv(Lv), e, xcur[0], rcur[0],
                                                  r, ya, h->red, h->sc, FIN_NONE, nullptr);
             }
             for (int k = 1; k < post - 1; ++k) {
                 Scope sc_(&h->prof, st, K_SMOOTH, by_smooth(Lv, V, 8, V));
-                k_smooth<T, double, T><<<g, TPB, 0, st>>>(S, val(Lv), minv(Lv), omega, r, ya, yb);
+                SELL_DISPATCH(h, S, launch_sell<RB>(k_smooth<RB, T, double, T>, g, st, S, val(Lv), minv(Lv), omega, r, ya, yb));
                 KERNEL_CHECK();
                 std::swap(ya, yb);
             }
             {
-                Scope sc_(&h->prof, st, K_SMOOTH, by_smooth(Lv, V, 8, 8));
-                k_smooth<T, double, double><<<g, TPB, 0, st>>>(S, val(Lv), minv(Lv), omega, r, ya, z);
+                Scope sc_(&h->prof, st, K_SMOOTH, by_smooth(Lv, V, 8, sizeof(TZ)));
+                SELL_DISPATCH(h, S, launch_sell<RB>(k_smooth<RB, T, double, TZ>, g, st, S, val(Lv), minv(Lv), omega, r, ya, z));
                 KERNEL_CHECK();
             }
             if (rz_mode != FIN_NONE) {
-                Scope sc_(&h->prof, st, K_DOT, 16.0 * n0);
-                k_dot<<<red_grid_rows(h, n0), TPB, 0, st>>>(n0, r, z, q2, h->red, h->sc, rz_mode);
+                Scope sc_(&h->prof, st, K_DOT, (8.0 + sizeof(TZ)) * n0);
+                launch_dep(k_dot<TZ>, red_grid_rows(h, n0), TPB, 0, st, n0, r, z, q2, h->red, h->sc, rz_mode);
                 KERNEL_CHECK();
             }
         }
@@ -1231,12 +1369,12 @@ void kc_apply(amg_hierarchy* h, int l, const T* in, T* out) {
     T* ra = lvec<T>(Lv, 2);
     {
         Scope sc_(&h->prof, st, K_PRE, by_pre(Lv, V, V));
-        launch_pre<T, T>(true, Lv.grid_pre[f32] ? Lv.grid_pre[f32] : sell_grid(h, S.nslices), st, S, O.valm(), O.wm(),
+        launch_pre<T, T>(h, true, Lv.grid_pre[f32] ? Lv.grid_pre[f32] : sell_grid(h, S.nslices), st, S, O.valm(), O.wm(),
                          omega, in, xa, ra);
     }
     {
         Scope sc_(&h->prof, st, K_RESTRICT, by_restrict(Lv.A.n, nc, V));
-        k_restrict<T><<<Lv.grid_restrict[f32] ? Lv.grid_restrict[f32] : vec_grid(h, nc), TPB, 0, st>>>(
+        launch_dep(k_restrict<T>, Lv.grid_restrict[f32] ? Lv.grid_restrict[f32] : vec_grid(h, nc), TPB, 0, st, 
             nc, Lv.pt_ptr, Lv.pt_idx, O.p(), ra, lvec<T>(Ln, 0));
         KERNEL_CHECK();
     }
@@ -1254,7 +1392,7 @@ void kc_apply(amg_hierarchy* h, int l, const T* in, T* out) {
         kc_apply<T>(h, l + 1, lvec<T>(Ln, 0), e);
     }
     Scope sc_(&h->prof, st, K_POST, by_post2(Lv, nc, V, V, false, true));
-    launch_post<T, T, T, false>(true, Lv.grid_post[f32] ? Lv.grid_post[f32] : sell_grid(h, S.nslices), st, SAP, O.apw(),
+    launch_post<T, T, T, false>(h, true, Lv.grid_post[f32] ? Lv.grid_post[f32] : sell_grid(h, S.nslices), st, SAP, O.apw(),
                                 O.wm(), Lv.agg, O.p(), e, xa, ra, (const T*)nullptr, out, h->red, h->sc, FIN_NONE,
                                 nullptr);
 }
@@ -1272,39 +1410,39 @@ void kc_fcg2(amg_hierarchy* h, int m, const T* b, T* e) {
     kc_apply<T>(h, m, b, d1);
     {
         Scope sc_(&h->prof, st, K_KFCG, by_spmv);
-        k_kc_spmv_dot<T><<<red_grid(h, S.nslices), TPB, 0, st>>>(S, O.val(), d1, q1, b, h->red, ks);
+        SELL_DISPATCH(h, S, launch_sell<RB>(k_kc_spmv_dot<RB, T>, red_grid(h, S.nslices), st, S, O.val(), d1, q1, b, h->red, ks));
         KERNEL_CHECK();
     }
     {
         Scope sc_(&h->prof, st, K_KFCG, 5.0 * n * V);
-        k_kc_update1<T><<<vec_grid(h, n), TPB, 0, st>>>(n, d1, q1, b, e, r2, ks);
+        launch_dep(k_kc_update1<T>, vec_grid(h, n), TPB, 0, st, n, d1, q1, b, e, r2, ks);
         KERNEL_CHECK();
     }
     kc_apply<T>(h, m, r2, z2);
     {
         Scope sc_(&h->prof, st, K_KFCG, 2.0 * n * V);
-        k_kc_dot<T><<<red_grid_rows(h, n), TPB, 0, st>>>(n, z2, q1, h->red, ks);
+        launch_dep(k_kc_dot<T>, red_grid_rows(h, n), TPB, 0, st, n, z2, q1, h->red, ks);
         KERNEL_CHECK();
     }
     {
         Scope sc_(&h->prof, st, K_KFCG, (double)Lm.A.nnz * (V + 4) + (double)n * 5 * V);
-        k_kc_spmv2<T><<<red_grid(h, S.nslices), TPB, 0, st>>>(S, O.val(), z2, q1, d1, r2, d2, h->red, ks);
+        SELL_DISPATCH(h, S, launch_sell<RB>(k_kc_spmv2<RB, T>, red_grid(h, S.nslices), st, S, O.val(), z2, q1, d1, r2, d2, h->red, ks));
         KERNEL_CHECK();
     }
     {
         Scope sc_(&h->prof, st, K_KFCG, 3.0 * n * V);
-        k_kc_update2<T><<<vec_grid(h, n), TPB, 0, st>>>(n, d2, e, ks);
+        launch_dep(k_kc_update2<T>, vec_grid(h, n), TPB, 0, st, n, d2, e, ks);
         KERNEL_CHECK();
     }
 }
 
 // z = B r with the K-cycle on level 0 (FP64 r and z; with rz_mode the r.z
 // (and q.z) sums of the outer CG are finished as in the V-cycle).
-template <typename T>
-void kcycle_typed(amg_hierarchy* h, const double* r, double* z, int rz_mode) {
+template <typename T, typename TZ>
+void kcycle_typed(amg_hierarchy* h, const double* r, TZ* z, int rz_mode) {
     const int L = (int)h->lev.size() - 1;
     if (L <= 1) {                          // no intermediate level: the K-cycle is the V-cycle
-        vcycle_typed<T>(h, r, z, rz_mode);
+        vcycle_typed<T, TZ>(h, r, z, rz_mode);
         return;
     }
     cudaStream_t st = h->stream;
@@ -1322,41 +1460,44 @@ void kcycle_typed(amg_hierarchy* h, const double* r, double* z, int rz_mode) {
     const int g = L0.grid_pre[f32] ? L0.grid_pre[f32] : sell_grid(h, S.nslices);
     if (f32 && !h->r32_ready) {                         // else the CG update already wrote it
         Scope sc_(&h->prof, st, K_CONVERT, 12.0 * n0);
-        k_to_f32<<<vec_grid(h, n0), TPB, 0, st>>>(n0, r, (float*)lvec<T>(L0, 0));
+        launch_dep(k_to_f32, vec_grid(h, n0), TPB, 0, st, n0, r, (float*)lvec<T>(L0, 0));
         KERNEL_CHECK();
     }
     {
         Scope sc_(&h->prof, st, K_PRE_L0, by_pre(L0, V, f32 ? V : 8));
-        if (f32) launch_pre<T, T>(true, g, st, S, O.valm(), O.wm(), omega, lvec<T>(L0, 0), xa, ra);
-        else launch_pre<T, double>(true, g, st, S, O.valm(), O.wm(), omega, r, xa, ra);
+        if (f32) launch_pre<T, T>(h, true, g, st, S, O.valm(), O.wm(), omega, lvec<T>(L0, 0), xa, ra);
+        else launch_pre<T, double>(h, true, g, st, S, O.valm(), O.wm(), omega, r, xa, ra);
     }
     {
         Scope sc_(&h->prof, st, K_RESTRICT, by_restrict(n0, nc, V));
-        k_restrict<T><<<L0.grid_restrict[f32] ? L0.grid_restrict[f32] : vec_grid(h, nc), TPB, 0, st>>>(
+        launch_dep(k_restrict<T>, L0.grid_restrict[f32] ? L0.grid_restrict[f32] : vec_grid(h, nc), TPB, 0, st, 
             nc, L0.pt_ptr, L0.pt_idx, O.p(), ra, lvec<T>(L1, 0));
         KERNEL_CHECK();
     }
     T* e = LevelOps<T>(L1).kv(5);
     kc_fcg2<T>(h, 1, lvec<T>(L1, 0), e);
-    Scope sc_(&h->prof, st, K_POST_L0, by_post2(L0, nc, V, 8, rz_mode != FIN_NONE, true));
+    Scope sc_(&h->prof, st, K_POST_L0, by_post2(L0, nc, V, sizeof(TZ), rz_mode != FIN_NONE, true));
     const int gp = L0.grid_post[f32] ? L0.grid_post[f32] : sell_grid(h, S.nslices);
     if (rz_mode != FIN_NONE)
-        launch_post<T, double, double, true>(true, red_grid(h, SAP.nslices), st, SAP, O.apw(), O.wm(), L0.agg, O.p(), e, xa, ra, r, z,
-                                             h->red, h->sc, rz_mode, q2);
+        launch_post<T, double, TZ, true>(h, true, red_grid(h, SAP.nslices), st, SAP, O.apw(), O.wm(), L0.agg, O.p(), e, xa,
+                                         ra, r, z, h->red, h->sc, rz_mode, q2);
     else
-        launch_post<T, double, double, false>(true, gp, st, SAP, O.apw(), O.wm(), L0.agg, O.p(), e, xa, ra, r, z,
-                                              h->red, h->sc, FIN_NONE, nullptr);
+        launch_post<T, double, TZ, false>(h, true, gp, st, SAP, O.apw(), O.wm(), L0.agg, O.p(), e, xa, ra, r, z, h->red, h->sc, FIN_NONE, nullptr);
 }
 
-void vcycle_dispatch(amg_hierarchy* h, const double* r, double* z, int rz_mode) {
-    const bool f32 = h->opt.precision == AMG_FP32_VCYCLE;
-    if (h->opt.cycle > 0) {
-        if (f32) kcycle_typed<float>(h, r, z, rz_mode);
-        else kcycle_typed<double>(h, r, z, rz_mode);
-    } else {
-        if (f32) vcycle_typed<float>(h, r, z, rz_mode);
-        else vcycle_typed<double>(h, r, z, rz_mode);
-    }
+template <typename T, typename TZ>
+void cycle_typed(amg_hierarchy* h, const double* r, TZ* z, int rz_mode) {
+    if (h->opt.cycle > 0) kcycle_typed<T, TZ>(h, r, z, rz_mode);
+    else vcycle_typed<T, TZ>(h, r, z, rz_mode);
+}
+
+// The CG's own z = B r stays in the FP32 V-cycle's type.
+bool float_z(const amg_hierarchy* h) { return h->opt.precision == AMG_FP32_VCYCLE && h->lev.size() > 1; }
+
+void cg_precondition(amg_hierarchy* h, int rz_mode) {
+    if (float_z(h)) cycle_typed<float, float>(h, h->r, reinterpret_cast<float*>(h->z), rz_mode);
+    else if (h->opt.precision == AMG_FP32_VCYCLE) cycle_typed<float, double>(h, h->r, h->z, rz_mode);
+    else cycle_typed<double, double>(h, h->r, h->z, rz_mode);
 }
 
 // Launch-shape candidates of a grid-stride kernel that needs at most `need`
@@ -1434,24 +1575,24 @@ void autotune_levels(amg_hierarchy* h) {
         Lv.grid_pre[f32] = tune_grid(h, tune_key(z0 ? "pre0" : "pre", V, S.n, Lv.A.nnz, S.nslices, 1, h->num_sms),
                                      cand, [&](int g) {
                                          if (z0 && !f32)
-                                             launch_pre<T, double>(U, g, st, S, valm, wm, omega, h->r, vx(Lv), vr(Lv));
+                                             launch_pre<T, double>(h, U, g, st, S, valm, wm, omega, h->r, vx(Lv), vr(Lv));
                                          else
-                                             launch_pre<T, T>(U, g, st, S, valm, wm, omega, vb(Lv), vx(Lv), vr(Lv));
+                                             launch_pre<T, T>(h, U, g, st, S, valm, wm, omega, vb(Lv), vx(Lv), vr(Lv));
                                      });
         if (h->opt.smooth_p) continue;     // the smoothed path has no fused post-smoother or member lists
         Lv.grid_post[f32] = tune_grid(
             h, tune_key(z0 ? "post0" : "post", V, SAP.n, Lv.ap_nnz, SAP.nslices, 1, h->num_sms), cand, [&](int g) {
                 if (z0)
-                    launch_post<T, double, double, false>(U, g, st, SAP, apv, wm, Lv.agg, p, vx(Ln), vx(Lv), vr(Lv),
-                                                          h->r, h->z, h->red, h->sc, FIN_NONE, nullptr);
+                    launch_post<T, double, T, false>(h, U, g, st, SAP, apv, wm, Lv.agg, p, vx(Ln), vx(Lv), vr(Lv), h->r,
+                                                     reinterpret_cast<T*>(h->z), h->red, h->sc, FIN_NONE, nullptr);
                 else
-                    launch_post<T, T, T, false>(U, g, st, SAP, apv, wm, Lv.agg, p, vx(Ln), vx(Lv), vr(Lv),
+                    launch_post<T, T, T, false>(h, U, g, st, SAP, apv, wm, Lv.agg, p, vx(Ln), vx(Lv), vr(Lv),
                                                 (const T*)nullptr, vy(Lv), h->red, h->sc, FIN_NONE, nullptr);
             });
         const int nc = Ln.A.n;
         Lv.grid_restrict[f32] = tune_grid(h, tune_key("restrict", V, nc, Lv.A.n, 0, 1, h->num_sms),
                                           grid_candidates(h, (nc + TPB - 1) / TPB), [&](int g) {
-                                              k_restrict<T><<<g, TPB, 0, st>>>(nc, Lv.pt_ptr, Lv.pt_idx, p, vr(Lv),
+                                              launch_dep(k_restrict<T>, g, TPB, 0, st, nc, Lv.pt_ptr, Lv.pt_idx, p, vr(Lv),
                                                                                vb(Ln));
                                               KERNEL_CHECK();
                                           });
@@ -1540,10 +1681,13 @@ void autotune_vcycle(amg_hierarchy* h) {
 
 void coarse_cg_solve(amg_hierarchy* h, const double* b, double* x) { coarse_solve_launch(h, b, x, false, true); }
 
-void vcycle_plain(amg_hierarchy* h, const double* r, double* z) { vcycle_dispatch(h, r, z, FIN_NONE); }
+void vcycle_plain(amg_hierarchy* h, const double* r, double* z) {
+    if (h->opt.precision == AMG_FP32_VCYCLE) cycle_typed<float, double>(h, r, z, FIN_NONE);
+    else cycle_typed<double, double>(h, r, z, FIN_NONE);
+}
 
 void vcycle_apply(amg_hierarchy* h, const double* r, double* z) {
-    vcycle_dispatch(h, r, z, FIN_NONE);
+    vcycle_plain(h, r, z);
     CUDA_CHECK(cudaStreamSynchronize(h->stream));
     h->prof.flush();
 }
@@ -1558,11 +1702,12 @@ amg_status solve(amg_hierarchy* h, const double* b, double* x, double rtol, int 
     PcgScalars* hs = h->sc_host;
 
     const double nnz = (double)L0.A.nnz;
-    const double by_res = 12.0 * nnz + 24.0 * n, by_spmv = 12.0 * nnz + 16.0 * n;
+    const double by_res = 12.0 * nnz + 24.0 * n;
+    const bool zf = float_z(h);
     CUDA_CHECK(cudaMemsetAsync(h->sc, 0, sizeof(PcgScalars), st));
     {
         Scope sc_(&h->prof, st, K_RESIDUAL, by_res);
-        k_residual<<<red_grid(h, S.nslices), TPB, 0, st>>>(S, A, x, b, h->r, h->red, h->sc);
+        SELL_DISPATCH(h, S, launch_sell<RB>(k_residual<RB>, red_grid(h, S.nslices), st, S, A, x, b, h->r, h->red, h->sc));
         KERNEL_CHECK();
     }
     read_scalars(h);
@@ -1589,37 +1734,46 @@ amg_status solve(amg_hierarchy* h, const double* b, double* x, double rtol, int 
         ~Ev() { if (e) cudaEventDestroy(e); }
     } ev;
     CUDA_CHECK(cudaEventCreateWithFlags(&ev.e, cudaEventDisableTiming));
-    // z = B r for the next iteration, then p = z + beta p
+    // z = B r and beta for the next iteration
     auto precondition = [&]() {
         h->r32_ready = r32 != nullptr;                  // level 0's float r is the one k_update_xr wrote
-        vcycle_dispatch(h, h->r, h->z,
-                        h->opt.krylov == 1 || h->opt.cycle > 0 ? FIN_RHO_UPDATE_FCG : FIN_RHO_UPDATE);
+        cg_precondition(h, h->opt.krylov == 1 || h->opt.cycle > 0 ? FIN_RHO_UPDATE_FCG : FIN_RHO_UPDATE);
         h->r32_ready = false;
-        Scope sc_(&h->prof, st, K_UPDATE_P, 24.0 * n);
-        k_update_p<<<vec_grid(h, n), TPB, 0, st>>>(n, h->z, h->p, h->sc);
-        KERNEL_CHECK();
     };
     if (rel <= rtol) status = AMG_OK;
     while (status != AMG_OK && it < maxit) {
         if (restart) {
-            vcycle_dispatch(h, h->r, h->z, FIN_RHO_INIT);
-            CUDA_CHECK(cudaMemcpyAsync(h->p, h->z, sizeof(double) * n, cudaMemcpyDeviceToDevice, st));
+            cg_precondition(h, FIN_RHO_INIT);              // beta = 0
             restart = false;
         }
-        {
-            Scope sc_(&h->prof, st, K_SPMV_DOT, by_spmv);
-            k_spmv_dot<<<red_grid(h, S.nslices), TPB, 0, st>>>(S, A, h->p, h->q, h->red, h->sc);
+        const float* z32 = reinterpret_cast<const float*>(h->z);
+        if (sell_small(h, S)) {
+            Scope sc_(&h->prof, st, K_SPMV_DOT, 12.0 * nnz + (zf ? 36.0 : 40.0) * n);
+            if (zf)
+                launch_sell<8>(k_direction<8, float>, red_grid(h, S.nslices), st, S, A, z32, h->p, h->q, h->red, h->sc);
+            else
+                launch_sell<8>(k_direction<8, double>, red_grid(h, S.nslices), st, S, A, h->z, h->p, h->q, h->red, h->sc);
+            KERNEL_CHECK();
+        } else {
+            {
+                Scope sc_(&h->prof, st, K_UPDATE_P, (zf ? 20.0 : 24.0) * n);
+                if (zf) launch_dep(k_update_p<float>, vec_grid(h, n), TPB, 0, st, n, z32, h->p, h->sc);
+                else launch_dep(k_update_p<double>, vec_grid(h, n), TPB, 0, st, n, h->z, h->p, h->sc);
+                KERNEL_CHECK();
+            }
+            Scope sc_(&h->prof, st, K_SPMV_DOT, 12.0 * nnz + 16.0 * n);
+            launch_sell<4>(k_spmv_dot<4>, red_grid(h, S.nslices), st, S, A, h->p, h->q, h->red, h->sc);
             KERNEL_CHECK();
         }
         {
             Scope sc_(&h->prof, st, K_UPDATE_XR, 48.0 * n + (r32 ? 4.0 * n : 0.0));
-            k_update_xr<<<red_grid_rows(h, n), TPB, 0, st>>>(n, h->p, h->q, x, h->r, r32, h->red, h->sc);
+            launch_dep(k_update_xr, red_grid_rows(h, n), TPB, 0, st, n, h->p, h->q, x, h->r, r32, h->red, h->sc);
             KERNEL_CHECK();
         }
         ++it;
         // The scalars go to the host. While the residual is well above the
-        // tolerance, the next iteration's preconditioner and direction update
-        // (which write only z, p and the device scalars) are queued behind the
+        // tolerance, the next iteration's preconditioner (which
+        // writes only z and the device scalars) are queued behind the
         // copy before the host waits for it, so the round trip overlaps the
         // V-cycle; if the check below ends the loop after all, x and r are
         // final and that work goes unused, and a restart recomputes rho and p
@@ -1635,7 +1789,7 @@ amg_status solve(amg_hierarchy* h, const double* b, double* x, double rtol, int 
         if (rel <= rtol) {
             {
                 Scope sc_(&h->prof, st, K_RESIDUAL, by_res);
-                k_residual<<<red_grid(h, S.nslices), TPB, 0, st>>>(S, A, x, b, h->t, h->red, h->sc);
+                SELL_DISPATCH(h, S, launch_sell<RB>(k_residual<RB>, red_grid(h, S.nslices), st, S, A, x, b, h->t, h->red, h->sc));
                 KERNEL_CHECK();
             }
             read_scalars(h);
@@ -1653,7 +1807,7 @@ amg_status solve(amg_hierarchy* h, const double* b, double* x, double rtol, int 
     if (!have_true) {
         {
             Scope sc_(&h->prof, st, K_RESIDUAL, by_res);
-            k_residual<<<red_grid(h, S.nslices), TPB, 0, st>>>(S, A, x, b, h->t, h->red, h->sc);
+            SELL_DISPATCH(h, S, launch_sell<RB>(k_residual<RB>, red_grid(h, S.nslices), st, S, A, x, b, h->t, h->red, h->sc));
             KERNEL_CHECK();
         }
         read_scalars(h);
