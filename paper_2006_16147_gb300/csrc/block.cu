@@ -68,31 +68,28 @@ __device__ __forceinline__ Grp make_grp(int G) {
 // The CPL consecutive values at p (a lane's columns of one row; lim of them
 // are live columns). With VEC the row stride is a multiple of CPL, so the
 // address is aligned to CPL values and all CPL lie inside the row: the loads
-// are vectors. Without VEC only the live columns are read. CG reads with plain
-// loads (values that other blocks write during the launch and a grid barrier
-// publishes; its fences order them).
-template <bool VEC, bool CG, int CPL, typename T>
+// are vectors. Without VEC only the live columns are read. Never ld.nc (see
+// dep_wait).
+template <bool VEC, int CPL, typename T>
 __device__ __forceinline__ void ld_cols(const T* p, T (&v)[CPL], int lim) {
     if constexpr (VEC && std::is_same<T, float>::value && CPL >= 4) {
 #pragma unroll
         for (int q = 0; q < CPL / 4; ++q) {
-            const float4 f = CG ? reinterpret_cast<const float4*>(p)[q]
-                                : __ldg(reinterpret_cast<const float4*>(p) + q);
+            const float4 f = __ldca(reinterpret_cast<const float4*>(p) + q);
             v[4 * q] = f.x; v[4 * q + 1] = f.y; v[4 * q + 2] = f.z; v[4 * q + 3] = f.w;
         }
     } else if constexpr (VEC && std::is_same<T, float>::value && CPL == 2) {
-        const float2 f = CG ? *reinterpret_cast<const float2*>(p) : __ldg(reinterpret_cast<const float2*>(p));
+        const float2 f = __ldca(reinterpret_cast<const float2*>(p));
         v[0] = f.x; v[1] = f.y;
     } else if constexpr (VEC && std::is_same<T, double>::value && CPL >= 2) {
 #pragma unroll
         for (int q = 0; q < CPL / 2; ++q) {
-            const double2 f = CG ? reinterpret_cast<const double2*>(p)[q]
-                                 : __ldg(reinterpret_cast<const double2*>(p) + q);
+            const double2 f = __ldca(reinterpret_cast<const double2*>(p) + q);
             v[2 * q] = f.x; v[2 * q + 1] = f.y;
         }
     } else {
 #pragma unroll
-        for (int m = 0; m < CPL; ++m) v[m] = m < lim ? (CG ? p[m] : __ldg(p + m)) : T(0);
+        for (int m = 0; m < CPL; ++m) v[m] = m < lim ? __ldca(p + m) : T(0);
     }
 }
 
@@ -154,7 +151,7 @@ __device__ __forceinline__ void st_cols(T* p, const T (&v)[CPL], int c0, int k) 
 // predicated): their indices and values are loaded first and the four
 // gathered rows of X are in flight together, so a row costs about two memory
 // latencies per four entries instead of two per entry.
-template <bool VEC, bool CG, int CPL, typename T>
+template <bool VEC, int CPL, typename T>
 __device__ __forceinline__ void sell_row_k(const SellV& S, const T* __restrict__ val, int ip, int c0, int k,
                                            const T* X, int ld, T (&acc)[CPL]) {
     if (c0 >= k) return;
@@ -173,7 +170,7 @@ __device__ __forceinline__ void sell_row_k(const SellV& S, const T* __restrict__
         }
         T xs[4][CPL];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) ld_cols<VEC, CG, CPL>(X + (size_t)j[u] * ld + c0, xs[u], k - c0);
+        for (int u = 0; u < 4; ++u) ld_cols<VEC, CPL>(X + (size_t)j[u] * ld + c0, xs[u], k - c0);
 #pragma unroll
         for (int u = 0; u < 4; ++u)
 #pragma unroll
@@ -191,7 +188,7 @@ __device__ __forceinline__ void sell_row_k(const SellV& S, const T* __restrict__
         T xs[4][CPL];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            if (e + u < w) ld_cols<VEC, CG, CPL>(X + (size_t)j[u] * ld + c0, xs[u], k - c0);
+            if (e + u < w) ld_cols<VEC, CPL>(X + (size_t)j[u] * ld + c0, xs[u], k - c0);
             else
 #pragma unroll
                 for (int m = 0; m < CPL; ++m) xs[u][m] = T(0);
@@ -203,6 +200,45 @@ __device__ __forceinline__ void sell_row_k(const SellV& S, const T* __restrict__
                 for (int m = 0; m < CPL; ++m) acc[m] = fma(a[u], xs[u][m], acc[m]);
     }
 }
+
+// The same for FP64 values and float X, in FP64 accuracy without the FP64 pipe
+// (SplitSum); a column in `on` to which that does not apply takes the FP64
+// chain. A matrix entry is split once for the lane's columns. One entry at a
+// time: in 64 registers the other warps hide the loads, and four blocks per SM
+// matter more (128^3 x 64 columns: 2407 us, 2600-3400 us with two or four
+// entries in flight and two or three blocks).
+template <bool VEC, int CPL>
+__device__ __forceinline__ void sell_row_split(const SellV& S, const double* __restrict__ val, int ip, int c0, int k,
+                                               const float* __restrict__ X, int ld, const bool (&on)[CPL],
+                                               double (&acc)[CPL]) {
+    const int s = ip >> 5, r = ip & 31;
+    const int s0 = __ldg(S.sptr + s);
+    const int w = __ldg(S.sptr + s + 1) - s0;
+    const long long base = (long long)s0 * 32 + r;
+    SplitSum sum[CPL];
+    for (int e = 0; e < w; ++e) {
+        const int j = __ldg(S.col + base + 32 * e);
+        const Split3 a = split3(__ldg(val + base + 32 * e));
+        float xs[CPL];
+        ld_cols<VEC, CPL>(X + (size_t)j * ld + c0, xs, k - c0);
+#pragma unroll
+        for (int m = 0; m < CPL; ++m) sum[m].add(a, xs[m]);
+    }
+#pragma unroll
+    for (int m = 0; m < CPL; ++m) {
+        acc[m] = sum[m].value();
+        if (on[m] && !sum[m].ok()) {
+            double t = 0.0;
+            for (int e = 0; e < w; ++e)
+                t = fma(__ldg(val + base + 32 * e),
+                        (double)ldv(X + (size_t)__ldg(S.col + base + 32 * e) * ld + c0 + m), t);
+            acc[m] = t;
+        }
+    }
+}
+
+__device__ __forceinline__ double to_d(double v) { return v; }
+__device__ __forceinline__ double to_d(float v) { return f2d(v); }
 
 // Sums over `count` blocks' partials (value j of column c of block b at
 // part[(b * 2 + j) * k + c]) by the whole block: tpc consecutive lanes per
@@ -308,6 +344,7 @@ template <typename T, int CPL, bool VEC>
 __global__ void __launch_bounds__(TPB) bk_pre(SellV S, const T* __restrict__ valm, const T* __restrict__ minv, T omega,
                                               const T* __restrict__ B, T* __restrict__ X, T* __restrict__ R, int k, int ld,
                                               int G) {
+    dep_wait();
     const Grp g = make_grp(G);
     const int c0 = g.gl * CPL;
     if (c0 >= k) return;
@@ -315,12 +352,12 @@ __global__ void __launch_bounds__(TPB) bk_pre(SellV S, const T* __restrict__ val
         T acc[CPL];
 #pragma unroll
         for (int m = 0; m < CPL; ++m) acc[m] = 0;
-        sell_row_k<VEC, false, CPL>(S, valm, ip, c0, k, B, ld, acc);
+        sell_row_k<VEC, CPL>(S, valm, ip, c0, k, B, ld, acc);
         const int i = rowid(S, ip);
         const T mi = omega * minv[i];
         const size_t o = (size_t)i * ld + c0;
         T bi[CPL], xo[CPL], ro[CPL];
-        ld_cols<VEC, false, CPL>(B + o, bi, k - c0);
+        ld_cols<VEC, CPL>(B + o, bi, k - c0);
 #pragma unroll
         for (int m = 0; m < CPL; ++m) {
             xo[m] = mi * bi[m];
@@ -331,20 +368,11 @@ __global__ void __launch_bounds__(TPB) bk_pre(SellV S, const T* __restrict__ val
     }
 }
 
-// FP32 copy of columns [0, k) of the level-0 residual (row-major, leading
-// dimension ld) for the FP32 V-cycle: one conversion per entry instead of one
-// per gathered matrix entry (the FP64 -> FP32 conversion runs at the FP64 rate).
-__global__ void __launch_bounds__(TPB) bk_to_f32(long long n, int k, int ld, const double* __restrict__ a,
-                                                 float* __restrict__ b) {
-    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n * ld;
-         t += (long long)gridDim.x * blockDim.x)
-        if (k == ld || (int)(t % ld) < k) b[t] = (float)a[t];
-}
-
 template <typename T, int CPL, bool VEC>
 __global__ void __launch_bounds__(TPB) bk_restrict(int nc, const int* __restrict__ pt_ptr,
                                                    const int* __restrict__ pt_idx, const T* __restrict__ p,
                                                    const T* __restrict__ R, T* __restrict__ Bc, int k, int ld, int G) {
+    dep_wait();
     const Grp g = make_grp(G);
     const int c0 = g.gl * CPL;
     if (c0 >= k) return;
@@ -356,7 +384,7 @@ __global__ void __launch_bounds__(TPB) bk_restrict(int nc, const int* __restrict
             const int i = __ldg(pt_idx + e);
             const T pi = __ldg(p + i);
             T rv[CPL];
-            ld_cols<VEC, false, CPL>(R + (size_t)i * ld + c0, rv, k - c0);
+            ld_cols<VEC, CPL>(R + (size_t)i * ld + c0, rv, k - c0);
 #pragma unroll
             for (int m = 0; m < CPL; ++m) acc[m] = fma(pi, rv[m], acc[m]);
         }
@@ -364,29 +392,43 @@ __global__ void __launch_bounds__(TPB) bk_restrict(int nc, const int* __restrict
     }
 }
 
-// X = A_L^{-1} B on the coarsest level, FP64 arithmetic.
+// X = A_L^{-1} B on the coarsest level, FP64 arithmetic. A block per row: TPB / G
+// slices of the row's entries, each by a group of G lanes over all columns, and
+// a tree over the slices. (A group per row ran all n entries in series: 50 us
+// for 64 rows and 64 columns, 6.5 us now.)
 template <typename TI, typename TO, int CPL, bool VEC>
 __global__ void __launch_bounds__(TPB) bk_coarse_dense(int n, const double* __restrict__ Ainv, const TI* __restrict__ B,
                                                        TO* __restrict__ X, int k, int ld, int G) {
-    const Grp g = make_grp(G);
-    const int c0 = g.gl * CPL;
-    if (c0 >= k) return;
-    for (int i = g.gw; i < n; i += g.ngroups) {
+    __shared__ double sm[TPB * CPL];
+    const int gl = threadIdx.x % G, slice = threadIdx.x / G, slices = TPB / G;
+    const int c0 = gl * CPL;
+    dep_wait();
+    for (int i = blockIdx.x; i < n; i += gridDim.x) {
         double acc[CPL];
 #pragma unroll
         for (int m = 0; m < CPL; ++m) acc[m] = 0.0;
         const double* row = Ainv + (size_t)i * n;
-        for (int j = 0; j < n; ++j) {
-            const double a = __ldg(row + j);
-            TI bv[CPL];
-            ld_cols<VEC, false, CPL>(B + (size_t)j * ld + c0, bv, k - c0);
+        if (c0 < k)
+#pragma unroll 4
+            for (int j = slice; j < n; j += slices) {
+                const double a = __ldg(row + j);
+                TI bv[CPL];
+                ld_cols<VEC, CPL>(B + (size_t)j * ld + c0, bv, k - c0);
 #pragma unroll
-            for (int m = 0; m < CPL; ++m) acc[m] = fma(a, (double)bv[m], acc[m]);
+                for (int m = 0; m < CPL; ++m) acc[m] = fma(a, to_d(bv[m]), acc[m]);
+            }
+#pragma unroll
+        for (int m = 0; m < CPL; ++m) sm[m * TPB + threadIdx.x] = acc[m];
+        __syncthreads();
+        for (int t = slices >> 1; t > 0; t >>= 1) {
+            for (int q = threadIdx.x; q < t * G * CPL; q += TPB) {
+                double* v = sm + q / (t * G) * TPB + q % (t * G);
+                *v += v[t * G];
+            }
+            __syncthreads();
         }
-        TO xo[CPL];
-#pragma unroll
-        for (int m = 0; m < CPL; ++m) xo[m] = (TO)acc[m];
-        st_cols<VEC, CPL>(X + (size_t)i * ld + c0, xo, c0, k);
+        for (int c = threadIdx.x; c < k; c += TPB) X[(size_t)i * ld + c] = (TO)sm[c % CPL * TPB + c / CPL];
+        __syncthreads();
     }
 }
 
@@ -416,6 +458,7 @@ __global__ void __launch_bounds__(TPB) bk_post(SellV SAP, const T* __restrict__ 
                                                const T* __restrict__ R, const double* __restrict__ Bdot,
                                                const double* __restrict__ Q2, TO* __restrict__ Out, int k, int ld, int G,
                                                double* partial, unsigned* ticket, BlockScalars sc, int flexible) {
+    dep_wait();
     const Grp g = make_grp(G);
     const int c0 = g.gl * CPL;
     double d[2][CPL];
@@ -426,7 +469,7 @@ __global__ void __launch_bounds__(TPB) bk_post(SellV SAP, const T* __restrict__ 
             T acc[CPL];
 #pragma unroll
             for (int m = 0; m < CPL; ++m) acc[m] = 0;
-            sell_row_k<VEC, false, CPL>(SAP, apval, ip, c0, k, E, ld, acc);
+            sell_row_k<VEC, CPL>(SAP, apval, ip, c0, k, E, ld, acc);
             const int i = rowid(SAP, ip);
             const int a = agg[i];
             const T pi = p[i];
@@ -434,9 +477,9 @@ __global__ void __launch_bounds__(TPB) bk_post(SellV SAP, const T* __restrict__ 
             const size_t o = (size_t)i * ld + c0;
             T ev[CPL], xv[CPL], rv[CPL];
             TO ov[CPL];
-            ld_cols<VEC, false, CPL>(E + (size_t)a * ld + c0, ev, k - c0);
-            ld_cols<VEC, false, CPL>(X + o, xv, k - c0);
-            ld_cols<VEC, false, CPL>(R + o, rv, k - c0);
+            ld_cols<VEC, CPL>(E + (size_t)a * ld + c0, ev, k - c0);
+            ld_cols<VEC, CPL>(X + o, xv, k - c0);
+            ld_cols<VEC, CPL>(R + o, rv, k - c0);
 #pragma unroll
             for (int m = 0; m < CPL; ++m) {
                 const T y = fma(pi, ev[m], xv[m]);
@@ -445,13 +488,14 @@ __global__ void __launch_bounds__(TPB) bk_post(SellV SAP, const T* __restrict__ 
             st_cols<VEC, CPL>(Out + o, ov, c0, k);
             if (DOT) {
                 double bd[CPL], qd[CPL];
-                ld_cols<VEC, false, CPL>(Bdot + o, bd, k - c0);
-                if (Q2) ld_cols<VEC, false, CPL>(Q2 + o, qd, k - c0);
+                ld_cols<VEC, CPL>(Bdot + o, bd, k - c0);
+                if (Q2) ld_cols<VEC, CPL>(Q2 + o, qd, k - c0);
 #pragma unroll
                 for (int m = 0; m < CPL; ++m) {
                     if (c0 + m >= k) continue;
-                    d[0][m] = fma(bd[m], (double)ov[m], d[0][m]);
-                    if (Q2) d[1][m] = fma(qd[m], (double)ov[m], d[1][m]);
+                    const double od = to_d(ov[m]);
+                    d[0][m] = fma(bd[m], od, d[0][m]);
+                    if (Q2) d[1][m] = fma(qd[m], od, d[1][m]);
                 }
             }
         }
@@ -597,7 +641,7 @@ __global__ void __launch_bounds__(CC_TPB) bk_coarse_cg(SellV S, const double* __
             const size_t o = (size_t)i * ld + c0;
             TI bt[CPL];
             double bi[CPL], zi[CPL], zero[CPL];
-            ld_cols<VEC, false, CPL>(B + o, bt, k - c0);
+            ld_cols<VEC, CPL>(B + o, bt, k - c0);
 #pragma unroll
             for (int m = 0; m < CPL; ++m) {
                 bi[m] = (double)bt[m];
@@ -642,10 +686,10 @@ __global__ void __launch_bounds__(CC_TPB) bk_coarse_cg(SellV S, const double* __
         double pv[CPL], qv[CPL], zv[CPL];
         auto own_row = [&](int i) {
             const size_t o = (size_t)i * ld + c0;
-            ld_cols<VEC, true, CPL>(z + o, zv, k - c0);
+            ld_cols<VEC, CPL>(z + o, zv, k - c0);
             if (it > 0) {
-                ld_cols<VEC, true, CPL>(p + o, pv, k - c0);
-                ld_cols<VEC, true, CPL>(q + o, qv, k - c0);
+                ld_cols<VEC, CPL>(p + o, pv, k - c0);
+                ld_cols<VEC, CPL>(q + o, qv, k - c0);
             }
         };
         auto finish_row = [&](int i, const double (&acc)[CPL]) {
@@ -666,7 +710,7 @@ __global__ void __launch_bounds__(CC_TPB) bk_coarse_cg(SellV S, const double* __
                 for (int m = 0; m < CPL; ++m) acc[m] = 0.0;
                 const int i = rowid(S, ip);
                 own_row(i);
-                sell_row_k<VEC, true, CPL>(S, sval, ip, c0, k, (const double*)z, ld, acc);
+                sell_row_k<VEC, CPL>(S, sval, ip, c0, k, (const double*)z, ld, acc);
                 finish_row(i, acc);
             }
         // long rows: a warp per row, its lane groups take the entries in turn
@@ -681,7 +725,7 @@ __global__ void __launch_bounds__(CC_TPB) bk_coarse_cg(SellV S, const double* __
                 for (int e = __ldg(cptr + i) + lane / G; e < e1; e += 32 / G) {
                     const double a = __ldg(cval + e);
                     double ze[CPL];
-                    ld_cols<VEC, true, CPL>((const double*)z + (size_t)__ldg(ccol + e) * ld + c0, ze, k - c0);
+                    ld_cols<VEC, CPL>((const double*)z + (size_t)__ldg(ccol + e) * ld + c0, ze, k - c0);
 #pragma unroll
                     for (int m = 0; m < CPL; ++m) acc[m] = fma(a, ze[m], acc[m]);
                 }
@@ -713,8 +757,8 @@ __global__ void __launch_bounds__(CC_TPB) bk_coarse_cg(SellV S, const double* __
                 const double mi = minv[i];
                 const size_t o = (size_t)i * ld + c0;
                 double pv[CPL], qv[CPL], xv[CPL], rv[CPL], zv[CPL];
-                ld_cols<VEC, true, CPL>(p + o, pv, k - c0);
-                ld_cols<VEC, true, CPL>(q + o, qv, k - c0);
+                ld_cols<VEC, CPL>(p + o, pv, k - c0);
+                ld_cols<VEC, CPL>(q + o, qv, k - c0);
                 ld_own<VEC, CPL>(x + o, xv, k - c0);
                 ld_own<VEC, CPL>(r + o, rv, k - c0);
 #pragma unroll
@@ -757,30 +801,61 @@ __global__ void __launch_bounds__(CC_TPB) bk_coarse_cg(SellV S, const double* __
 }
 
 // ------------------------------------------------------------- CG ----------
-// Q = A P; p . q per column; alpha = rho / p.q for ACTIVE columns, else 0.
-template <int CPL, bool VEC>
-__global__ void __launch_bounds__(TPB) bk_spmv_dot(SellV S, const double* __restrict__ val,
-                                                   const double* __restrict__ P, double* __restrict__ Q, int k, int ld, int G,
-                                                   double* partial, unsigned* ticket, BlockScalars sc) {
+// ACTIVE columns: P = Z + beta P, Q = A Z + beta Q (= A P; a column that just
+// started has beta = 0 and reads neither), p . q and alpha = rho / p.q; alpha =
+// 0 for the others, whose P and Q keep their values. The product takes Z, the
+// V-cycle's output in its own type: for FP32 the products are formed in FP32
+// pieces, so FP64 instructions are 5 a row and column instead of 9 in the
+// product and direction passes that this replaces, which were bound by them:
+// 128^3 rows x 64 columns 2143 + 495 us, 2407 us now; 64^3 x 16 about 107 us,
+// 95 us now.
+template <typename TZ, int CPL, bool VEC>
+__global__ void __launch_bounds__(TPB, sizeof(TZ) == 4 && CPL <= 4 ? 4 : 1) bk_direction(SellV S, const double* __restrict__ val,
+                                                    const TZ* __restrict__ Z, double* __restrict__ P,
+                                                    double* __restrict__ Q, int k, int ld, int G, double* partial,
+                                                    unsigned* ticket, BlockScalars sc) {
+    dep_wait();
     const Grp g = make_grp(G);
     const int c0 = g.gl * CPL;
-    double d[1][CPL];
+    double be[CPL], d[1][CPL];
+    bool on[CPL], any = false, old = false;
 #pragma unroll
-    for (int m = 0; m < CPL; ++m) d[0][m] = 0.0;
-    if (c0 < k) {
+    for (int m = 0; m < CPL; ++m) {
+        const int c = c0 + m;
+        on[m] = c < k && sc.mode[c] == COL_ACTIVE;
+        be[m] = on[m] ? sc.beta[c] : 0.0;
+        any |= on[m];
+        old |= c < k && (!on[m] || be[m] != 0.0);
+        d[0][m] = 0.0;
+    }
+    if (any) {
         for (int ip = g.gw; ip < S.n; ip += g.ngroups) {
-            double acc[CPL];
-#pragma unroll
-            for (int m = 0; m < CPL; ++m) acc[m] = 0.0;
-            sell_row_k<VEC, false, CPL>(S, val, ip, c0, k, P, ld, acc);
             const int i = rowid(S, ip);
             const size_t o = (size_t)i * ld + c0;
-            double pv[CPL];
-            ld_cols<VEC, false, CPL>(P + o, pv, k - c0);
-            st_cols<VEC, CPL>(Q + o, acc, c0, k);
+            double acc[CPL], pv[CPL], qv[CPL];
+            TZ zv[CPL];
+            if constexpr (sizeof(TZ) == 4) {
+                sell_row_split<VEC, CPL>(S, val, ip, c0, k, Z, ld, on, acc);
+            } else {
 #pragma unroll
-            for (int m = 0; m < CPL; ++m)
-                if (c0 + m < k) d[0][m] = fma(pv[m], acc[m], d[0][m]);
+                for (int m = 0; m < CPL; ++m) acc[m] = 0.0;
+                sell_row_k<VEC, CPL>(S, val, ip, c0, k, Z, ld, acc);
+            }
+            ld_cols<VEC, CPL>(Z + o, zv, k - c0);
+            if (old) {
+                ld_own<VEC, CPL>(P + o, pv, k - c0);
+                ld_own<VEC, CPL>(Q + o, qv, k - c0);
+            }
+#pragma unroll
+            for (int m = 0; m < CPL; ++m) {
+                if (!on[m]) continue;
+                const double zd = to_d(zv[m]);
+                pv[m] = be[m] == 0.0 ? zd : fma(be[m], pv[m], zd);
+                qv[m] = be[m] == 0.0 ? acc[m] : fma(be[m], qv[m], acc[m]);
+                d[0][m] = fma(pv[m], qv[m], d[0][m]);
+            }
+            st_cols<VEC, CPL>(P + o, pv, c0, k);
+            st_cols<VEC, CPL>(Q + o, qv, c0, k);
         }
     }
     colsum<CPL, 1>(d, g, k, ld, partial, ticket, [&](int c, double pq, double) {
@@ -801,10 +876,14 @@ __global__ void __launch_bounds__(TPB) bk_spmv_dot(SellV S, const double* __rest
 
 // ACTIVE columns: X += alpha P, R -= alpha Q, ||R||^2; convergence -> CHECK.
 // Other columns are written back unchanged when a vector store covers them.
+// With R32 set (FP32 V-cycle) also the float copy of R that the V-cycle reads:
+// this kernel and bk_residual, the two that write R, keep it.
 template <int CPL, bool VEC>
 __global__ void __launch_bounds__(TPB) bk_update_xr(int n, const double* __restrict__ P, const double* __restrict__ Q,
-                                                    double* __restrict__ X, double* __restrict__ R, int k, int ld, int G,
+                                                    double* __restrict__ X, double* __restrict__ R,
+                                                    float* __restrict__ R32, int k, int ld, int G,
                                                     double* partial, unsigned* ticket, BlockScalars sc) {
+    dep_wait();
     const Grp g = make_grp(G);
     const int c0 = g.gl * CPL;
     double al[CPL];
@@ -824,8 +903,8 @@ __global__ void __launch_bounds__(TPB) bk_update_xr(int n, const double* __restr
         for (int i = g.gw; i < n; i += g.ngroups) {
             const size_t o = (size_t)i * ld + c0;
             double pv[CPL], qv[CPL], xv[CPL], rv[CPL];
-            ld_cols<VEC, false, CPL>(P + o, pv, k - c0);
-            ld_cols<VEC, false, CPL>(Q + o, qv, k - c0);
+            ld_cols<VEC, CPL>(P + o, pv, k - c0);
+            ld_cols<VEC, CPL>(Q + o, qv, k - c0);
             ld_own<VEC, CPL>(X + o, xv, k - c0);
             ld_own<VEC, CPL>(R + o, rv, k - c0);
 #pragma unroll
@@ -837,6 +916,12 @@ __global__ void __launch_bounds__(TPB) bk_update_xr(int n, const double* __restr
             }
             st_cols<VEC, CPL>(X + o, xv, c0, k);
             st_cols<VEC, CPL>(R + o, rv, c0, k);
+            if (R32) {
+                float rf[CPL];
+#pragma unroll
+                for (int m = 0; m < CPL; ++m) rf[m] = d2f(rv[m]);
+                st_cols<VEC, CPL>(R32 + o, rf, c0, k);
+            }
         }
     }
     colsum<CPL, 1>(d, g, k, ld, partial, ticket, [&](int c, double rr, double) {
@@ -845,35 +930,6 @@ __global__ void __launch_bounds__(TPB) bk_update_xr(int n, const double* __restr
         sc.iters[c] += 1;
         if (rr <= sc.rtol[c] * sc.rtol[c] * sc.bb[c]) sc.mode[c] = COL_CHECK;
     });
-}
-
-// ACTIVE columns: P = Z + beta P (P = Z when beta = 0, whatever P held).
-template <int CPL, bool VEC>
-__global__ void __launch_bounds__(TPB) bk_update_p(int n, const double* __restrict__ Z, double* __restrict__ P, int k,
-                                                   int ld, int G, BlockScalars sc) {
-    const Grp g = make_grp(G);
-    const int c0 = g.gl * CPL;
-    double be[CPL];
-    bool on[CPL];
-    bool any = false;
-#pragma unroll
-    for (int m = 0; m < CPL; ++m) {
-        const int c = c0 + m;
-        on[m] = c < k && sc.mode[c] == COL_ACTIVE;
-        be[m] = on[m] ? sc.beta[c] : 0.0;
-        any |= on[m];
-    }
-    if (!any) return;
-    for (int i = g.gw; i < n; i += g.ngroups) {
-        const size_t o = (size_t)i * ld + c0;
-        double zv[CPL], pv[CPL];
-        ld_cols<VEC, false, CPL>(Z + o, zv, k - c0);
-        ld_own<VEC, CPL>(P + o, pv, k - c0);
-#pragma unroll
-        for (int m = 0; m < CPL; ++m)
-            if (on[m]) pv[m] = be[m] == 0.0 ? zv[m] : fma(be[m], pv[m], zv[m]);
-        st_cols<VEC, CPL>(P + o, pv, c0, k);
-    }
 }
 
 // R = B - A X for the selected columns, ||R||^2 and ||B||^2.
@@ -886,8 +942,10 @@ __global__ void __launch_bounds__(TPB) bk_update_p(int n, const double* __restri
 template <int CPL, bool VEC>
 __global__ void __launch_bounds__(TPB) bk_residual(SellV S, const double* __restrict__ val,
                                                    const double* __restrict__ X, const double* __restrict__ B,
-                                                   double* __restrict__ R, int k, int ld, int G, double* partial,
+                                                   double* __restrict__ R, float* __restrict__ R32, int k, int ld,
+                                                   int G, double* partial,
                                                    unsigned* ticket, BlockScalars sc, int stage) {
+    dep_wait();
     const Grp g = make_grp(G);
     const int c0 = g.gl * CPL;
     bool on[CPL];
@@ -907,11 +965,11 @@ __global__ void __launch_bounds__(TPB) bk_residual(SellV S, const double* __rest
             double acc[CPL];
 #pragma unroll
             for (int m = 0; m < CPL; ++m) acc[m] = 0.0;
-            sell_row_k<VEC, false, CPL>(S, val, ip, c0, k, X, ld, acc);
+            sell_row_k<VEC, CPL>(S, val, ip, c0, k, X, ld, acc);
             const int i = rowid(S, ip);
             const size_t o = (size_t)i * ld + c0;
             double bv[CPL], rv[CPL];
-            ld_cols<VEC, false, CPL>(B + o, bv, k - c0);
+            ld_cols<VEC, CPL>(B + o, bv, k - c0);
             ld_own<VEC, CPL>(R + o, rv, k - c0);
 #pragma unroll
             for (int m = 0; m < CPL; ++m) {
@@ -921,6 +979,12 @@ __global__ void __launch_bounds__(TPB) bk_residual(SellV S, const double* __rest
                 d[1][m] = fma(bv[m], bv[m], d[1][m]);
             }
             st_cols<VEC, CPL>(R + o, rv, c0, k);
+            if (R32) {
+                float rf[CPL];
+#pragma unroll
+                for (int m = 0; m < CPL; ++m) rf[m] = d2f(rv[m]);
+                st_cols<VEC, CPL>(R32 + o, rf, c0, k);
+            }
         }
     }
     colsum<CPL, 2>(d, g, k, ld, partial, ticket, [&](int c, double rr, double bb) {
@@ -1043,28 +1107,23 @@ void block_vcycle(amg_hierarchy* h, BlockWork& W, int k, int flexible) {
         const int g = grid_rows(h, Lv.S.n, G);
         Scope sc_(&h->prof, st, l == 0 ? K_PRE_L0 : K_PRE,
                   (double)Lv.A.nnz * (sizeof(T) + 4) + (double)Lv.A.n * k * ((l == 0 ? 8 : sizeof(T)) + 2.0 * sizeof(T)));
-        if (l == 0 && f32) {
-            bk_to_f32<<<blocks_for((long long)Lv.A.n * ld, TPB, h->num_sms * 8), TPB, 0, st>>>(
-                Lv.A.n, k, ld, W.R, reinterpret_cast<float*>(W.b[0]));
-            KERNEL_CHECK();
-        }
         if (l == 0 && !f32)
-            DISPATCH_CPL(cpl, ld, bk_pre<T, CPL, VEC><<<g, TPB, 0, st>>>(sv(Lv.S), valm, minv, omega, (const T*)W.R, lv(W.x, 0),
+            DISPATCH_CPL(cpl, ld, launch_dep(bk_pre<T, CPL, VEC>, g, TPB, 0, st, sv(Lv.S), valm, minv, omega, (const T*)W.R, lv(W.x, 0),
                                                                        lv(W.r, 0), k, ld, G));
         else
-            DISPATCH_CPL(cpl, ld, bk_pre<T, CPL, VEC><<<g, TPB, 0, st>>>(sv(Lv.S), valm, minv, omega, lv(W.b, l), lv(W.x, l),
+            DISPATCH_CPL(cpl, ld, launch_dep(bk_pre<T, CPL, VEC>, g, TPB, 0, st, sv(Lv.S), valm, minv, omega, lv(W.b, l), lv(W.x, l),
                                                                   lv(W.r, l), k, ld, G));
         KERNEL_CHECK();
         const int nc = h->lev[l + 1].A.n;
         const T* p = f32 ? (const T*)Lv.p32 : (const T*)Lv.p;
-        DISPATCH_CPL(cpl, ld, bk_restrict<T, CPL, VEC><<<grid_rows(h, nc, G), TPB, 0, st>>>(nc, Lv.pt_ptr, Lv.pt_idx, p,
+        DISPATCH_CPL(cpl, ld, launch_dep(bk_restrict<T, CPL, VEC>, grid_rows(h, nc, G), TPB, 0, st, nc, Lv.pt_ptr, Lv.pt_idx, p,
                                                                                    lv(W.r, l), lv(W.b, l + 1), k, ld, G));
         KERNEL_CHECK();
     }
     {
         Scope sc_(&h->prof, st, K_COARSE, 8.0 * h->nc * h->nc + 16.0 * h->nc * k);
         if (!h->coarse_cg) {
-            DISPATCH_CPL(cpl, ld, bk_coarse_dense<T, T, CPL, VEC><<<grid_rows(h, h->nc, G), TPB, 0, st>>>(
+            DISPATCH_CPL(cpl, ld, launch_dep(bk_coarse_dense<T, T, CPL, VEC>, std::min(h->nc, h->num_sms * 8), TPB, 0, st, 
                                   h->nc, h->coarse_inv, lv(W.b, L), lv(W.x, L), k, ld, G));
             KERNEL_CHECK();
         } else {
@@ -1103,13 +1162,13 @@ void block_vcycle(amg_hierarchy* h, BlockWork& W, int k, int flexible) {
         Scope sc_(&h->prof, st, l == 0 ? K_POST_L0 : K_POST,
                   (double)Lv.ap_nnz * (sizeof(T) + 4) + (double)Lv.A.n * k * (4.0 * sizeof(T) + 8));
         if (l > 0)
-            DISPATCH_CPL(cpl, ld, bk_post<T, T, CPL, false, VEC><<<g, TPB, 0, st>>>(
+            DISPATCH_CPL(cpl, ld, launch_dep(bk_post<T, T, CPL, false, VEC>, g, TPB, 0, st, 
                                   sv(Lv.AP), apv, minv, omega, Lv.agg, p, e, lv(W.x, l), lv(W.r, l), nullptr, nullptr,
                                   lv(W.y, l), k, ld, G, W.partial, W.ticket, W.sc, flexible));
         else
-            DISPATCH_CPL(cpl, ld, bk_post<T, double, CPL, true, VEC><<<red_grid(h, W, G), TPB, 0, st>>>(
+            DISPATCH_CPL(cpl, ld, launch_dep(bk_post<T, T, CPL, true, VEC>, red_grid(h, W, G), TPB, 0, st, 
                                   sv(Lv.AP), apv, minv, omega, Lv.agg, p, e, lv(W.x, 0), lv(W.r, 0), W.R,
-                                  flexible ? W.Q : nullptr, W.Z, k, ld, G, W.partial, W.ticket, W.sc, flexible));
+                                  flexible ? W.Q : nullptr, (T*)W.Z, k, ld, G, W.partial, W.ticket, W.sc, flexible));
         KERNEL_CHECK();
     }
 }
@@ -1245,6 +1304,11 @@ size_t block_bytes_per_column(const amg_hierarchy* h) {
     return rows * 4 * V + (size_t)h->lev[0].A.n * 5 * 8;
 }
 
+// Level 0's float copy of R (FP32 V-cycle), else null.
+static float* r32_of(amg_hierarchy* h) {
+    return h->opt.precision == AMG_FP32_VCYCLE ? static_cast<float*>(h->blk->b[0]) : nullptr;
+}
+
 // INIT columns among [0, k): residual of X, then START (or DONE for b = 0,
 // whose X column is zeroed). Launches only.
 void block_init_launch(amg_hierarchy* h, const double* B, double* X, int k) {
@@ -1253,8 +1317,8 @@ void block_init_launch(amg_hierarchy* h, const double* B, double* X, int k) {
     int G, cpl;
     group_shape(W, k, &G, &cpl);
     Level& L0 = h->lev[0];
-    DISPATCH_CPL(cpl, W.K, bk_residual<CPL, VEC><<<red_grid(h, W, G), TPB, 0, st>>>(sv(L0.S), L0.S.val, X, B, W.R, k, W.K, G, W.partial,
-                                                             W.ticket, W.sc, 0));
+    DISPATCH_CPL(cpl, W.K, launch_dep(bk_residual<CPL, VEC>, red_grid(h, W, G), TPB, 0, st, sv(L0.S), L0.S.val, X, B, W.R, r32_of(h), k, W.K, G,
+                                                             W.partial, W.ticket, W.sc, 0));
     KERNEL_CHECK();
     bk_zero_cols<<<blocks_for((long long)L0.A.n * k, TPB, h->num_sms * 8), TPB, 0, st>>>(L0.A.n, X, k, W.K, W.sc.mode,
                                                                                       W.sc.bb);
@@ -1264,7 +1328,7 @@ void block_init_launch(amg_hierarchy* h, const double* B, double* X, int k) {
 namespace {
 
 // The kernels of one step of columns [0, k): with `any_active` the CG half
-// (q = A p, x and r updates), then the V-cycle and p = z + beta p.
+// (p and q from the last step's z, x and r updates), then the V-cycle.
 void block_step_kernels(amg_hierarchy* h, double* X, int k, bool any_active) {
     BlockWork& W = *h->blk;
     cudaStream_t st = h->stream;
@@ -1275,27 +1339,28 @@ void block_step_kernels(amg_hierarchy* h, double* X, int k, bool any_active) {
     Level& L0 = h->lev[0];
     const int n = L0.A.n;
     const double nnz = (double)L0.A.nnz;
+    const bool f32 = h->opt.precision == AMG_FP32_VCYCLE;
     if (any_active) {
         {
-            Scope sc_(&h->prof, st, K_SPMV_DOT, 12.0 * nnz + 16.0 * n * k);
-            DISPATCH_CPL(cpl, ld, bk_spmv_dot<CPL, VEC><<<red_grid(h, W, G), TPB, 0, st>>>(sv(L0.S), L0.S.val, W.P, W.Q, k, ld, G,
-                                                                     W.partial, W.ticket, W.sc));
+            Scope sc_(&h->prof, st, K_SPMV_DOT, 12.0 * nnz + (f32 ? 36.0 : 40.0) * n * k);
+            if (f32)
+                DISPATCH_CPL(cpl, ld, launch_dep(bk_direction<float, CPL, VEC>, red_grid(h, W, G), TPB, 0, st, 
+                                          sv(L0.S), L0.S.val, (const float*)W.Z, W.P, W.Q, k, ld, G, W.partial,
+                                          W.ticket, W.sc));
+            else
+                DISPATCH_CPL(cpl, ld, launch_dep(bk_direction<double, CPL, VEC>, red_grid(h, W, G), TPB, 0, st, 
+                                          sv(L0.S), L0.S.val, W.Z, W.P, W.Q, k, ld, G, W.partial, W.ticket, W.sc));
             KERNEL_CHECK();
         }
         {
-            Scope sc_(&h->prof, st, K_UPDATE_XR, 48.0 * n * k);
-            DISPATCH_CPL(cpl, ld, bk_update_xr<CPL, VEC><<<red_grid(h, W, G), TPB, 0, st>>>(n, W.P, W.Q, X, W.R, k, ld, G, W.partial,
-                                                                      W.ticket, W.sc));
+            Scope sc_(&h->prof, st, K_UPDATE_XR, (f32 ? 52.0 : 48.0) * n * k);
+            DISPATCH_CPL(cpl, ld, launch_dep(bk_update_xr<CPL, VEC>, red_grid(h, W, G), TPB, 0, st, n, W.P, W.Q, X, W.R, r32_of(h), k, ld, G,
+                                                                      W.partial, W.ticket, W.sc));
             KERNEL_CHECK();
         }
     }
-    if (h->opt.precision == AMG_FP32_VCYCLE) block_vcycle<float>(h, W, k, flexible);
+    if (f32) block_vcycle<float>(h, W, k, flexible);
     else block_vcycle<double>(h, W, k, flexible);
-    {
-        Scope sc_(&h->prof, st, K_UPDATE_P, 24.0 * n * k);
-        DISPATCH_CPL(cpl, ld, bk_update_p<CPL, VEC><<<grid_rows(h, n, G), TPB, 0, st>>>(n, W.Z, W.P, k, ld, G, W.sc));
-        KERNEL_CHECK();
-    }
 }
 
 bool any_active_column(const BlockWork& W, int k) {
@@ -1378,8 +1443,8 @@ bool block_check_launch(amg_hierarchy* h, const double* B, double* X, int k) {
     Level& L0 = h->lev[0];
     const double nnz = (double)L0.A.nnz;
     Scope sc_(&h->prof, h->stream, K_RESIDUAL, 12.0 * nnz + 24.0 * L0.A.n * k);
-    DISPATCH_CPL(cpl, W.K, bk_residual<CPL, VEC><<<red_grid(h, W, G), TPB, 0, h->stream>>>(sv(L0.S), L0.S.val, X, B, W.R, k, W.K, G,
-                                                                    W.partial, W.ticket, W.sc, 1));
+    DISPATCH_CPL(cpl, W.K, launch_dep(bk_residual<CPL, VEC>, red_grid(h, W, G), TPB, 0, h->stream, sv(L0.S), L0.S.val, X, B, W.R, r32_of(h), k,
+                                                                    W.K, G, W.partial, W.ticket, W.sc, 1));
     KERNEL_CHECK();
     copy_state_async(h, W);
     return true;
@@ -1390,8 +1455,8 @@ void block_report_launch(amg_hierarchy* h, const double* B, const double* X, int
     int G, cpl;
     group_shape(W, k, &G, &cpl);
     Level& L0 = h->lev[0];
-    DISPATCH_CPL(cpl, W.K, bk_residual<CPL, VEC><<<red_grid(h, W, G), TPB, 0, h->stream>>>(sv(L0.S), L0.S.val, X, B, W.T, k, W.K, G,
-                                                                    W.partial, W.ticket, W.sc, 2));
+    DISPATCH_CPL(cpl, W.K, launch_dep(bk_residual<CPL, VEC>, red_grid(h, W, G), TPB, 0, h->stream, sv(L0.S), L0.S.val, X, B, W.T, nullptr, k, W.K,
+                                                                    G, W.partial, W.ticket, W.sc, 2));
     KERNEL_CHECK();
     copy_state_async(h, W);
 }

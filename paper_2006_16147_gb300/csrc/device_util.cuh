@@ -112,21 +112,26 @@ template <typename T>
 __device__ __forceinline__ T ldv(const T* p) { return __ldca(p); }
 
 // ----------------------------------------- FP64 beside a slow FP64 pipe ----
-// Conversions and adds of doubles cost 64 issue cycles per warp here, FP32 and
-// integer instructions one or two. The conversions below are the same values
-// from the IEEE formats' fields; the rare cases that are not a matter of moving
-// fields (subnormal results and inputs, infinities, NaN) take the conversion
-// instruction.
+// An FP64 instruction takes 64 cycles of a sub-partition's pipe per warp here, a
+// conversion from or to float twice that, also where a predicate turns it off;
+// FP32 and integer instructions take one or two. f2d is the same value moved
+// field by field without a branch.
 __device__ __forceinline__ double f2d(float f) {
-    const unsigned u = __float_as_uint(f), a = u & 0x7fffffffu;
-    if (a - 0x00800000u >= 0x7f000000u && a != 0u) return (double)f;
-    return __hiloint2double((int)((a ? (a >> 3) + 0x38000000u : 0u) | (u & 0x80000000u)), (int)(u << 29));
+    const unsigned a0 = __float_as_uint(f) & 0x7fffffffu;
+    const bool small = a0 < 0x00800000u;                          // zero or subnormal: scaled to a normal first
+    const unsigned u = __float_as_uint(small ? f * 0x1p64f : f), a = u & 0x7fffffffu;
+    unsigned off = small ? 0x38000000u - (64u << 20) : 0x38000000u;
+    off = a0 >= 0x7f800000u ? 0x70000000u : off;                  // infinity, NaN
+    return __hiloint2double((int)((a ? (a >> 3) + off : 0u) | (u & 0x80000000u)), (int)(u << 29));
 }
 
+// The nearest float, for results that are normal; else by the conversion, in a
+// call so that it is not predicated.
+static __device__ __noinline__ float d2f_rare(double d) { return (float)d; }
 __device__ __forceinline__ float d2f(double d) {
     const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
     const unsigned e = (hi >> 20) & 0x7ffu;
-    if (e - 897u >= 253u && ((hi << 1) | lo)) return (float)d;    // results from 2^-126 below 2^127: never overflows
+    if (e - 897u >= 253u && ((hi << 1) | lo)) return d2f_rare(d);   // else the result is in 2^-126 .. 2^127, or zero
     unsigned t = (__funnelshift_l(lo, hi, 3) - (896u << 23)) & 0x7fffffffu;
     const unsigned rest = lo << 3;                                // the 29 bits below the result's last
     t += rest > 0x80000000u || (rest == 0x80000000u && (t & 1u));

@@ -958,22 +958,12 @@ __global__ void SELL_BOUNDS k_spmv_dot(SellView S, const double* __restrict__ va
 template <typename TZ>
 __global__ void __launch_bounds__(TPB) k_update_p(int n, const TZ* __restrict__ z, double* __restrict__ p,
                                                   const PcgScalars* sc) {
-    dep_wait();
     const double beta = sc->beta;
-    const int stride = gridDim.x * blockDim.x;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += 4 * stride) {
-        TZ zv[4];
-        double pv[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-            if (i + u * stride < n) {
-                zv[u] = ldv(z + i + u * stride);
-                pv[u] = p[i + u * stride];
-            }
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-            if (i + u * stride < n) p[i + u * stride] = beta == 0.0 ? to_d(zv[u]) : fma(beta, pv[u], to_d(zv[u]));
-    }
+    if (beta == 0.0)
+        for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) p[i] = to_d(z[i]);
+    else
+        for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
+            p[i] = fma(beta, p[i], to_d(z[i]));
 }
 
 // x += alpha p; r -= alpha q; ||r||^2.
@@ -1757,8 +1747,8 @@ amg_status solve(amg_hierarchy* h, const double* b, double* x, double rtol, int 
         } else {
             {
                 Scope sc_(&h->prof, st, K_UPDATE_P, (zf ? 20.0 : 24.0) * n);
-                if (zf) launch_dep(k_update_p<float>, vec_grid(h, n), TPB, 0, st, n, z32, h->p, h->sc);
-                else launch_dep(k_update_p<double>, vec_grid(h, n), TPB, 0, st, n, h->z, h->p, h->sc);
+                if (zf) k_update_p<float><<<vec_grid(h, n), TPB, 0, st>>>(n, z32, h->p, h->sc);
+                else k_update_p<double><<<vec_grid(h, n), TPB, 0, st>>>(n, h->z, h->p, h->sc);
                 KERNEL_CHECK();
             }
             Scope sc_(&h->prof, st, K_SPMV_DOT, 12.0 * nnz + 16.0 * n);
