@@ -107,12 +107,16 @@ struct DevCsr {
 // would pad more than 30%, rows are sorted by length inside windows of 256
 // (SELL-C-sigma) and perm maps slice positions to rows.
 constexpr int SELL_C = 32;
+constexpr int SELL_SMALL = 32;               // slices per SM up to which a matrix is small (all resident in the solve)
+constexpr int SELL_NO_DELTA = 0x7fffffff;    // DevSell::delta: the lanes of this slice differ
 struct DevSell {
     int n = 0;
     int nslices = 0;
     int64_t padded = 0;
     int* sptr = nullptr;   // nslices + 1, in units of 32 entries
     int* perm = nullptr;   // row held by each slice position (SELL-C-sigma); null: identity
+    int* delta = nullptr;  // col - row shared by the 32 lanes of place k of slice s, at sptr[s] + k (SELL_NO_DELTA at
+                           // sptr[s]: they differ); null: not built
     int nlong = 0;         // hybrid layout only: rows kept out of the slices (read from the CSR)
     int* long_rows = nullptr;
     int* col = nullptr;
@@ -133,9 +137,9 @@ struct SweepRecord {
 struct Level {
     DevCsr A;
     DevSell S;                  // A_l in SELL-32 (PCG product, extra smoothing sweeps)
-    double* valm = nullptr;     // A_l M_l^{-1} values in S's layout (first pre-smoothing sweep)
+    double* valm = nullptr;     // -omega A_l M_l^{-1} values in S's layout (valm32: A_l M_l^{-1}), first pre-smoothing sweep
     float* valm32 = nullptr;
-    DevSell AP;                 // omega M_l^{-1} A_l P_l in SELL-32 (coarse-correction residual update)
+    DevSell AP;                 // P_l - omega M_l^{-1} A_l P_l in SELL-32 (FP32 cycles: omega M_l^{-1} A_l P_l)
     int64_t ap_nnz = 0;
     double* w = nullptr;        // smooth vector on this level
     double* minv = nullptr;     // l1-Jacobi inverse diagonal

@@ -340,6 +340,7 @@ __device__ __forceinline__ void colsum(double (&v)[NV][CPL], const Grp& g, int k
 }
 
 // ---------------------------------------------------------- V-cycle --------
+// x = omega M^-1 b, r = b - omega (A M^-1) b; valm = -omega A M^-1, in FP32 A M^-1.
 template <typename T, int CPL, bool VEC>
 __global__ void __launch_bounds__(TPB) bk_pre(SellV S, const T* __restrict__ valm, const T* __restrict__ minv, T omega,
                                               const T* __restrict__ B, T* __restrict__ X, T* __restrict__ R, int k, int ld,
@@ -349,22 +350,37 @@ __global__ void __launch_bounds__(TPB) bk_pre(SellV S, const T* __restrict__ val
     const int c0 = g.gl * CPL;
     if (c0 >= k) return;
     for (int ip = g.gw; ip < S.n; ip += g.ngroups) {
-        T acc[CPL];
+        if constexpr (sizeof(T) == 8) {
+            const int i = rowid(S, ip);
+            const size_t o = (size_t)i * ld + c0;
+            T bi[CPL], xo[CPL], ro[CPL];
+            ld_cols<VEC, CPL>(B + o, bi, k - c0);
 #pragma unroll
-        for (int m = 0; m < CPL; ++m) acc[m] = 0;
-        sell_row_k<VEC, CPL>(S, valm, ip, c0, k, B, ld, acc);
-        const int i = rowid(S, ip);
-        const T mi = omega * minv[i];
-        const size_t o = (size_t)i * ld + c0;
-        T bi[CPL], xo[CPL], ro[CPL];
-        ld_cols<VEC, CPL>(B + o, bi, k - c0);
+            for (int m = 0; m < CPL; ++m) ro[m] = bi[m];
+            sell_row_k<VEC, CPL>(S, valm, ip, c0, k, B, ld, ro);
+            const T mi = omega * minv[i];
 #pragma unroll
-        for (int m = 0; m < CPL; ++m) {
-            xo[m] = mi * bi[m];
-            ro[m] = fma(-omega, acc[m], bi[m]);
+            for (int m = 0; m < CPL; ++m) xo[m] = mi * bi[m];
+            st_cols<VEC, CPL>(X + o, xo, c0, k);
+            st_cols<VEC, CPL>(R + o, ro, c0, k);
+        } else {
+            T acc[CPL];
+#pragma unroll
+            for (int m = 0; m < CPL; ++m) acc[m] = 0;
+            sell_row_k<VEC, CPL>(S, valm, ip, c0, k, B, ld, acc);
+            const int i = rowid(S, ip);
+            const T mi = omega * minv[i];
+            const size_t o = (size_t)i * ld + c0;
+            T bi[CPL], xo[CPL], ro[CPL];
+            ld_cols<VEC, CPL>(B + o, bi, k - c0);
+#pragma unroll
+            for (int m = 0; m < CPL; ++m) {
+                xo[m] = mi * bi[m];
+                ro[m] = fma(-omega, acc[m], bi[m]);
+            }
+            st_cols<VEC, CPL>(X + o, xo, c0, k);
+            st_cols<VEC, CPL>(R + o, ro, c0, k);
         }
-        st_cols<VEC, CPL>(X + o, xo, c0, k);
-        st_cols<VEC, CPL>(R + o, ro, c0, k);
     }
 }
 
@@ -448,9 +464,8 @@ __device__ __forceinline__ void fin_rz(const BlockScalars& sc, int c, double rz,
     }
 }
 
-// out = x + P e + omega M^-1 r - (omega M^-1 A P) e (the stored A P values
-// carry the row scaling); on level 0 also r_cg . out and
-// (flexible CG) q . out per column.
+// out = x + omega M^-1 r + (P - omega M^-1 A P) e (FP64: the stored values are
+// those of the bracket; FP32: omega M^-1 A P, and P e from agg and p); on level 0 also r_cg . out and (flexible CG) q . out per column.
 template <typename T, typename TO, int CPL, bool DOT, bool VEC>
 __global__ void __launch_bounds__(TPB) bk_post(SellV SAP, const T* __restrict__ apval, const T* __restrict__ minv,
                                                T omega, const int* __restrict__ agg, const T* __restrict__ p,
@@ -466,24 +481,35 @@ __global__ void __launch_bounds__(TPB) bk_post(SellV SAP, const T* __restrict__ 
     for (int m = 0; m < CPL; ++m) d[0][m] = d[1][m] = 0.0;
     if (c0 < k) {
         for (int ip = g.gw; ip < SAP.n; ip += g.ngroups) {
-            T acc[CPL];
-#pragma unroll
-            for (int m = 0; m < CPL; ++m) acc[m] = 0;
-            sell_row_k<VEC, CPL>(SAP, apval, ip, c0, k, E, ld, acc);
             const int i = rowid(SAP, ip);
-            const int a = agg[i];
-            const T pi = p[i];
-            const T mi = omega * minv[i];
             const size_t o = (size_t)i * ld + c0;
-            T ev[CPL], xv[CPL], rv[CPL];
+            T acc[CPL], xv[CPL], rv[CPL];
             TO ov[CPL];
-            ld_cols<VEC, CPL>(E + (size_t)a * ld + c0, ev, k - c0);
-            ld_cols<VEC, CPL>(X + o, xv, k - c0);
-            ld_cols<VEC, CPL>(R + o, rv, k - c0);
+            if constexpr (sizeof(T) == 8) {
+                const T mi = omega * minv[i];
+                ld_cols<VEC, CPL>(X + o, xv, k - c0);
+                ld_cols<VEC, CPL>(R + o, rv, k - c0);
 #pragma unroll
-            for (int m = 0; m < CPL; ++m) {
-                const T y = fma(pi, ev[m], xv[m]);
-                ov[m] = (TO)(fma(mi, rv[m], y) - acc[m]);         // acc: rows of omega M^-1 A P
+                for (int m = 0; m < CPL; ++m) acc[m] = fma(mi, rv[m], xv[m]);
+                sell_row_k<VEC, CPL>(SAP, apval, ip, c0, k, E, ld, acc);
+#pragma unroll
+                for (int m = 0; m < CPL; ++m) ov[m] = (TO)acc[m];
+            } else {
+#pragma unroll
+                for (int m = 0; m < CPL; ++m) acc[m] = 0;
+                sell_row_k<VEC, CPL>(SAP, apval, ip, c0, k, E, ld, acc);
+                const int a = agg[i];
+                const T pi = p[i];
+                const T mi = omega * minv[i];
+                T ev[CPL];
+                ld_cols<VEC, CPL>(E + (size_t)a * ld + c0, ev, k - c0);
+                ld_cols<VEC, CPL>(X + o, xv, k - c0);
+                ld_cols<VEC, CPL>(R + o, rv, k - c0);
+#pragma unroll
+                for (int m = 0; m < CPL; ++m) {
+                    const T y = fma(pi, ev[m], xv[m]);
+                    ov[m] = (TO)(fma(mi, rv[m], y) - acc[m]);
+                }
             }
             st_cols<VEC, CPL>(Out + o, ov, c0, k);
             if (DOT) {

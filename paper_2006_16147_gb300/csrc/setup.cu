@@ -1469,30 +1469,98 @@ __global__ void k_sell_width(int n, int nslices, const int* __restrict__ ptr, co
     }
 }
 
+// Entries of the slices. With agg and p set, row i of P - X for the source X
+// (one entry p_i in column agg_i of P, which every row of X = M^{-1} A P holds).
+template <bool POST>
 __global__ void k_sell_fill(int n, int nslices, const int* __restrict__ ptr, const int* __restrict__ rlen,
                             const int* __restrict__ col, const double* __restrict__ val,
                             const int* __restrict__ sptr, const int* __restrict__ perm, int* __restrict__ scol,
-                            double* __restrict__ sval) {
+                            double* __restrict__ sval, const int* __restrict__ agg, const double* __restrict__ p) {
     for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < (long long)nslices * 32;
          t += (long long)gridDim.x * blockDim.x) {
         const int s = (int)(t >> 5), lane = (int)(t & 31);
         const int ip = (int)t;
         const int width = sptr[s + 1] - sptr[s];
         long long pos = (long long)sptr[s] * 32 + lane;
-        int len = 0, b = 0;
+        int len = 0, b = 0, ai = -1;
+        double pi = 0.0;
         if (ip < n) {
             const int i = perm ? perm[ip] : ip;
             b = ptr[i];
             len = src_len(ptr, rlen, i);
+            if (POST) {
+                ai = agg[i];
+                pi = p[i];
+            }
         }
         // padding repeats the row's last column (a valid index of this
         // matrix's column space, also for rectangular A P) with value 0
         const int pad = len > 0 ? col[b + len - 1] : 0;
         for (int k = 0; k < width; ++k, pos += 32) {
-            if (k < len) { scol[pos] = col[b + k]; sval[pos] = val[b + k]; }
-            else { scol[pos] = pad; sval[pos] = 0.0; }
+            if (k < len) {
+                const int c = col[b + k];
+                const double v = val[b + k];
+                scol[pos] = c;
+                sval[pos] = !POST ? v : (c == ai ? pi - v : -v);
+            } else { scol[pos] = pad; sval[pos] = 0.0; }
         }
     }
+}
+
+// The same for a square matrix in row order, with the entries of a slice lined
+// up by col - row where that needs no wider slice (a warp per slice: the
+// smallest difference left on any lane takes the next place; lanes without it
+// get a zero there). delta holds the differences of such a slice, and the row
+// products need no column indices there: a stencil's matrix is read as its
+// values alone. delta[sptr[s]] = SELL_NO_DELTA for the other slices. uniform
+// counts the places of lined-up slices.
+__global__ void __launch_bounds__(TPB) k_sell_fill_aligned(int n, int nslices, const int* __restrict__ ptr,
+                                                           const int* __restrict__ col, const double* __restrict__ val,
+                                                           const int* __restrict__ sptr, int* __restrict__ scol,
+                                                           double* __restrict__ sval, int* __restrict__ delta,
+                                                           int* __restrict__ uniform) {
+    const int lane = threadIdx.x & 31;
+    const int nw = (gridDim.x * blockDim.x) >> 5;
+    int found = 0;
+    for (int s = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; s < nslices; s += nw) {
+        const int i = s * 32 + lane, s0 = sptr[s], width = sptr[s + 1] - s0;
+        const int b = i < n ? ptr[i] : 0, len = i < n ? ptr[i + 1] - b : 0;
+        long long pos = (long long)s0 * 32 + lane;
+        int c = 0, places = 0;
+        if (s * 32 + 32 <= n)
+            for (;;) {
+                const int d = c < len ? col[b + c] - i : SELL_NO_DELTA;
+                const int m = __reduce_min_sync(FULL_MASK, d);
+                if (m == SELL_NO_DELTA || ++places > width) break;
+                c += d == m;
+            }
+        if (places == width && s * 32 + 32 <= n) {
+            bool shared = width > 0;
+            c = 0;
+            for (int k = 0; k < width; ++k, pos += 32) {
+                const int d = c < len ? col[b + c] - i : SELL_NO_DELTA;
+                const int m = __reduce_min_sync(FULL_MASK, d);
+                const bool take = d == m, in = i + m >= 0 && i + m < n;
+                const bool all = __all_sync(FULL_MASK, in);
+                shared = shared && all;
+                scol[pos] = in ? i + m : i;
+                sval[pos] = take ? val[b + c] : 0.0;
+                if (lane == 0) delta[s0 + k] = all ? m : SELL_NO_DELTA;
+                c += take;
+            }
+            if (!shared && width > 0 && lane == 0) delta[s0] = SELL_NO_DELTA;
+            if (shared && lane == 0) found += width;
+        } else {
+            const int pad = len > 0 ? col[b + len - 1] : 0;
+            for (int k = 0; k < width; ++k, pos += 32) {
+                scol[pos] = k < len ? col[b + k] : pad;
+                sval[pos] = k < len ? val[b + k] : 0.0;
+                if (lane == 0) delta[s0 + k] = SELL_NO_DELTA;
+            }
+        }
+    }
+    found = block_sum_int(found);
+    if (threadIdx.x == 0 && found) atomicAdd(uniform, found);
 }
 
 // SELL-C-sigma row order: inside each window of SIGMA consecutive rows, rows
@@ -1784,7 +1852,6 @@ __global__ void __launch_bounds__(DI_T) k_dense_inverse(int n, int r0, const int
     }
 }
 
-// Column scaling for the pre-smoother: valm_k = val_k * minv[col_k].
 // omega M^{-1} when omega != 1.
 __global__ void k_scale_vec(int n, double omega, const double* __restrict__ a, double* __restrict__ b,
                             float* __restrict__ b32) {
@@ -1795,11 +1862,12 @@ __global__ void k_scale_vec(int n, double omega, const double* __restrict__ a, d
     }
 }
 
-__global__ void k_scale_cols(long long m, const int* __restrict__ col, const double* __restrict__ val,
+// Pre-smoother values in A's layout: -omega A M^{-1}, in FP32 A M^{-1}.
+__global__ void k_scale_cols(long long m, double omega, const int* __restrict__ col, const double* __restrict__ val,
                              const double* __restrict__ minv, double* __restrict__ valm, float* __restrict__ valm32) {
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < m; k += (long long)gridDim.x * blockDim.x) {
         const double v = val[k] * minv[col[k]];
-        valm[k] = v;
+        valm[k] = -omega * v;
         if (valm32) valm32[k] = (float)v;
     }
 }
@@ -2912,9 +2980,13 @@ DevCsr galerkin_pairwise(amg_hierarchy* h, Scratch& S, const DevCsr& A, const Sw
 
 // SELL of A. With len set, row i of the source starts at A.ptr[i] and has
 // len[i] entries (A.nnz is then counted here); wtmp is the slice-width
-// scratch (S.ub when null).
+// scratch (S.ub when null). With agg and p set, P minus the source (k_sell_fill).
+// With `lined` set (a square A), a matrix of more than SELL_SMALL slices in row
+// order gets lined-up slices and E.delta; the places that share a difference
+// are counted in S.cnt[20], read with the setup's last synchronisation.
 void build_sell(amg_hierarchy* h, DevCsr A, DevSell& E, Scratch& S, bool fp32, const int* len = nullptr,
-                int* wtmp = nullptr, int64_t* nnz_out = nullptr) {
+                int* wtmp = nullptr, int64_t* nnz_out = nullptr, const int* agg = nullptr, const double* p = nullptr,
+                bool lined = false) {
     cudaStream_t st = h->stream;
     int* width = wtmp ? wtmp : S.ub;
     E.n = A.n;
@@ -2944,8 +3016,20 @@ void build_sell(amg_hierarchy* h, DevCsr A, DevSell& E, Scratch& S, bool fp32, c
     }
     E.col = h->mem.alloc<int>(E.padded);
     E.val = h->mem.alloc<double>(E.padded);
-    k_sell_fill<<<blocks_for((long long)E.nslices * 32, TPB, h->num_sms * 16), TPB, 0, st>>>(
-        A.n, E.nslices, A.ptr, len, A.col, A.val, E.sptr, E.perm, E.col, E.val);
+    const int fgrid = blocks_for((long long)E.nslices * 32, TPB, h->num_sms * 16);
+    if (lined && !E.perm && E.nslices > SELL_SMALL * h->num_sms) {
+        E.delta = h->mem.alloc<int>(E.padded / SELL_C);
+        CUDA_CHECK(cudaMemsetAsync(S.cnt + 20, 0, sizeof(int), st));
+        k_sell_fill_aligned<<<fgrid, TPB, 0, st>>>(A.n, E.nslices, A.ptr, A.col, A.val, E.sptr, E.col, E.val, E.delta,
+                                                   S.cnt + 20);
+    } else {
+        if (agg)
+            k_sell_fill<true><<<fgrid, TPB, 0, st>>>(A.n, E.nslices, A.ptr, len, A.col, A.val, E.sptr, E.perm, E.col,
+                                                     E.val, agg, p);
+        else
+            k_sell_fill<false><<<fgrid, TPB, 0, st>>>(A.n, E.nslices, A.ptr, len, A.col, A.val, E.sptr, E.perm, E.col,
+                                                      E.val, nullptr, nullptr);
+    }
     KERNEL_CHECK();
     if (fp32) {
         E.val32 = h->mem.alloc<float>(E.padded);
@@ -2994,25 +3078,26 @@ void build_sell_hybrid(amg_hierarchy* h, const DevCsr& A, DevSell& E, Scratch& S
     E.padded = (int64_t)read_int(E.sptr + E.nslices, S.host, st) * SELL_C;
     E.col = h->mem.alloc<int>(E.padded);
     E.val = h->mem.alloc<double>(E.padded);
-    k_sell_fill<<<wgrid, TPB, 0, st>>>(nshort, E.nslices, A.ptr, nullptr, A.col, A.val, E.sptr, E.perm, E.col,
-                                       E.val);
+    k_sell_fill<false><<<wgrid, TPB, 0, st>>>(nshort, E.nslices, A.ptr, nullptr, A.col, A.val, E.sptr, E.perm, E.col,
+                                       E.val, nullptr, nullptr);
     KERNEL_CHECK();
     S.mem.release(short_rows);
 }
 
-// Column-scaled values of A M^{-1} in A's SELL layout (padding stays 0).
+// The pre-smoother's values in A's SELL layout (padding stays 0).
 void build_scaled(amg_hierarchy* h, Level& L, bool fp32) {
     cudaStream_t st = h->stream;
     const long long m = L.S.padded;
     L.valm = h->mem.alloc<double>(m);
     if (fp32) L.valm32 = h->mem.alloc<float>(m);
-    k_scale_cols<<<blocks_for(m, TPB, h->num_sms * 16), TPB, 0, st>>>(m, L.S.col, L.S.val, L.minv, L.valm, L.valm32);
+    k_scale_cols<<<blocks_for(m, TPB, h->num_sms * 16), TPB, 0, st>>>(m, h->opt.omega, L.S.col, L.S.val, L.minv,
+                                                                   L.valm, L.valm32);
     KERNEL_CHECK();
 }
 
-// omega M_l^{-1} A_l P_l in SELL (rows of A_l scaled by omega / M_ii, columns
-// the aggregates of level l+1): the coarse-correction term of the fused
-// post-smoother needs no per-row scaling in the solve.
+// P_l - omega M_l^{-1} A_l P_l in SELL (rows of A_l scaled by omega / M_ii,
+// columns the aggregates of level l+1): the whole coarse-correction term of the
+// fused post-smoother. With FP32 cycles omega M_l^{-1} A_l P_l alone.
 void build_ap(amg_hierarchy* h, Level& L, int nc, Scratch& S, bool fp32) {
     cudaStream_t st = h->stream;
     const int n = L.A.n;
@@ -3030,7 +3115,7 @@ void build_ap(amg_hierarchy* h, Level& L, int nc, Scratch& S, bool fp32) {
     AP.ptr = L.A.ptr;
     AP.col = S.skey;
     AP.val = S.sval;
-    build_sell(h, AP, L.AP, S, fp32, S.ub, S.off, &L.ap_nnz);
+    build_sell(h, AP, L.AP, S, fp32, S.ub, S.off, &L.ap_nnz, fp32 ? nullptr : L.agg, L.p);
 }
 
 void build_members(amg_hierarchy* h, Level& L, int nc, Scratch& S) {
@@ -3577,7 +3662,8 @@ void setup_hierarchy(amg_hierarchy* h, const amg_csr* Ain, const double* w_in) {
         Scope sc_(&h->prof, st, S_FORMAT, 24.0 * L.A.nnz);
         const bool coarsest_cg = l == nlev - 1 && L.A.n > o.max_dense;
         if (coarsest_cg && l > 0) build_sell_hybrid(h, L.A, L.S, S);
-        else if (l == 0 || l < nlev - 1 || coarsest_cg) build_sell(h, L.A, L.S, S, fp32);
+        else if (l == 0 || l < nlev - 1 || coarsest_cg)
+            build_sell(h, L.A, L.S, S, fp32, nullptr, nullptr, nullptr, nullptr, nullptr, l == 0);
         if (l == nlev - 1) break;
         build_scaled(h, L, fp32);
         if (o.smooth_p) {
@@ -3663,7 +3749,13 @@ void setup_hierarchy(amg_hierarchy* h, const amg_csr* Ain, const double* w_in) {
         dense_inverse(h, D, Lc.A, 0, nc, h->coarse_inv, h->coarse_L);
         D.check(S, st, "coarsest-level Cholesky hit a non-positive pivot");
     }
+    DevSell& E0 = h->lev[0].S;
+    if (E0.delta) CUDA_CHECK(cudaMemcpyAsync(S.host, S.cnt + 20, sizeof(int), cudaMemcpyDeviceToHost, st));
     CUDA_CHECK(cudaStreamSynchronize(st));
+    if (E0.delta && 4LL * S.host[0] < 3 * (E0.padded / SELL_C)) {   // few shared differences: read the columns
+        h->mem.release(E0.delta);
+        E0.delta = nullptr;
+    }
     h->prof.flush();
     h->setup_ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
 }

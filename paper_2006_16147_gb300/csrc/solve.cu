@@ -3,7 +3,8 @@
 // Every level holds its matrix in SELL-32: one warp per 32-row slice, one
 // lane per row, entries of a slice stored column-major so that each step of
 // the row loop is one fully coalesced 128-byte (float) / 256-byte (double)
-// load of values and a 128-byte load of column indices.
+// load of values and a 128-byte load of column indices (none in a stencil's
+// lined-up slices).
 //
 // V-cycle for level l < L (input b_l, zero initial guess):
 //   pre-smooth + residual (fused):  x = omega M^-1 b;  r = b - A x
@@ -111,6 +112,7 @@ struct SellView {
     const int* __restrict__ sptr;
     const int* __restrict__ col;
     const int* __restrict__ perm;   // row held by slice position (null: identity)
+    const int* __restrict__ delta;  // col - row shared by a slice's lanes (null: read the columns)
 };
 
 // Row index held by SELL position ip (rows may be permuted by length).
@@ -129,12 +131,13 @@ __device__ __forceinline__ T ld(const T* p) { return __ldg(p); }
 //   RB = 4  the others, in 32 registers: with all 64 warps of an SM the FP64
 //           pipe and the memory work side by side; at half of them they take
 //           turns (256^3 level 0 with RB = 8: k_post 262 -> 452 us)
-// Two accumulators shorten the FMA chain (latency-bound kernels); one saves the
-// final add, which pays in the fused smoothers, where the FP64 pipe (this GPU's
+// The order of the additions is the same. Two accumulators (the second takes
+// every other entry of the full fours) shorten the FMA chain (latency-bound
+// kernels); one saves the final add, which pays in the fused smoothers, where the FP64 pipe (this GPU's
 // FP64 rate is 1/64 of its FP32 rate) is the bound.
 template <int RB, typename T>
 struct RowBatch {
-    int w;
+    int w, i;                       // entries, slice position
     long long base;
     int j[RB];
     T v[RB];
@@ -149,16 +152,58 @@ struct RowBatch {
     __device__ __forceinline__ void load(const SellView& S, const T* __restrict__ val, int s) {
         const int s0 = ld(S.sptr + s);
         w = ld(S.sptr + s + 1) - s0;
+        i = s * 32 + (threadIdx.x & 31);
         base = (long long)s0 * 32 + (threadIdx.x & 31);
         if (RB == 8) fetch(S.col, val, 0);
     }
-    template <int NACC = 2, typename F>
-    __device__ __forceinline__ T dot(const SellView& S, const T* __restrict__ val, F&& xv) {
-        T a0 = 0, a1 = 0;
+    template <int NACC = 2, bool DELTA = true, typename F>
+    __device__ __forceinline__ T dot(const SellView& S, const T* __restrict__ val, F&& xv, T init = T(0)) {
+        T a0 = init, a1 = 0;
         if constexpr (RB == 4) {
             const int* c = S.col + base;
             const T* a = val + base;
             int k = 0;
+            // a stencil's slice: columns from the differences its lanes share. FP32
+            // takes whole slices (192^3 solve 12.1 -> 11.7 ms; by places k_pre is as
+            // slow as with columns); in FP64, where the pipe is the bound, a test per
+            // place does better (256^3 k_pre with columns 363 us, by slices 295, by
+            // places 282; k_spmv_dot 314, 296, 299; a step 60.4 -> 57.9 ms)
+            const int* dl = S.delta + (base >> 5);
+            if (sizeof(T) == 4 && DELTA && S.delta && w > 0 && ld(dl) != SELL_NO_DELTA) {
+                for (; k + 4 <= w; k += 4, dl += 4, a += 128) {
+                    const int j0 = i + ld(dl), j1 = i + ld(dl + 1), j2 = i + ld(dl + 2), j3 = i + ld(dl + 3);
+                    const T v0 = ld(a), v1 = ld(a + 32), v2 = ld(a + 64), v3 = ld(a + 96);
+                    const T x0 = xv(j0), x1 = xv(j1), x2 = xv(j2), x3 = xv(j3);
+                    a0 = fma(v0, x0, a0);
+                    if (NACC == 1) a0 = fma(v1, x1, a0);
+                    else a1 = fma(v1, x1, a1);
+                    a0 = fma(v2, x2, a0);
+                    if (NACC == 1) a0 = fma(v3, x3, a0);
+                    else a1 = fma(v3, x3, a1);
+                }
+                for (; k < w; ++k, ++dl, a += 32) a0 = fma(ld(a), xv(i + ld(dl)), a0);
+                return NACC == 1 ? a0 : a0 + a1;
+            }
+            if (sizeof(T) == 8 && DELTA && S.delta) {
+                auto column = [&](int u) {
+                    const int d = ld(dl + u);
+                    return d != SELL_NO_DELTA ? i + d : ld(c + 32 * u);
+                };
+                for (; k + 4 <= w; k += 4, c += 128, a += 128, dl += 4) {
+                    const int j0 = column(0), j1 = column(1), j2 = column(2), j3 = column(3);
+                    const T v0 = ld(a), v1 = ld(a + 32), v2 = ld(a + 64), v3 = ld(a + 96);
+                    const T x0 = xv(j0), x1 = xv(j1), x2 = xv(j2), x3 = xv(j3);
+                    a0 = fma(v0, x0, a0);
+                    if (NACC == 1) a0 = fma(v1, x1, a0);
+                    else a1 = fma(v1, x1, a1);
+                    a0 = fma(v2, x2, a0);
+                    if (NACC == 1) a0 = fma(v3, x3, a0);
+                    else a1 = fma(v3, x3, a1);
+                }
+#pragma unroll 1
+                for (; k < w; ++k, c += 32, a += 32, ++dl) a0 = fma(ld(a), xv(column(0)), a0);
+                return NACC == 1 ? a0 : a0 + a1;
+            }
             for (; k + 4 <= w; k += 4, c += 128, a += 128) {
                 const int j0 = ld(c), j1 = ld(c + 32), j2 = ld(c + 64), j3 = ld(c + 96);
                 const T v0 = ld(a), v1 = ld(a + 32), v2 = ld(a + 64), v3 = ld(a + 96);
@@ -181,7 +226,7 @@ struct RowBatch {
 #pragma unroll
             for (int u = 0; u < RB; ++u)
                 if (k + u < w) {
-                    if (NACC == 1 || u % 2 == 0) a0 = fma(v[u], x[u], a0);
+                    if (NACC == 1 || u % 2 == 0 || k + u >= (w & ~3)) a0 = fma(v[u], x[u], a0);
                     else a1 = fma(v[u], x[u], a1);
                 }
             k += RB;
@@ -216,21 +261,21 @@ __device__ __forceinline__ double to_d(float v) { return f2d(v); }
 // --------------------------------------------------------- V-cycle ---------
 // First pre-smoothing sweep from a zero guess, fused with the residual:
 //   x = omega M^-1 b,  r = b - omega (A M^-1) b,
-// with the column-scaled values valm = A M^-1 (one FMA per stored entry) and
-// wm = omega M^-1. With U (one pre-smoothing sweep), x is not stored but
+// with the values valm = -omega A M^-1 (FP64: one FMA per stored entry, from b
+// on), resp. A M^-1 (FP32), and wm = omega M^-1. With U (one pre-smoothing sweep), x is not stored but
 // u = x + omega M^-1 r = omega M^-1 (b + r), the part of the post-smoother
 // that does not depend on the coarse correction.
 template <int RB, typename T, typename TB, bool U>
-__global__ void SELL_BOUNDS k_pre(SellView S, const T* __restrict__ valm, const T* __restrict__ wm,
-                                             T omega, const TB* __restrict__ b, T* __restrict__ x,
+__global__ void SELL_BOUNDS k_pre(SellView S, const T* __restrict__ valm, const T* __restrict__ wm, T omega,
+                                  const TB* __restrict__ b, T* __restrict__ x,
                                              T* __restrict__ r) {
     SELL_LOOP(S, T, valm) {
-        const T acc = row.template dot<1>(S, valm, [&](int j) { return (T)ldx<RB>(b + j); });
         const int ip = s * 32 + lane;
-        if (ip < S.n) {
-            const int i = sell_rowid(S, ip);
-            const T bi = (T)ldx<RB>(b + i);
-            const T ri = fma(-omega, acc, bi);
+        const int i = ip < S.n ? sell_rowid(S, ip) : -1;
+        const T bi = i >= 0 ? (T)ldx<RB>(b + i) : T(0);
+        const T acc = row.template dot<1>(S, valm, [&](int j) { return (T)ldx<RB>(b + j); }, sizeof(T) == 8 ? bi : T(0));
+        const T ri = sizeof(T) == 8 ? acc : fma(-omega, acc, bi);
+        if (i >= 0) {
             r[i] = ri;
             x[i] = U ? wm[i] * (bi + ri) : wm[i] * bi;
         }
@@ -283,29 +328,31 @@ __global__ void __launch_bounds__(TPB) k_restrict(int nc, const int* __restrict_
 
 // Coarse correction and first post-smoothing sweep, fused:
 //   y = x + P e,  out = y + omega M^-1 (b - A y),
-// evaluated as out = (x + omega M^-1 r) + P e - (omega M^-1 A P) e, since
-// b - A y = r - A P e with r = b - A x from the pre-smoother. The stored
-// apw = omega M^-1 A P has about half the entries of A and gathers only the
-// short coarse vector e. With U the first term u = x + omega M^-1 r comes
-// ready from the pre-smoother; otherwise it is formed here from x, r and
-// wm = omega M^-1. With DOT, also bdot . out (r . z of CG on level 0),
-// finished into the CG scalars. FP64 work per row: one FMA per entry of
-// apw, two more, and the dot.
+// evaluated as out = (x + omega M^-1 r) + (P - omega M^-1 A P) e, since
+// b - A y = r - A P e with r = b - A x from the pre-smoother. FP64 stores apw =
+// P - omega M^-1 A P, which has about half the entries of A and gathers only the
+// short coarse vector e: one FMA per entry and the dot, three FP64 instructions
+// and 12 bytes a row less than with P e apart (256^3 level 0 262 us, 215 now).
+// FP32 stores apw = omega M^-1 A P and takes P e from agg and p: rounding the
+// sum of the two to a float would be another preconditioner, and it gains
+// little. With U the first term u = x + omega M^-1 r comes ready from the
+// pre-smoother; otherwise it is formed here from x, r and wm = omega M^-1. With
+// DOT, also bdot . out (r . z of CG on level 0), finished into the CG scalars.
 template <int RB, typename T, typename TB, typename TO, bool DOT, bool U>
 __global__ void SELL_BOUNDS k_post(SellView SAP, const T* __restrict__ apw, const T* __restrict__ wm,
-                                              const int* __restrict__ agg, const T* __restrict__ p,
-                                              const T* __restrict__ e, const T* __restrict__ x,
-                                              const T* __restrict__ r, const TB* __restrict__ bdot,
-                                              TO* __restrict__ out, Reducer red, PcgScalars* sc, int mode,
-                                              const double* __restrict__ q2) {
+                                   const int* __restrict__ agg, const T* __restrict__ p, const T* __restrict__ e, const T* __restrict__ x, const T* __restrict__ r,
+                                   const TB* __restrict__ bdot, TO* __restrict__ out, Reducer red, PcgScalars* sc,
+                                   int mode, const double* __restrict__ q2) {
     double dot = 0.0, dot2 = 0.0;
     SELL_LOOP(SAP, T, apw) {
-        const T acc = row.template dot<1>(SAP, apw, [&](int q) { return ldx<RB>(e + q); });
         const int ip = s * 32 + lane;
-        if (ip < SAP.n) {
-            const int i = sell_rowid(SAP, ip);
-            const T ui = U ? ldx<RB>(x + i) : fma(wm[i], ldx<RB>(r + i), ldx<RB>(x + i));
-            const T o = fma(p[i], ldx<RB>(e + agg[i]), ui) - acc;
+        const int i = ip < SAP.n ? sell_rowid(SAP, ip) : -1;
+        T ui = 0;
+        if (i >= 0) ui = U ? ldx<RB>(x + i) : fma(wm[i], ldx<RB>(r + i), ldx<RB>(x + i));
+        const T acc = row.template dot<1, false>(SAP, apw, [&](int q) { return ldx<RB>(e + q); },
+                                                 sizeof(T) == 8 ? ui : T(0));
+        if (i >= 0) {
+            const T o = sizeof(T) == 8 ? acc : fma(p[i], ldx<RB>(e + agg[i]), ui) - acc;
             out[i] = (TO)o;
             if (DOT) {
                 const double od = to_d((TO)o);
@@ -322,7 +369,7 @@ __global__ void SELL_BOUNDS k_post(SellView SAP, const T* __restrict__ apw, cons
 
 // Whether all slices are resident at once with four blocks of the RB = 8
 // kernels per SM.
-bool sell_small(const amg_hierarchy* h, const SellView& S) { return S.nslices <= h->num_sms * 4 * WARPS; }
+bool sell_small(const amg_hierarchy* h, const SellView& S) { return S.nslices <= h->num_sms * SELL_SMALL; }
 // RB = 8 kernels begin beside the kernel before; for a large matrix that gains
 // nothing, and the compiler keeps its freedom with ld.nc.
 template <int RB, typename... P, typename... A>
@@ -382,7 +429,7 @@ __global__ void SELL_BOUNDS k_kc_spmv_dot(SellView S, const T* __restrict__ val,
                                                      KcScalars* ks) {
     double dq = 0.0, db = 0.0;
     SELL_LOOP(S, T, val) {
-        const T acc = row.dot(S, val, [&](int j) { return ldx<RB>(d1 + j); });
+        const T acc = row.template dot<2, false>(S, val, [&](int j) { return ldx<RB>(d1 + j); });
         const int ip = s * 32 + lane;
         if (ip < S.n) {
             const int i = sell_rowid(S, ip);
@@ -429,7 +476,7 @@ __global__ void SELL_BOUNDS k_kc_spmv2(SellView S, const T* __restrict__ val, co
     double dq = 0.0, dr = 0.0;
     SELL_LOOP(S, T, val) {
         const T be = (T)ks->beta;
-        const T acc = row.dot(S, val, [&](int j) { return ldx<RB>(z2 + j); });
+        const T acc = row.template dot<2, false>(S, val, [&](int j) { return ldx<RB>(z2 + j); });
         const int ip = s * 32 + lane;
         if (ip < S.n) {
             const int i = sell_rowid(S, ip);
@@ -528,7 +575,7 @@ template <int RB, typename T>
 __global__ void SELL_BOUNDS k_prolong(SellView S, const T* __restrict__ val, const T* __restrict__ e,
                                                  T* __restrict__ x) {
     SELL_LOOP(S, T, val) {
-        const T acc = row.dot(S, val, [&](int q) { return ldx<RB>(e + q); });
+        const T acc = row.template dot<2, false>(S, val, [&](int q) { return ldx<RB>(e + q); });
         const int ip = s * 32 + lane;
         if (ip < S.n) {
             const int i = sell_rowid(S, ip);
@@ -667,7 +714,8 @@ __device__ __forceinline__ void cg_partials(const double (&v)[NV], double* part,
 // and 1024 threads per SM instead of 512, one coarsest solve of 374K rows (30
 // iterations) takes 1.10 ms, 1.61 ms before; with two barriers an iteration
 // (the direction update inside the product), a row's loads together and hubs
-// kept out of the slices 1.01 ms. A third of that is the FP64 pipe.
+// kept out of the slices 1.01 ms, with eight lanes a hub 0.95 ms. A third of
+// that is the FP64 pipe.
 template <int NV, int NO, typename FIN>
 __device__ __forceinline__ void cg_sums(const double* part, int G, double (&out)[NO], FIN&& fin) {
     __shared__ double tot[NO];
@@ -750,31 +798,44 @@ __global__ void __launch_bounds__(CG_TPB, 1) k_coarse_cg(SellView S, const doubl
                 pq = fma(pi, acc, pq);
             };
             const int lane = threadIdx.x & 31, nw = G * (blockDim.x >> 5);
-            // long rows: one warp per row, straight from the CSR
-            for (int lr = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); lr < nlong; lr += nw) {
-                const int i = __ldg(long_rows + lr);
-                const Own o = own(i);
-                const int e = __ldg(cptr + i + 1);
-                double acc = 0.0;
-                for (int k = __ldg(cptr + i) + lane; k < e; k += 128) {
-                    int j[4];
-                    double v[4], zv[4];
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const bool ok = k + 32 * u < e;
-                        j[u] = ok ? __ldg(ccol + k + 32 * u) : -1;
-                        v[u] = ok ? __ldg(cval + k + 32 * u) : 0.0;
+            // tasks of a warp: four long rows straight from the CSR, eight lanes
+            // each (a warp per row spent five additions and three steps of one
+            // lane on every row), then slices
+            const int ntask = (nlong + 3) / 4 + S.nslices;
+            for (int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); t < ntask; t += nw) {
+                if (t < (nlong + 3) / 4) {
+                    const int lr = 4 * t + (lane >> 3);
+                    const int i = lr < nlong ? __ldg(long_rows + lr) : -1;
+                    Own o{};
+                    int k = 0, e = 0;
+                    if (i >= 0) {
+                        o = own(i);
+                        k = __ldg(cptr + i) + (lane & 7);
+                        e = __ldg(cptr + i + 1);
                     }
+                    double acc = 0.0;
+                    for (; k < e; k += 32) {
+                        int j[4];
+                        double v[4], zv[4];
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) zv[u] = j[u] >= 0 ? z[j[u]] : 0.0;
+                        for (int u = 0; u < 4; ++u) {
+                            const bool ok = k + 8 * u < e;
+                            j[u] = ok ? __ldg(ccol + k + 8 * u) : -1;
+                            v[u] = ok ? __ldg(cval + k + 8 * u) : 0.0;
+                        }
 #pragma unroll
-                    for (int u = 0; u < 4; ++u)
-                        if (j[u] >= 0) acc = fma(v[u], zv[u], acc);
+                        for (int u = 0; u < 4; ++u) zv[u] = j[u] >= 0 ? z[j[u]] : 0.0;
+#pragma unroll
+                        for (int u = 0; u < 4; ++u)
+                            if (j[u] >= 0) acc = fma(v[u], zv[u], acc);
+                    }
+                    __syncwarp();
+#pragma unroll
+                    for (int w = 4; w > 0; w >>= 1) acc += __shfl_xor_sync(FULL_MASK, acc, w);
+                    if (i >= 0 && (lane & 7) == 0) finish_row(i, o, acc);
+                    continue;
                 }
-                acc = warp_sum(acc);
-                if (lane == 0) finish_row(i, o, acc);
-            }
-            for (int sl = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); sl < S.nslices; sl += nw) {
+                const int sl = t - (nlong + 3) / 4;
                 const int ip = sl * 32 + lane;
                 const int i = ip < S.n ? sell_rowid(S, ip) : -1;
                 const int s0 = __ldg(S.sptr + sl), w = __ldg(S.sptr + sl + 1) - s0;
@@ -988,20 +1049,22 @@ __global__ void __launch_bounds__(TPB) k_update_xr(int n, const double* __restri
 // ------------------------------------------------------------ host ---------
 // Algorithmic bytes of one launch: every array the kernel must touch, read
 // or written once (index 4 B, value V B, the level-0 input/output in FP64);
-// matrix entries counted without SELL padding.
-double by_pre(const Level& L, int V, int Vb) { return (double)L.A.nnz * (V + 4) + (double)L.A.n * (Vb + 3.0 * V); }
-// post: omega M^-1 A P entries + u, p (V) [x, r, omega M^-1 instead of u without
-// the fused u: 3V] + agg (4) + out (Vo) [+ CG r for the dot] + e (n_c)
+// matrix entries counted without SELL padding, lined-up slices with one index
+// per 32 entries.
+double by_index(const Level& L) { return L.S.delta ? 0.125 : 4.0; }
+double by_pre(const Level& L, int V, int Vb) { return (double)L.A.nnz * (V + by_index(L)) + (double)L.A.n * (Vb + 3.0 * V); }
+// post: P - omega M^-1 A P entries + u (V) [x, r, omega M^-1 instead of u without
+// the fused u: 3V] + p, agg (FP32: 8) + out (Vo) [+ CG r for the dot] + e (n_c)
 double by_post2(const Level& L, int nc, int V, int Vo, bool dot, bool u) {
-    return (double)L.ap_nnz * (V + 4) + (double)L.A.n * ((u ? 2.0 : 4.0) * V + 4 + Vo + (dot ? 8 : 0)) +
+    return (double)L.ap_nnz * (V + 4) + (double)L.A.n * ((u ? 1.0 : 3.0) * V + (V == 4 ? 8 : 0) + Vo + (dot ? 8 : 0)) +
            (double)nc * V;
 }
-double by_resid(const Level& L, int V, int Vb) { return (double)L.A.nnz * (V + 4) + (double)L.A.n * (Vb + 2.0 * V); }
+double by_resid(const Level& L, int V, int Vb) { return (double)L.A.nnz * (V + by_index(L)) + (double)L.A.n * (Vb + 2.0 * V); }
 double by_restrict(int n, int nc, int V) { return (double)n * (4 + 2.0 * V) + (double)nc * (4 + V); }
-double by_smooth(const Level& L, int V, int Vb, int Vo) { return (double)L.A.nnz * (V + 4) + (double)L.A.n * (2.0 * V + Vb + Vo); }
+double by_smooth(const Level& L, int V, int Vb, int Vo) { return (double)L.A.nnz * (V + by_index(L)) + (double)L.A.n * (2.0 * V + Vb + Vo); }
 double by_coarse(int nc, int Vi, int Vo) { return 8.0 * nc * nc + (double)nc * (Vi + Vo); }
 
-SellView view(const Level& L) { return SellView{L.S.n, L.S.nslices, L.S.sptr, L.S.col, L.S.perm}; }
+SellView view(const Level& L) { return SellView{L.S.n, L.S.nslices, L.S.sptr, L.S.col, L.S.perm, L.S.delta}; }
 
 int sell_grid(const amg_hierarchy* h, int nslices) {
     int g = (nslices + WARPS - 1) / WARPS;
@@ -1041,7 +1104,7 @@ void coarse_solve_launch(amg_hierarchy* h, const void* b, void* x, bool fp32_in,
         CoarseCg& C = h->ccg;
         Scope sc_(&h->prof, h->stream, K_COARSE, 8.0 * 30 * (3.0 * Lc.A.nnz + 10.0 * n));
         CUDA_CHECK(cudaMemsetAsync(C.ctl, 0, sizeof(int) * 4, h->stream));
-        SellView S{Lc.S.n, Lc.S.nslices, Lc.S.sptr, Lc.S.col, Lc.S.perm};
+        SellView S{Lc.S.n, Lc.S.nslices, Lc.S.sptr, Lc.S.col, Lc.S.perm, nullptr};
         const double* val = Lc.S.val;
         int nrows = Lc.A.n;
         int nlong = Lc.S.nlong;
@@ -1175,7 +1238,7 @@ void vcycle_typed(amg_hierarchy* h, const double* r, TZ* z, int rz_mode) {
         spare[l] = (xa == vec(Lv, VX)) ? vec(Lv, VT) : vec(Lv, VX);
         const int nc = h->lev[l + 1].A.n;
         if (SA) {
-            const SellView SPT{Lv.PBT.n, Lv.PBT.nslices, Lv.PBT.sptr, Lv.PBT.col, Lv.PBT.perm};
+            const SellView SPT{Lv.PBT.n, Lv.PBT.nslices, Lv.PBT.sptr, Lv.PBT.col, Lv.PBT.perm, nullptr};
             Scope sc_(&h->prof, st, K_RESTRICT, (double)Lv.pbar_t.nnz * (V + 4) + (double)(Lv.A.n + nc) * V);
             if (!f32 && wide(Lv.pbar_t, WIDE_MIN_P))
                 launch_dep(k_wide<W_SPMV>, wide_grid(h, nc), TPB, 0, st, nc, Lv.pbar_t.ptr, Lv.pbar_t.col, Lv.pbar_t.val,
@@ -1199,13 +1262,13 @@ void vcycle_typed(amg_hierarchy* h, const double* r, TZ* z, int rz_mode) {
     for (int l = L - 1; l >= 0; --l) {
         Level& Lv = h->lev[l];
         const SellView S = view(Lv);
-        const SellView SAP{Lv.AP.n, Lv.AP.nslices, Lv.AP.sptr, Lv.AP.col, Lv.AP.perm};
+        const SellView SAP{Lv.AP.n, Lv.AP.nslices, Lv.AP.sptr, Lv.AP.col, Lv.AP.perm, nullptr};
         const int g = Lv.grid_post[f32] ? Lv.grid_post[f32] : sell_grid(h, S.nslices);
         const T* e = out[l + 1];
         const int nc = h->lev[l + 1].A.n;
         if (SA) {
             // x <- x + Pbar e, then one l1-Jacobi sweep on A (the unfused post-smoother)
-            const SellView SPB{Lv.PB.n, Lv.PB.nslices, Lv.PB.sptr, Lv.PB.col, Lv.PB.perm};
+            const SellView SPB{Lv.PB.n, Lv.PB.nslices, Lv.PB.sptr, Lv.PB.col, Lv.PB.perm, nullptr};
             {
                 Scope sc_(&h->prof, st, l == 0 ? K_POST_L0 : K_POST,
                           (double)Lv.pbar.nnz * (V + 4) + 2.0 * Lv.A.n * V + (double)nc * V);
@@ -1352,7 +1415,7 @@ void kc_apply(amg_hierarchy* h, int l, const T* in, T* out) {
     Level& Ln = h->lev[l + 1];
     const LevelOps<T> O(Lv);
     const SellView S = view(Lv);
-    const SellView SAP{Lv.AP.n, Lv.AP.nslices, Lv.AP.sptr, Lv.AP.col, Lv.AP.perm};
+    const SellView SAP{Lv.AP.n, Lv.AP.nslices, Lv.AP.sptr, Lv.AP.col, Lv.AP.perm, nullptr};
     const int V = sizeof(T), nc = Ln.A.n;
     const T omega = (T)h->opt.omega;
     T* xa = lvec<T>(Lv, 1);
@@ -1442,7 +1505,7 @@ void kcycle_typed(amg_hierarchy* h, const double* r, TZ* z, int rz_mode) {
     Level& L1 = h->lev[1];
     const LevelOps<T> O(L0);
     const SellView S = view(L0);
-    const SellView SAP{L0.AP.n, L0.AP.nslices, L0.AP.sptr, L0.AP.col, L0.AP.perm};
+    const SellView SAP{L0.AP.n, L0.AP.nslices, L0.AP.sptr, L0.AP.col, L0.AP.perm, nullptr};
     const int V = sizeof(T), n0 = L0.A.n, nc = L1.A.n;
     const T omega = (T)h->opt.omega;
     T* xa = lvec<T>(L0, 1);
@@ -1553,7 +1616,7 @@ void autotune_levels(amg_hierarchy* h) {
         Level& Lv = h->lev[l];
         Level& Ln = h->lev[l + 1];
         const SellView S = view(Lv);
-        const SellView SAP{Lv.AP.n, Lv.AP.nslices, Lv.AP.sptr, Lv.AP.col, Lv.AP.perm};
+        const SellView SAP{Lv.AP.n, Lv.AP.nslices, Lv.AP.sptr, Lv.AP.col, Lv.AP.perm, nullptr};
         const T* valm = f32 ? (const T*)Lv.valm32 : (const T*)Lv.valm;
         const T* apv = f32 ? (const T*)Lv.AP.val32 : (const T*)Lv.AP.val;
         const T* wm = f32 ? (const T*)Lv.wminv32 : (const T*)Lv.wminv;
@@ -1676,6 +1739,20 @@ void vcycle_plain(amg_hierarchy* h, const double* r, double* z) {
     else cycle_typed<double, double>(h, r, z, FIN_NONE);
 }
 
+void level0_product(amg_hierarchy* h, const double* x, double* y) {
+    const SellView S = view(h->lev[0]);
+    SELL_DISPATCH(h, S, launch_sell<RB>(k_sell_spmv<RB, double>, sell_grid(h, S.nslices), h->stream, S,
+                                        (const double*)h->lev[0].S.val, x, y));
+    KERNEL_CHECK();
+}
+
+void level0_residual(amg_hierarchy* h, const double* b, const double* x, double* r) {
+    const SellView S = view(h->lev[0]);
+    SELL_DISPATCH(h, S, launch_sell<RB>(k_resid<RB, double, double>, sell_grid(h, S.nslices), h->stream, S,
+                                        (const double*)h->lev[0].S.val, b, x, r));
+    KERNEL_CHECK();
+}
+
 void vcycle_apply(amg_hierarchy* h, const double* r, double* z) {
     vcycle_plain(h, r, z);
     CUDA_CHECK(cudaStreamSynchronize(h->stream));
@@ -1692,7 +1769,7 @@ amg_status solve(amg_hierarchy* h, const double* b, double* x, double rtol, int 
     PcgScalars* hs = h->sc_host;
 
     const double nnz = (double)L0.A.nnz;
-    const double by_res = 12.0 * nnz + 24.0 * n;
+    const double by_mat = (8.0 + by_index(L0)) * nnz, by_res = by_mat + 24.0 * n;
     const bool zf = float_z(h);
     CUDA_CHECK(cudaMemsetAsync(h->sc, 0, sizeof(PcgScalars), st));
     {
@@ -1738,7 +1815,7 @@ amg_status solve(amg_hierarchy* h, const double* b, double* x, double rtol, int 
         }
         const float* z32 = reinterpret_cast<const float*>(h->z);
         if (sell_small(h, S)) {
-            Scope sc_(&h->prof, st, K_SPMV_DOT, 12.0 * nnz + (zf ? 36.0 : 40.0) * n);
+            Scope sc_(&h->prof, st, K_SPMV_DOT, by_mat + (zf ? 36.0 : 40.0) * n);
             if (zf)
                 launch_sell<8>(k_direction<8, float>, red_grid(h, S.nslices), st, S, A, z32, h->p, h->q, h->red, h->sc);
             else
@@ -1751,7 +1828,7 @@ amg_status solve(amg_hierarchy* h, const double* b, double* x, double rtol, int 
                 else k_update_p<double><<<vec_grid(h, n), TPB, 0, st>>>(n, h->z, h->p, h->sc);
                 KERNEL_CHECK();
             }
-            Scope sc_(&h->prof, st, K_SPMV_DOT, 12.0 * nnz + 16.0 * n);
+            Scope sc_(&h->prof, st, K_SPMV_DOT, by_mat + 16.0 * n);
             launch_sell<4>(k_spmv_dot<4>, red_grid(h, S.nslices), st, S, A, h->p, h->q, h->red, h->sc);
             KERNEL_CHECK();
         }
