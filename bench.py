@@ -86,18 +86,18 @@ def _args():
 # valid for the 7-point Poisson workload in FP64 and only while the kernel
 # source it was taken on is unchanged (checked by hash).
 _TRAFFIC = {
-    "post_smooth_l0": {"kernel": "k_post", "bytes_per_row": (314713600 + 22986240) / 4096000},
-    "pre_residual_l0": {"kernel": "k_pre", "bytes_per_row": (408948992 + 53501184) / 4096000},
+    "post_smooth_l0": {"kernel": "k_post", "bytes_per_row": (267579648 + 23638272) / 4096000},
+    "pre_residual_l0": {"kernel": "k_pre", "bytes_per_row": (298250752 + 50765824) / 4096000},
 }
-_TRAFFIC_SRC_HASH = "e5fe5e8b08565c47"
+_TRAFFIC_SRC_HASH = "a06695819099df22"
 
 
 def _kernel_source_hash(names):
-    """sha256 (16 hex) of the named kernels' and sell_row's source in solve.cu."""
+    """sha256 (16 hex) of the named kernels' and the row product's source in solve.cu."""
     import hashlib
     lines = open(os.path.join(ROOT, "paper_2006_16147_gb300", "csrc", "solve.cu")).read().splitlines()
     parts = []
-    for name in list(names) + ["sell_row"]:
+    for name in list(names) + ["dot"]:
         for i, line in enumerate(lines):
             if f" {name}(" in line and ("__global__" in line or "__device__" in line):
                 j = i
