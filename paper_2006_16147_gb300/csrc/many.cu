@@ -276,6 +276,9 @@ amg_status solve_many(amg_hierarchy* h, const double* b, double* x, double rtol,
     const int flexible = h->opt.krylov == 1;
     const int vgrid = blocks_for(n, TPB, h->num_sms * 8);
     double *r = h->r, *z = h->z, *p = h->p, *q = h->q, *t = h->t;
+    // a system that is done before its first step never gets a direction, but
+    // the product reads p of every system
+    CUDA_CHECK(cudaMemsetAsync(p, 0, sizeof(double) * n, st));
 
     // r = b - A x0, per-system norms
     level0_residual(h, b, x, r);
