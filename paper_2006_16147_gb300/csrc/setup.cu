@@ -1513,12 +1513,15 @@ __global__ void k_sell_fill(int n, int nslices, const int* __restrict__ ptr, con
 // get a zero there). delta holds the differences of such a slice, and the row
 // products need no column indices there: a stencil's matrix is read as its
 // values alone. delta[sptr[s]] = SELL_NO_DELTA for the other slices. uniform
-// counts the places of lined-up slices.
+// counts the places of lined-up slices. A place that would take a lane out of
+// the matrix, or in a batch (sys set: system of each row) out of its row's
+// system, is not shared: that lane's zero stands at its own column, as 0 times
+// another system's infinity or NaN is NaN.
 __global__ void __launch_bounds__(TPB) k_sell_fill_aligned(int n, int nslices, const int* __restrict__ ptr,
                                                            const int* __restrict__ col, const double* __restrict__ val,
                                                            const int* __restrict__ sptr, int* __restrict__ scol,
                                                            double* __restrict__ sval, int* __restrict__ delta,
-                                                           int* __restrict__ uniform) {
+                                                           int* __restrict__ uniform, const int* __restrict__ sys) {
     const int lane = threadIdx.x & 31;
     const int nw = (gridDim.x * blockDim.x) >> 5;
     int found = 0;
@@ -1540,7 +1543,7 @@ __global__ void __launch_bounds__(TPB) k_sell_fill_aligned(int n, int nslices, c
             for (int k = 0; k < width; ++k, pos += 32) {
                 const int d = c < len ? col[b + c] - i : SELL_NO_DELTA;
                 const int m = __reduce_min_sync(FULL_MASK, d);
-                const bool take = d == m, in = i + m >= 0 && i + m < n;
+                const bool take = d == m, in = i + m >= 0 && i + m < n && (!sys || sys[i + m] == sys[i]);
                 const bool all = __all_sync(FULL_MASK, in);
                 shared = shared && all;
                 scol[pos] = in ? i + m : i;
@@ -2981,12 +2984,13 @@ DevCsr galerkin_pairwise(amg_hierarchy* h, Scratch& S, const DevCsr& A, const Sw
 // SELL of A. With len set, row i of the source starts at A.ptr[i] and has
 // len[i] entries (A.nnz is then counted here); wtmp is the slice-width
 // scratch (S.ub when null). With agg and p set, P minus the source (k_sell_fill).
-// With `lined` set (a square A), a matrix of more than SELL_SMALL slices in row
-// order gets lined-up slices and E.delta; the places that share a difference
-// are counted in S.cnt[20], read with the setup's last synchronisation.
+// With `lined` set (a square A; sys: system of each row of a batch, or null), a
+// matrix of more than SELL_SMALL slices per SM in row order gets lined-up slices
+// and E.delta; the places that share a difference are counted in S.cnt[20], read
+// with the setup's last synchronisation.
 void build_sell(amg_hierarchy* h, DevCsr A, DevSell& E, Scratch& S, bool fp32, const int* len = nullptr,
                 int* wtmp = nullptr, int64_t* nnz_out = nullptr, const int* agg = nullptr, const double* p = nullptr,
-                bool lined = false) {
+                bool lined = false, const int* sys = nullptr) {
     cudaStream_t st = h->stream;
     int* width = wtmp ? wtmp : S.ub;
     E.n = A.n;
@@ -3021,7 +3025,7 @@ void build_sell(amg_hierarchy* h, DevCsr A, DevSell& E, Scratch& S, bool fp32, c
         E.delta = h->mem.alloc<int>(E.padded / SELL_C);
         CUDA_CHECK(cudaMemsetAsync(S.cnt + 20, 0, sizeof(int), st));
         k_sell_fill_aligned<<<fgrid, TPB, 0, st>>>(A.n, E.nslices, A.ptr, A.col, A.val, E.sptr, E.col, E.val, E.delta,
-                                                   S.cnt + 20);
+                                                   S.cnt + 20, sys);
     } else {
         if (agg)
             k_sell_fill<true><<<fgrid, TPB, 0, st>>>(A.n, E.nslices, A.ptr, len, A.col, A.val, E.sptr, E.perm, E.col,
@@ -3663,7 +3667,8 @@ void setup_hierarchy(amg_hierarchy* h, const amg_csr* Ain, const double* w_in) {
         const bool coarsest_cg = l == nlev - 1 && L.A.n > o.max_dense;
         if (coarsest_cg && l > 0) build_sell_hybrid(h, L.A, L.S, S);
         else if (l == 0 || l < nlev - 1 || coarsest_cg)
-            build_sell(h, L.A, L.S, S, fp32, nullptr, nullptr, nullptr, nullptr, nullptr, l == 0);
+            build_sell(h, L.A, L.S, S, fp32, nullptr, nullptr, nullptr, nullptr, nullptr, l == 0,
+                       h->seg_row0);
         if (l == nlev - 1) break;
         build_scaled(h, L, fp32);
         if (o.smooth_p) {

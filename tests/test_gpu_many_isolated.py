@@ -1,7 +1,8 @@
 """Batches above the size at which level 0's slices are lined up (32 slices per
-SM): a system with a right-hand side of zeros, which takes no step, changes no
-bit of the others, whatever an earlier solve left in the kept vectors. The
-reference is the same batch with finite right-hand sides in every system."""
+SM): a system with a right-hand side of zeros, which takes no step, or with one
+that holds a NaN changes no bit of the others, whatever an earlier solve left in
+the kept vectors. The reference is the same batch with finite right-hand sides
+in every system."""
 import numpy as np
 import pytest
 
@@ -9,7 +10,7 @@ from gpu_util import dev
 from paper_2006_16147_gb300 import workloads as W
 
 pytestmark = pytest.mark.gpu
-ODD = 12                                     # the system with zeros
+ODD = 12                                     # the system with zeros or a NaN
 
 
 def batch(kind):
@@ -68,5 +69,29 @@ def test_zero_right_hand_side(kind, precision):
     st, x1, it1 = solve(h, b, m)
     h.close()
     assert st == 0 and it1[ODD] == 0 and not x1[offs[ODD]:offs[ODD + 1]].any()
+    assert it0[:ODD] + it0[ODD + 1:] == it1[:ODD] + it1[ODD + 1:]
+    assert same_elsewhere(offs, x1, x0)
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("kind", ["boxes", "mixed"])
+@pytest.mark.parametrize("row", [0, -1])
+def test_right_hand_side_with_nan(kind, precision, row):
+    import torch
+    from paper_2006_16147_gb300 import amg
+    mats, offs = batch(kind)
+    m = len(mats)
+    b = W.rhs_normal(offs[-1], 4)
+    h = setup(mats, precision)
+    st, x0, it0 = solve(h, b, m)
+    assert st == 0
+    z = [torch.empty(len(b), dtype=torch.float64, device="cuda:0") for _ in range(2)]
+    amg.amg_vcycle(h, dev(b), z[0])
+    b[offs[ODD] if row == 0 else offs[ODD + 1] - 1] = np.nan
+    amg.amg_vcycle(h, dev(b), z[1])
+    assert same_elsewhere(offs, z[1].cpu().numpy(), z[0].cpu().numpy())
+    st, x1, it1 = solve(h, b, m)
+    h.close()
+    assert st == amg.AMG_ERR_BREAKDOWN                       # of that system alone
     assert it0[:ODD] + it0[ODD + 1:] == it1[:ODD] + it1[ODD + 1:]
     assert same_elsewhere(offs, x1, x0)
