@@ -228,6 +228,10 @@ __device__ __forceinline__ void sell_row_split(const SellV& S, const double* __r
     for (int m = 0; m < CPL; ++m) {
         acc[m] = sum[m].value();
         if (on[m] && !sum[m].ok()) {
+            if (sum[m].ok_far()) {
+                acc[m] = sum[m].value_far();
+                continue;
+            }
             double t = 0.0;
             for (int e = 0; e < w; ++e)
                 t = fma(__ldg(val + base + 32 * e),

@@ -138,15 +138,16 @@ __device__ __forceinline__ float d2f(double d) {
     return __uint_as_float((e ? t : 0u) | (hi & 0x80000000u));
 }
 
-// A double of magnitude 2^-80 .. 2^127 as three floats, exactly: 24, 23 and 6
-// bits of its mantissa. Anything else but zero gives NaN.
+// A double of magnitude 2^-104 .. 2^103 times 2^SPLIT_UP as three floats,
+// exactly: 24, 23 and 6 bits of its mantissa. Anything else but zero gives NaN.
+constexpr unsigned SPLIT_UP = 24;
 struct Split3 {
     float h, m, l;
     bool one;         // the double is a float: m = l = 0
 };
 __device__ __forceinline__ Split3 split3(double a) {
     const unsigned hi = (unsigned)__double2hiint(a), lo = (unsigned)__double2loint(a);
-    const unsigned sgn = hi & 0x80000000u, t = (__funnelshift_l(lo, hi, 3) - (896u << 23)) & 0x7fffffffu;
+    const unsigned sgn = hi & 0x80000000u, t = (__funnelshift_l(lo, hi, 3) - ((896u - SPLIT_UP) << 23)) & 0x7fffffffu;
     const unsigned rest = lo & 0x1fffffffu;
     Split3 s{__uint_as_float(t | sgn), 0.0f, 0.0f, rest == 0u};
     if (rest) {
@@ -154,7 +155,7 @@ __device__ __forceinline__ Split3 split3(double a) {
         s.m = __uint_as_float(em | (rest >> 6)) - __uint_as_float(em);
         s.l = __uint_as_float(el | ((rest & 63u) << 17)) - __uint_as_float(el);
     }
-    if (((hi >> 20) & 0x7ffu) - 943u > 207u) s.h = ((hi << 1) | lo) ? __uint_as_float(0x7fc00000u) : 0.0f;
+    if (((hi >> 20) & 0x7ffu) - (943u - SPLIT_UP) > 207u) s.h = ((hi << 1) | lo) ? __uint_as_float(0x7fc00000u) : 0.0f;
     return s;
 }
 
@@ -163,8 +164,15 @@ __device__ __forceinline__ Split3 split3(double a) {
 // by fma, Knuth's two-sum), what those leave, 2^-46 of the largest product and
 // below, into s3. value() rounds twice in FP64, so the sum is nearer than a
 // chain of FP64 FMAs, as long as ok(): the largest product lies in
-// 2^-60 .. 2^120 and nothing was infinite or NaN (else the caller takes the
-// FP64 chain).
+// 2^-84 .. 2^96 and nothing was infinite or NaN. The pieces stand 2^SPLIT_UP
+// higher, which puts that window in the middle of a float's exponents. Where the
+// largest product lies in 2^-112 .. 2^103, ok_far(), the pieces hold the sum too,
+// but for parts below a float's last bit, 2^-57 of that product and 2^-60 more
+// per entry; value_far() takes some ten instructions more to move them into a
+// double, which every row would pay for in value() (a solve of 112^3 rows x 64
+// columns 140 ms, 144 ms with them). Beyond, the caller takes the FP64 chain after
+// the pieces: with right-hand sides scaled by 2^-70 that solve took 209 ms while
+// the window ended at 2^-60, 143 ms now.
 struct SplitSum {
     float s1 = 0.0f, s2 = 0.0f, s3 = 0.0f, big = 0.0f;
     static __device__ __forceinline__ float two_sum(float& s, float x) {
@@ -189,13 +197,21 @@ struct SplitSum {
     __device__ __forceinline__ bool ok() const {
         return big >= 0x1p-60f && big <= 0x1p120f && fabsf(s1) <= 0x1p126f;   // false for NaN
     }
-    // as f2d, with magnitudes below 2^-126 (2^-66 of the largest product) taken as zero
+    // f 2^-SPLIT_UP field by field as in f2d, from f 2^UP, whose magnitudes below 2^-126 are taken as zero
+    template <unsigned UP>
     static __device__ __forceinline__ double wide(float f) {
-        const unsigned u = __float_as_uint(f), a = u & 0x7fffffffu;
-        return a < 0x00800000u ? 0.0
-                               : __hiloint2double((int)((a >> 3) + 0x38000000u | (u & 0x80000000u)), (int)(u << 29));
+        const unsigned u = __float_as_uint(UP ? f * (float)(1u << UP) : f), a = u & 0x7fffffffu;
+        constexpr unsigned off = 0x38000000u - ((UP + SPLIT_UP) << 20);
+        return a < 0x00800000u ? 0.0 : __hiloint2double((int)((a >> 3) + off | (u & 0x80000000u)), (int)(u << 29));
     }
-    __device__ __forceinline__ double value() const { return wide(s1) + (wide(s2) + wide(s3)); }
+    __device__ __forceinline__ double value() const { return wide<0>(s1) + (wide<0>(s2) + wide<0>(s3)); }
+    // s2 and s3 keep below infinity when scaled up; a sum that overflowed on the way stays infinite or NaN in s1
+    __device__ __forceinline__ bool ok_far() const {
+        return big >= 0x1p-88f && fabsf(s1) <= 0x1.fffffep127f && fabsf(s2) + fabsf(s3) <= 0x1p107f;
+    }
+    __device__ __forceinline__ double value_far() const {
+        return (fabsf(s1) < 0x1p-100f ? wide<20>(s1) : wide<0>(s1)) + (wide<20>(s2) + wide<20>(s3));
+    }
 };
 
 // Block-wide exclusive scan of ints.
