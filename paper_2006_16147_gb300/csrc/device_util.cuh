@@ -167,7 +167,7 @@ __device__ __forceinline__ Split3 split3(double a) {
 // 2^-84 .. 2^96 and nothing was infinite or NaN. The pieces stand 2^SPLIT_UP
 // higher, which puts that window in the middle of a float's exponents. Where the
 // largest product lies in 2^-112 .. 2^103, ok_far(), the pieces hold the sum too,
-// but for parts below a float's last bit, 2^-57 of that product and 2^-60 more
+// but for parts below a float's last bit, 2^-56 of that product and 2^-60 more
 // per entry; value_far() takes some ten instructions more to move them into a
 // double, which every row would pay for in value() (a solve of 112^3 rows x 64
 // columns 140 ms, 144 ms with them). Beyond, the caller takes the FP64 chain after

@@ -1143,7 +1143,7 @@ void coarse_solve_launch(amg_hierarchy* h, const void* b, void* x, bool fp32_in,
 // FIN_NONE, also finishes r . z. A single level (the coarsest solve alone) has
 // an FP64 z.
 template <typename T, typename TZ>
-void vcycle_typed(amg_hierarchy* h, const double* r, TZ* z, int rz_mode) {
+void vcycle_typed(amg_hierarchy* h, const double* r, TZ* z, int rz_mode, bool r32_ready) {
     cudaStream_t st = h->stream;
     const double* q2 = rz_mode == FIN_RHO_UPDATE_FCG ? h->q : nullptr;
     const int L = (int)h->lev.size() - 1;
@@ -1188,7 +1188,7 @@ void vcycle_typed(amg_hierarchy* h, const double* r, TZ* z, int rz_mode) {
         const int g = Lv.grid_pre[f32] ? Lv.grid_pre[f32] : sell_grid(h, S.nslices);
         T *xa = vec(Lv, VX), *ra = vec(Lv, VR), *xb = vec(Lv, VT);
         const int Vb = l == 0 ? 8 : V;
-        if (l == 0 && f32 && !h->r32_ready) {           // else the CG update already wrote it
+        if (l == 0 && f32 && !r32_ready) {           // else the CG update already wrote it
             Scope sc_(&h->prof, st, K_CONVERT, 12.0 * Lv.A.n);
             launch_dep(k_to_f32, vec_grid(h, Lv.A.n), TPB, 0, st, Lv.A.n, r, (float*)vec(Lv, VB));
             KERNEL_CHECK();
@@ -1492,10 +1492,10 @@ void kc_fcg2(amg_hierarchy* h, int m, const T* b, T* e) {
 // z = B r with the K-cycle on level 0 (FP64 r and z; with rz_mode the r.z
 // (and q.z) sums of the outer CG are finished as in the V-cycle).
 template <typename T, typename TZ>
-void kcycle_typed(amg_hierarchy* h, const double* r, TZ* z, int rz_mode) {
+void kcycle_typed(amg_hierarchy* h, const double* r, TZ* z, int rz_mode, bool r32_ready) {
     const int L = (int)h->lev.size() - 1;
     if (L <= 1) {                          // no intermediate level: the K-cycle is the V-cycle
-        vcycle_typed<T, TZ>(h, r, z, rz_mode);
+        vcycle_typed<T, TZ>(h, r, z, rz_mode, r32_ready);
         return;
     }
     cudaStream_t st = h->stream;
@@ -1511,7 +1511,7 @@ void kcycle_typed(amg_hierarchy* h, const double* r, TZ* z, int rz_mode) {
     T* xa = lvec<T>(L0, 1);
     T* ra = lvec<T>(L0, 2);
     const int g = L0.grid_pre[f32] ? L0.grid_pre[f32] : sell_grid(h, S.nslices);
-    if (f32 && !h->r32_ready) {                         // else the CG update already wrote it
+    if (f32 && !r32_ready) {                         // else the CG update already wrote it
         Scope sc_(&h->prof, st, K_CONVERT, 12.0 * n0);
         launch_dep(k_to_f32, vec_grid(h, n0), TPB, 0, st, n0, r, (float*)lvec<T>(L0, 0));
         KERNEL_CHECK();
@@ -1539,18 +1539,19 @@ void kcycle_typed(amg_hierarchy* h, const double* r, TZ* z, int rz_mode) {
 }
 
 template <typename T, typename TZ>
-void cycle_typed(amg_hierarchy* h, const double* r, TZ* z, int rz_mode) {
-    if (h->opt.cycle > 0) kcycle_typed<T, TZ>(h, r, z, rz_mode);
-    else vcycle_typed<T, TZ>(h, r, z, rz_mode);
+void cycle_typed(amg_hierarchy* h, const double* r, TZ* z, int rz_mode, bool r32_ready) {
+    if (h->opt.cycle > 0) kcycle_typed<T, TZ>(h, r, z, rz_mode, r32_ready);
+    else vcycle_typed<T, TZ>(h, r, z, rz_mode, r32_ready);
 }
 
 // The CG's own z = B r stays in the FP32 V-cycle's type.
 bool float_z(const amg_hierarchy* h) { return h->opt.precision == AMG_FP32_VCYCLE && h->lev.size() > 1; }
 
-void cg_precondition(amg_hierarchy* h, int rz_mode) {
-    if (float_z(h)) cycle_typed<float, float>(h, h->r, reinterpret_cast<float*>(h->z), rz_mode);
-    else if (h->opt.precision == AMG_FP32_VCYCLE) cycle_typed<float, double>(h, h->r, h->z, rz_mode);
-    else cycle_typed<double, double>(h, h->r, h->z, rz_mode);
+// r32_ready: level 0's float copy of h->r is the one k_update_xr wrote (FP32).
+void cg_precondition(amg_hierarchy* h, int rz_mode, bool r32_ready) {
+    if (float_z(h)) cycle_typed<float, float>(h, h->r, reinterpret_cast<float*>(h->z), rz_mode, r32_ready);
+    else if (h->opt.precision == AMG_FP32_VCYCLE) cycle_typed<float, double>(h, h->r, h->z, rz_mode, r32_ready);
+    else cycle_typed<double, double>(h, h->r, h->z, rz_mode, false);
 }
 
 // Launch-shape candidates of a grid-stride kernel that needs at most `need`
@@ -1735,8 +1736,8 @@ void autotune_vcycle(amg_hierarchy* h) {
 void coarse_cg_solve(amg_hierarchy* h, const double* b, double* x) { coarse_solve_launch(h, b, x, false, true); }
 
 void vcycle_plain(amg_hierarchy* h, const double* r, double* z) {
-    if (h->opt.precision == AMG_FP32_VCYCLE) cycle_typed<float, double>(h, r, z, FIN_NONE);
-    else cycle_typed<double, double>(h, r, z, FIN_NONE);
+    if (h->opt.precision == AMG_FP32_VCYCLE) cycle_typed<float, double>(h, r, z, FIN_NONE, false);
+    else cycle_typed<double, double>(h, r, z, FIN_NONE, false);
 }
 
 void level0_product(amg_hierarchy* h, const double* x, double* y) {
@@ -1795,7 +1796,6 @@ amg_status solve(amg_hierarchy* h, const double* b, double* x, double rtol, int 
     bool restart = true;
     // FP32 V-cycle: the CG update also writes level 0's float copy of r
     float* r32 = h->opt.precision == AMG_FP32_VCYCLE ? h->lev[0].b32 : nullptr;
-    h->r32_ready = false;
     struct Ev {
         cudaEvent_t e = nullptr;
         ~Ev() { if (e) cudaEventDestroy(e); }
@@ -1803,14 +1803,12 @@ amg_status solve(amg_hierarchy* h, const double* b, double* x, double rtol, int 
     CUDA_CHECK(cudaEventCreateWithFlags(&ev.e, cudaEventDisableTiming));
     // z = B r and beta for the next iteration
     auto precondition = [&]() {
-        h->r32_ready = r32 != nullptr;                  // level 0's float r is the one k_update_xr wrote
-        cg_precondition(h, h->opt.krylov == 1 || h->opt.cycle > 0 ? FIN_RHO_UPDATE_FCG : FIN_RHO_UPDATE);
-        h->r32_ready = false;
+        cg_precondition(h, h->opt.krylov == 1 || h->opt.cycle > 0 ? FIN_RHO_UPDATE_FCG : FIN_RHO_UPDATE, r32 != nullptr);
     };
     if (rel <= rtol) status = AMG_OK;
     while (status != AMG_OK && it < maxit) {
         if (restart) {
-            cg_precondition(h, FIN_RHO_INIT);              // beta = 0
+            cg_precondition(h, FIN_RHO_INIT, false);       // beta = 0
             restart = false;
         }
         const float* z32 = reinterpret_cast<const float*>(h->z);
@@ -1840,7 +1838,7 @@ amg_status solve(amg_hierarchy* h, const double* b, double* x, double rtol, int 
         ++it;
         // The scalars go to the host. While the residual is well above the
         // tolerance, the next iteration's preconditioner (which
-        // writes only z and the device scalars) are queued behind the
+        // writes only z and the device scalars) is queued behind the
         // copy before the host waits for it, so the round trip overlaps the
         // V-cycle; if the check below ends the loop after all, x and r are
         // final and that work goes unused, and a restart recomputes rho and p
