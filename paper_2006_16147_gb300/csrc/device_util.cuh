@@ -96,14 +96,14 @@ __device__ __forceinline__ double block_sums(const double (&v)[NV]) {
     return w < NV ? warp_sum(s0) : 0.0;
 }
 
-// Programmatic dependent launch: a kernel started with launch_dep (below, host
-// side) may begin while the kernel before it on the stream still runs. It does
-// what needs only the hierarchy's arrays, then dep_wait() returns when that
-// kernel is done and its writes are visible; and only then may the next one
-// begin, so at most two kernels overlap. Vectors that an earlier kernel wrote
-// are read after the wait and with ldv: an ordinary load, never ld.nc, which
-// the compiler picks for const __restrict__ pointers and which the wait does
-// not order.
+// Programmatic dependent launch: a kernel started with launch_dep
+// (amg_internal.cuh) may begin while the kernel before it on the stream still
+// runs. It does what needs only the hierarchy's arrays, then dep_wait() returns
+// when that kernel is done and its writes are visible; and only then may the
+// next one begin, so at most two kernels overlap. Vectors that an earlier kernel
+// wrote are read after the wait and with ldv: an ordinary load, never ld.nc,
+// which the compiler picks for const __restrict__ pointers and which the wait
+// does not order.
 __device__ __forceinline__ void dep_wait() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -136,6 +136,52 @@ __device__ __forceinline__ float d2f(double d) {
     const unsigned rest = lo << 3;                                // the 29 bits below the result's last
     t += rest > 0x80000000u || (rest == 0x80000000u && (t & 1u));
     return __uint_as_float((e ? t : 0u) | (hi & 0x80000000u));
+}
+
+__device__ __forceinline__ float rcp_approx(float y) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(y));
+    return r;
+}
+
+// Correctly rounded quotient of doubles without the FP64 pipe (a division
+// holds it for some ten instructions of 64 cycles a warp). Mantissas n, d: the
+// integer Q = floor(n 2^53 / d), by a 24-bit reciprocal, one Newton step in
+// 64-bit integers and an exact remainder that corrects the last bits; the
+// quotient of two doubles is never half-way between two, so Q's last bit alone
+// decides the rounding. Zero, subnormal, infinite or NaN operands and quotients
+// near the ends of the range take the division instruction sequence.
+__device__ __forceinline__ double div_rn(double a, double b) {
+    const unsigned long long ua = (unsigned long long)__double_as_longlong(a);
+    const unsigned long long ub = (unsigned long long)__double_as_longlong(b);
+    const int ea = (int)(ua >> 52) & 0x7ff, eb = (int)(ub >> 52) & 0x7ff;
+    int e = ea - eb + 1023;
+    if ((unsigned)(ea - 1) >= 2046u || (unsigned)(eb - 1) >= 2046u || (unsigned)(e - 2) >= 2044u) return __ddiv_rn(a, b);
+    const unsigned long long one = 1ull << 52;
+    unsigned long long n = (ua & (one - 1)) | one;
+    const unsigned long long d = (ub & (one - 1)) | one;
+    if (n < d) {                                          // quotient in [1, 2)
+        n <<= 1;
+        --e;
+    }
+    // x 2^-23 ~ 2^53 / d, in (1, 2]: from d's top 24 bits as a float in [1, 2)
+    const float y = __uint_as_float(0x3f800000u | (unsigned)((d >> 29) & 0x7fffffu));
+    const unsigned x = (unsigned)(rcp_approx(y) * 0x1p24f);
+    const long long r0 = -(long long)(d * x);             // 2^76 - x d, below 2^55
+    const unsigned long long x1 = ((unsigned long long)x << 36) + (unsigned long long)(((r0 >> 20) * (long long)x) >> 20);
+    // x1 2^-59 ~ 2^53 / d; Q ~ n x1 2^-59
+    unsigned long long q = __umul64hi(n << 10, x1) >> 5;
+    long long r = (long long)((n << 53) - q * d);         // exact: below 2^63
+    const long long dq = ((r >> 30) * (long long)x) >> 46;
+    q += (unsigned long long)dq;
+    r -= dq * (long long)d;
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+        if (r < 0) { r += (long long)d; --q; }
+        else if (r >= (long long)d) { r -= (long long)d; ++q; }
+    }
+    q = (q + 1) >> 1;                                     // at most 2^53: then the exponent below carries
+    return __longlong_as_double((long long)(((ua ^ ub) & (1ull << 63)) | (((unsigned long long)(e - 1) << 52) + q)));
 }
 
 // A double of magnitude 2^-104 .. 2^103 times 2^SPLIT_UP as three floats,

@@ -112,53 +112,6 @@ __global__ void k_dww(int n, double* __restrict__ diag, const double* __restrict
         diag[i] = __dmul_rn(__dmul_rn(diag[i], w[i]), w[i]);
 }
 
-// ---------------------------------------------------------- division ----
-__device__ __forceinline__ float rcp_approx(float y) {
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(y));
-    return r;
-}
-
-// Correctly rounded quotient of doubles without the FP64 pipe (a division
-// holds it for some ten instructions of 64 cycles a warp). Mantissas n, d: the
-// integer Q = floor(n 2^53 / d), by a 24-bit reciprocal, one Newton step in
-// 64-bit integers and an exact remainder that corrects the last bits; the
-// quotient of two doubles is never half-way between two, so Q's last bit alone
-// decides the rounding. Zero, subnormal, infinite or NaN operands and quotients
-// near the ends of the range take the division instruction sequence.
-__device__ __forceinline__ double div_rn(double a, double b) {
-    const unsigned long long ua = (unsigned long long)__double_as_longlong(a);
-    const unsigned long long ub = (unsigned long long)__double_as_longlong(b);
-    const int ea = (int)(ua >> 52) & 0x7ff, eb = (int)(ub >> 52) & 0x7ff;
-    int e = ea - eb + 1023;
-    if ((unsigned)(ea - 1) >= 2046u || (unsigned)(eb - 1) >= 2046u || (unsigned)(e - 2) >= 2044u) return __ddiv_rn(a, b);
-    const unsigned long long one = 1ull << 52;
-    unsigned long long n = (ua & (one - 1)) | one;
-    const unsigned long long d = (ub & (one - 1)) | one;
-    if (n < d) {                                          // quotient in [1, 2)
-        n <<= 1;
-        --e;
-    }
-    // x 2^-23 ~ 2^53 / d, in (1, 2]: from d's top 24 bits as a float in [1, 2)
-    const float y = __uint_as_float(0x3f800000u | (unsigned)((d >> 29) & 0x7fffffu));
-    const unsigned x = (unsigned)(rcp_approx(y) * 0x1p24f);
-    const long long r0 = -(long long)(d * x);             // 2^76 - x d, below 2^55
-    const unsigned long long x1 = ((unsigned long long)x << 36) + (unsigned long long)(((r0 >> 20) * (long long)x) >> 20);
-    // x1 2^-59 ~ 2^53 / d; Q ~ n x1 2^-59
-    unsigned long long q = __umul64hi(n << 10, x1) >> 5;
-    long long r = (long long)((n << 53) - q * d);         // exact: below 2^63
-    const long long dq = ((r >> 30) * (long long)x) >> 46;
-    q += (unsigned long long)dq;
-    r -= dq * (long long)d;
-#pragma unroll
-    for (int t = 0; t < 2; ++t) {
-        if (r < 0) { r += (long long)d; --q; }
-        else if (r >= (long long)d) { r -= (long long)d; ++q; }
-    }
-    q = (q + 1) >> 1;                                     // at most 2^53: then the exponent below carries
-    return __longlong_as_double((long long)(((ua ^ ub) & (1ull << 63)) | (((unsigned long long)(e - 1) << 52) + q)));
-}
-
 // --------------------------------------------------- Eq. 3 edge weights ----
 // c_ij = 1 - 2 a_ij w_i w_j / (a_ii w_i^2 + a_jj w_j^2) for the pair {lo, hi}
 // from the upper entry a_{lo,hi}; written at both stored positions of the
@@ -2641,7 +2594,9 @@ struct Scratch {
     int* cnt = nullptr;       // [0,1] list counters, [2,3] match counters, [4] rounds, [5] flags, [6..7] totals,
                               // [8] rows left by the group row-product kernels, [9] by the group edge sort,
                               // [10..13] sparse-product and pair-sort overflow and list counters,
-                              // [13, 14] also rows left by the long-row kernels
+                              // [13, 14] also rows left by the long-row kernels, [15] the matching's round,
+                              // [16] its error, [19] longest row or entries kept, [20] places of lined-up
+                              // slices, [24..26] rows of a sparse product by path, [32] grid barrier
     int* flag = nullptr;      // n
     int* qid = nullptr;       // n
     int* heads = nullptr;     // n
