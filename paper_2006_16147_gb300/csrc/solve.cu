@@ -133,8 +133,10 @@ __device__ __forceinline__ T ld(const T* p) { return __ldg(p); }
 //           turns (256^3 level 0 with RB = 8: k_post 262 -> 452 us)
 // The order of the additions is the same. Two accumulators (the second takes
 // every other entry of the full fours) shorten the FMA chain (latency-bound
-// kernels); one saves the final add, which pays in the fused smoothers, where the FP64 pipe (this GPU's
-// FP64 rate is 1/64 of its FP32 rate) is the bound.
+// kernels); one saves the final add, which pays in the fused smoothers, where the
+// FP64 pipe (one warp instruction per 76 cycles of an SM sub-partition) is the
+// bound. The other products keep two at both sizes, a ninth FP64 instruction a
+// row on large stencils (256^3: k_spmv_dot 294 us, its nine take 285 at that rate).
 template <int RB, typename T>
 struct RowBatch {
     int w, i;                       // entries, slice position
