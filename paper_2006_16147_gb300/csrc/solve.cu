@@ -27,6 +27,7 @@ namespace {
 constexpr int TPB = 256;
 constexpr int WARPS = TPB / 32;
 constexpr int CG_TPB = 1024;  // threads of the iterative coarsest solve's blocks
+constexpr int CG_EIGHT = 256; // entries of a long row that eight lanes take there
 
 enum FinMode : int {
     FIN_NORMS = 0, FIN_PQ = 1, FIN_RR = 2, FIN_RHO_INIT = 3, FIN_RHO_UPDATE = 4, FIN_NONE = 5, FIN_RHO_UPDATE_FCG = 6
@@ -739,7 +740,9 @@ __device__ __forceinline__ void cg_sums(const double* part, int G, double (&out)
     for (int j = 0; j < NO; ++j) out[j] = tot[j];
 }
 
-template <typename TI, typename TO>
+// HUB: a row is longer than CG_EIGHT (the loop for it costs the others registers:
+// 256^3 jump coefficients 108.4 -> 109.1 ms).
+template <typename TI, typename TO, bool HUB>
 __global__ void __launch_bounds__(CG_TPB, 1) k_coarse_cg(SellView S, const double* __restrict__ val, int n,
                                                    int nlong, const int* __restrict__ long_rows,
                                                    const int* __restrict__ cptr, const int* __restrict__ ccol,
@@ -802,38 +805,55 @@ __global__ void __launch_bounds__(CG_TPB, 1) k_coarse_cg(SellView S, const doubl
             const int lane = threadIdx.x & 31, nw = G * (blockDim.x >> 5);
             // tasks of a warp: four long rows straight from the CSR, eight lanes
             // each (a warp per row spent five additions and three steps of one
-            // lane on every row), then slices
+            // lane on every row), then slices. What a row has beyond CG_EIGHT
+            // entries the whole warp takes, one row after the other: eight lanes
+            // alone made a hub of 5000 entries the chain that the grid waits for
+            // (22K rows with such a hub, 30 iterations: 3172 us, 1299 so)
             const int ntask = (nlong + 3) / 4 + S.nslices;
             for (int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); t < ntask; t += nw) {
                 if (t < (nlong + 3) / 4) {
                     const int lr = 4 * t + (lane >> 3);
                     const int i = lr < nlong ? __ldg(long_rows + lr) : -1;
                     Own o{};
-                    int k = 0, e = 0;
+                    int k0 = 0, e = 0;
                     if (i >= 0) {
                         o = own(i);
-                        k = __ldg(cptr + i) + (lane & 7);
+                        k0 = __ldg(cptr + i);
                         e = __ldg(cptr + i + 1);
                     }
-                    double acc = 0.0;
-                    for (; k < e; k += 32) {
-                        int j[4];
-                        double v[4], zv[4];
+                    // entries k, k + L, .. below end, four of them in flight
+                    auto part = [&](int k, int end, auto L) {
+                        double s = 0.0;
+                        for (; k < end; k += 4 * L()) {
+                            int j[4];
+                            double v[4], zv[4];
 #pragma unroll
-                        for (int u = 0; u < 4; ++u) {
-                            const bool ok = k + 8 * u < e;
-                            j[u] = ok ? __ldg(ccol + k + 8 * u) : -1;
-                            v[u] = ok ? __ldg(cval + k + 8 * u) : 0.0;
+                            for (int u = 0; u < 4; ++u) {
+                                const bool ok = k + L() * u < end;
+                                j[u] = ok ? __ldg(ccol + k + L() * u) : -1;
+                                v[u] = ok ? __ldg(cval + k + L() * u) : 0.0;
+                            }
+#pragma unroll
+                            for (int u = 0; u < 4; ++u) zv[u] = j[u] >= 0 ? z[j[u]] : 0.0;
+#pragma unroll
+                            for (int u = 0; u < 4; ++u)
+                                if (j[u] >= 0) s = fma(v[u], zv[u], s);
                         }
-#pragma unroll
-                        for (int u = 0; u < 4; ++u) zv[u] = j[u] >= 0 ? z[j[u]] : 0.0;
-#pragma unroll
-                        for (int u = 0; u < 4; ++u)
-                            if (j[u] >= 0) acc = fma(v[u], zv[u], acc);
-                    }
-                    __syncwarp();
+                        __syncwarp();
+                        return s;
+                    };
+                    const bool hub = HUB && e - k0 > CG_EIGHT;
+                    double acc = part(k0 + (lane & 7), hub ? k0 + CG_EIGHT : e, std::integral_constant<int, 8>());
 #pragma unroll
                     for (int w = 4; w > 0; w >>= 1) acc += __shfl_xor_sync(FULL_MASK, acc, w);
+                    if constexpr (HUB) {
+                        for (unsigned hubs = __ballot_sync(FULL_MASK, hub && (lane & 7) == 0); hubs; hubs &= hubs - 1) {
+                            const int src = __ffs(hubs) - 1;
+                            const int kq = __shfl_sync(FULL_MASK, k0, src) + CG_EIGHT, eq = __shfl_sync(FULL_MASK, e, src);
+                            const double s = warp_sum(part(kq + lane, eq, std::integral_constant<int, 32>()));
+                            if (lane == src) acc += s;
+                        }
+                    }
                     if (i >= 0 && (lane & 7) == 0) finish_row(i, o, acc);
                     continue;
                 }
@@ -1083,6 +1103,12 @@ int red_grid(const amg_hierarchy* h, int nslices) { return blocks_for(nslices, W
 int red_grid_rows(const amg_hierarchy* h, int n) { return blocks_for(n, TPB, h->red.blocks); }
 int wide_grid(const amg_hierarchy* h, long long rows) { return blocks_for(rows * 32, TPB, h->num_sms * 16); }
 
+template <bool HUB>
+const void* coarse_cg_kernel(bool fp32_in, bool fp64_out) {
+    if (!fp32_in) return (const void*)k_coarse_cg<double, double, HUB>;
+    return fp64_out ? (const void*)k_coarse_cg<float, double, HUB> : (const void*)k_coarse_cg<float, float, HUB>;
+}
+
 void coarse_solve_launch(amg_hierarchy* h, const void* b, void* x, bool fp32_in, bool fp64_out) {
     const int n = h->nc;
     if (h->segL_ptr) {
@@ -1121,8 +1147,8 @@ void coarse_solve_launch(amg_hierarchy* h, const void* b, void* x, bool fp32_in,
         double rtol = 1e-4;
         void* args[] = {&S, &val, &nrows, &nlong, &long_rows, &cptr, &ccol, &cval, &minv, const_cast<void**>(&b), &x,
                         &C.x, &C.r, &C.z, &C.p, &C.q, &C.part, &bar, &err, &maxit, &rtol};
-        const void* fn = !fp32_in ? (const void*)k_coarse_cg<double, double>
-                                  : (fp64_out ? (const void*)k_coarse_cg<float, double> : (const void*)k_coarse_cg<float, float>);
+        const void* fn = Lc.A.max_row > CG_EIGHT ? coarse_cg_kernel<true>(fp32_in, fp64_out)
+                                                 : coarse_cg_kernel<false>(fp32_in, fp64_out);
         CUDA_CHECK(cudaLaunchCooperativeKernel(fn, dim3(C.blocks), dim3(CG_TPB), args, 0, h->stream));
         KERNEL_CHECK();
         return;
@@ -1686,7 +1712,7 @@ void prepare_solve(amg_hierarchy* h) {
         const int nc = h->lev.back().A.n;
         CoarseCg& C = h->ccg;
         int per_sm = 0;
-        CUDA_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_coarse_cg<double, double>, CG_TPB, 0));
+        CUDA_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_coarse_cg<double, double, true>, CG_TPB, 0));
         if (per_sm < 1) AMG_THROW(AMG_ERR_CUDA, "coarsest CG kernel cannot be resident");
         C.blocks = h->num_sms;
         C.x = h->mem.alloc<double>(nc);
