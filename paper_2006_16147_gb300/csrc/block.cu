@@ -206,8 +206,13 @@ __device__ __forceinline__ void sell_row_k(const SellV& S, const T* __restrict__
 // chain. A matrix entry is split once for the lane's columns. One entry at a
 // time: in 64 registers the other warps hide the loads, and four blocks per SM
 // matter more (128^3 x 64 columns: 2407 us, 2600-3400 us with two or four
-// entries in flight and two or three blocks).
-template <bool VEC, int CPL>
+// entries in flight and two or three blocks). In a slice wider than SPLIT_WIDE
+// one row is a chain that other warps do not hide, and its entries are loaded
+// four at a time: with a hub of 5000 entries 1760 us one by one, 828 so, in the
+// same order of additions. The loop for that stands in a kernel of its own
+// (WIDE), as it costs the other rows registers (128^3 x 64 columns: 208 -> 213 ms).
+constexpr int SPLIT_WIDE = 64;
+template <bool VEC, int CPL, bool WIDE>
 __device__ __forceinline__ void sell_row_split(const SellV& S, const double* __restrict__ val, int ip, int c0, int k,
                                                const float* __restrict__ X, int ld, const bool (&on)[CPL],
                                                double (&acc)[CPL]) {
@@ -216,7 +221,28 @@ __device__ __forceinline__ void sell_row_split(const SellV& S, const double* __r
     const int w = __ldg(S.sptr + s + 1) - s0;
     const long long base = (long long)s0 * 32 + r;
     SplitSum sum[CPL];
-    for (int e = 0; e < w; ++e) {
+    int e = 0;
+    if (WIDE && w > SPLIT_WIDE)
+#pragma unroll 1
+        for (; e + 4 <= w; e += 4) {
+            int j[4];
+            double a[4];
+            float xs[4][CPL];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                j[u] = __ldg(S.col + base + 32 * (e + u));
+                a[u] = __ldg(val + base + 32 * (e + u));
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) ld_cols<VEC, CPL>(X + (size_t)j[u] * ld + c0, xs[u], k - c0);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const Split3 s = split3(a[u]);
+#pragma unroll
+                for (int m = 0; m < CPL; ++m) sum[m].add(s, xs[u][m]);
+            }
+        }
+    for (; e < w; ++e) {
         const int j = __ldg(S.col + base + 32 * e);
         const Split3 a = split3(__ldg(val + base + 32 * e));
         float xs[CPL];
@@ -839,7 +865,8 @@ __global__ void __launch_bounds__(CC_TPB) bk_coarse_cg(SellV S, const double* __
 // product and direction passes that this replaces, which were bound by them:
 // 128^3 rows x 64 columns 2143 + 495 us, 2407 us now; 64^3 x 16 about 107 us,
 // 95 us now.
-template <typename TZ, int CPL, bool VEC>
+// WIDE (FP32): a row is longer than SPLIT_WIDE.
+template <typename TZ, int CPL, bool VEC, bool WIDE>
 __global__ void __launch_bounds__(TPB, sizeof(TZ) == 4 && CPL <= 4 ? 4 : 1) bk_direction(SellV S, const double* __restrict__ val,
                                                     const TZ* __restrict__ Z, double* __restrict__ P,
                                                     double* __restrict__ Q, int k, int ld, int G, double* partial,
@@ -865,7 +892,7 @@ __global__ void __launch_bounds__(TPB, sizeof(TZ) == 4 && CPL <= 4 ? 4 : 1) bk_d
             double acc[CPL], pv[CPL], qv[CPL];
             TZ zv[CPL];
             if constexpr (sizeof(TZ) == 4) {
-                sell_row_split<VEC, CPL>(S, val, ip, c0, k, Z, ld, on, acc);
+                sell_row_split<VEC, CPL, WIDE>(S, val, ip, c0, k, Z, ld, on, acc);
             } else {
 #pragma unroll
                 for (int m = 0; m < CPL; ++m) acc[m] = 0.0;
@@ -1373,12 +1400,16 @@ void block_step_kernels(amg_hierarchy* h, double* X, int k, bool any_active) {
     if (any_active) {
         {
             Scope sc_(&h->prof, st, K_SPMV_DOT, 12.0 * nnz + (f32 ? 36.0 : 40.0) * n * k);
-            if (f32)
-                DISPATCH_CPL(cpl, ld, launch_dep(bk_direction<float, CPL, VEC>, red_grid(h, W, G), TPB, 0, st, 
+            if (f32 && L0.A.max_row > SPLIT_WIDE)
+                DISPATCH_CPL(cpl, ld, launch_dep(bk_direction<float, CPL, VEC, true>, red_grid(h, W, G), TPB, 0, st,
+                                          sv(L0.S), L0.S.val, (const float*)W.Z, W.P, W.Q, k, ld, G, W.partial,
+                                          W.ticket, W.sc));
+            else if (f32)
+                DISPATCH_CPL(cpl, ld, launch_dep(bk_direction<float, CPL, VEC, false>, red_grid(h, W, G), TPB, 0, st,
                                           sv(L0.S), L0.S.val, (const float*)W.Z, W.P, W.Q, k, ld, G, W.partial,
                                           W.ticket, W.sc));
             else
-                DISPATCH_CPL(cpl, ld, launch_dep(bk_direction<double, CPL, VEC>, red_grid(h, W, G), TPB, 0, st, 
+                DISPATCH_CPL(cpl, ld, launch_dep(bk_direction<double, CPL, VEC, false>, red_grid(h, W, G), TPB, 0, st, 
                                           sv(L0.S), L0.S.val, W.Z, W.P, W.Q, k, ld, G, W.partial, W.ticket, W.sc));
             KERNEL_CHECK();
         }
