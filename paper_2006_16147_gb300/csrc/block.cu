@@ -1548,8 +1548,8 @@ void block_set_columns(amg_hierarchy* h, int c0, int cnt, int mode, double rtol)
     for (int c = c0; c < c0 + cnt; ++c) W.mode_host[c] = mode;
 }
 
-amg_status solve_batch(amg_hierarchy* h, int k, const double* B, double* X, double rtol, int maxit,
-                       amg_solve_info* infos) {
+static amg_status solve_columns(amg_hierarchy* h, int k, const double* B, double* X, double rtol, int maxit,
+                                amg_solve_info* infos) {
     auto t0 = std::chrono::steady_clock::now();
     BlockWork& W = block_ensure(h, k, false);
     block_set_columns(h, 0, k, COL_INIT, rtol);
@@ -1590,6 +1590,25 @@ amg_status solve_batch(amg_hierarchy* h, int k, const double* B, double* X, doub
             infos[c].solve_ms = ms;
         }
     }
+    return status;
+}
+
+// The kernels load two doubles of B and X at once: blocks that start off a
+// 16-byte boundary are solved in copies.
+amg_status solve_batch(amg_hierarchy* h, int k, const double* B, double* X, double rtol, int maxit,
+                       amg_solve_info* infos) {
+    if (((reinterpret_cast<uintptr_t>(B) | reinterpret_cast<uintptr_t>(X)) & 15) == 0 || k > MAXK)
+        return solve_columns(h, k, B, X, rtol, maxit, infos);
+    const size_t count = (size_t)h->lev[0].A.n * k;
+    DevArena mem;
+    mem.stream = h->stream;
+    double* Bc = mem.alloc<double>(count);
+    double* Xc = mem.alloc<double>(count);
+    CUDA_CHECK(cudaMemcpyAsync(Bc, B, sizeof(double) * count, cudaMemcpyDeviceToDevice, h->stream));
+    CUDA_CHECK(cudaMemcpyAsync(Xc, X, sizeof(double) * count, cudaMemcpyDeviceToDevice, h->stream));
+    const amg_status status = solve_columns(h, k, Bc, Xc, rtol, maxit, infos);
+    CUDA_CHECK(cudaMemcpyAsync(X, Xc, sizeof(double) * count, cudaMemcpyDeviceToDevice, h->stream));
+    CUDA_CHECK(cudaStreamSynchronize(h->stream));
     return status;
 }
 
