@@ -36,6 +36,7 @@ void set_last_error(const std::string& m);
     do {                                                                                  \
         cudaError_t _e = (expr);                                                          \
         if (_e != cudaSuccess) {                                                          \
+            cudaGetLastError(); /* reported here, not by the next launch check as well */ \
             amg_status _s = (_e == cudaErrorMemoryAllocation) ? AMG_ERR_OOM : AMG_ERR_CUDA; \
             AMG_THROW(_s, "%s failed: %s (%s:%d)", #expr, cudaGetErrorString(_e), __FILE__, __LINE__); \
         }                                                                                 \
