@@ -17,6 +17,7 @@
 #include <algorithm>
 #include <chrono>
 #include <cmath>
+#include <memory>
 #include <type_traits>
 
 #include "amg_internal.cuh"
@@ -1312,9 +1313,11 @@ BlockWork& block_ensure(amg_hierarchy* h, int K, bool fixed_width) {
         delete h->blk;
         h->blk = nullptr;
     }
-    BlockWork* W = new BlockWork;
+    // the hierarchy gets the workspace when it is whole: one that an allocation
+    // ended would be taken for it by the next call of the same width
+    std::unique_ptr<BlockWork> own(new BlockWork);
+    BlockWork* W = own.get();
     W->mem.stream = h->stream;
-    h->blk = W;
     W->K = K;
     W->fixed_width = fixed_width;
     const bool f32 = h->opt.precision == AMG_FP32_VCYCLE;
@@ -1364,7 +1367,8 @@ BlockWork& block_ensure(amg_hierarchy* h, int K, bool fixed_width) {
         if (per_sm < 1) AMG_THROW(AMG_ERR_CUDA, "multi-column coarsest CG kernel cannot be resident");
     }
     if (h->opt.autotune && !fixed_width) block_autotune(h, *W);
-    return *W;
+    h->blk = own.release();
+    return *h->blk;
 }
 
 size_t block_bytes_per_column(const amg_hierarchy* h) {

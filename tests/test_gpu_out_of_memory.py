@@ -39,3 +39,26 @@ def test_setup_after_a_failed_one():
     h = amg.amg_setup(*c)
     assert amg.amg_hierarchy_info(h)["n"][0] == A.n
     h.close()
+
+
+def test_block_solve_after_a_failed_one():
+    import torch
+    from paper_2006_16147_gb300 import amg
+    A = W.poisson3d(64)
+    k = 192                                        # some 4 GB of work arrays
+    h = setup(A)
+    B = dev(W.rhs_normal(A.n, 2, k))
+    X = torch.zeros_like(B)
+    hog = leave(1 << 30)
+    with pytest.raises(amg.AmgError) as e:
+        amg.amg_solve_batch(h, B, X)
+    assert e.value.status == amg.AMG_ERR_OOM
+    few = torch.zeros((A.n, 2), dtype=torch.float64, device="cuda:0")
+    assert amg.amg_solve_batch(h, B[:, :2].contiguous(), few)[0]["status"] == 0
+    del hog
+    torch.cuda.empty_cache()
+    infos = amg.amg_solve_batch(h, B, X)
+    assert infos[0]["status"] == 0 and max(i["true_relres"] for i in infos) <= 1e-6
+    r = B[:, 0].cpu().numpy() - W.csr_matvec(A, X[:, 0].cpu().numpy())
+    assert np.linalg.norm(r) <= 1.01e-6 * np.linalg.norm(B[:, 0].cpu().numpy())
+    h.close()
