@@ -1136,15 +1136,18 @@ void group_shape(const BlockWork& W, int k, int* G, int* cpl) {
     } while (0)
 
 // A kernel over rows, started beside the one before it (launch_dep) where its
-// entries times columns (`work`) are few, after it otherwise: a large kernel gains
-// nothing, and the blocks that already wait take its place in the caches and on
-// the SMs (rows of 60 entries, 100K x 16 columns, FP64: 18.8 ms a solve with all
-// dependent, 17.8 so; rows of 300, 50K x 16: 23.5, 22.1; 64^3 x 64: 38.3, 37.3;
-// small ones lose 3% without). 2M and 8M are alike.
-constexpr long long DEP_WORK = 2LL << 20;
+// entries times columns (`work`) are few, after it otherwise: in a block solve a
+// large kernel gains nothing, and the blocks that already wait take its place in
+// the caches and on the SMs (rows of 60 entries, 100K x 16 columns, FP64: 18.8 ms
+// a solve with all dependent, 17.6 so; rows of 300, 50K x 16: 23.5, 21.9; 64^3 x
+// 64: 38.3, 37.3; small ones lose 3% without; a bound of 2M or 24M is as good).
+// The server's kernels (fixed width), launched one by one on several streams, are
+// all dependent: with the same bound 12 requests on 3 operators take 3% longer.
+constexpr long long DEP_WORK = 8LL << 20;
 template <typename... P, typename... A>
-void launch_rows(long long work, void (*kernel)(P...), int grid, int threads, size_t smem, cudaStream_t st, A&&... args) {
-    if (work <= DEP_WORK) launch_dep(kernel, grid, threads, smem, st, std::forward<A>(args)...);
+void launch_rows(const BlockWork& W, long long work, void (*kernel)(P...), int grid, int threads, size_t smem,
+                 cudaStream_t st, A&&... args) {
+    if (W.fixed_width || work <= DEP_WORK) launch_dep(kernel, grid, threads, smem, st, std::forward<A>(args)...);
     else kernel<<<grid, threads, smem, st>>>(std::forward<A>(args)...);
 }
 
@@ -1179,15 +1182,15 @@ void block_vcycle(amg_hierarchy* h, BlockWork& W, int k, int flexible) {
         Scope sc_(&h->prof, st, l == 0 ? K_PRE_L0 : K_PRE,
                   (double)Lv.A.nnz * (sizeof(T) + 4) + (double)Lv.A.n * k * ((l == 0 ? 8 : sizeof(T)) + 2.0 * sizeof(T)));
         if (l == 0 && !f32)
-            DISPATCH_CPL(cpl, ld, launch_rows((long long)Lv.A.nnz * k, bk_pre<T, CPL, VEC>, g, TPB, 0, st, sv(Lv.S), valm, minv, omega, (const T*)W.R, lv(W.x, 0),
+            DISPATCH_CPL(cpl, ld, launch_rows(W, (long long)Lv.A.nnz * k, bk_pre<T, CPL, VEC>, g, TPB, 0, st, sv(Lv.S), valm, minv, omega, (const T*)W.R, lv(W.x, 0),
                                                                        lv(W.r, 0), k, ld, G));
         else
-            DISPATCH_CPL(cpl, ld, launch_rows((long long)Lv.A.nnz * k, bk_pre<T, CPL, VEC>, g, TPB, 0, st, sv(Lv.S), valm, minv, omega, lv(W.b, l), lv(W.x, l),
+            DISPATCH_CPL(cpl, ld, launch_rows(W, (long long)Lv.A.nnz * k, bk_pre<T, CPL, VEC>, g, TPB, 0, st, sv(Lv.S), valm, minv, omega, lv(W.b, l), lv(W.x, l),
                                                                   lv(W.r, l), k, ld, G));
         KERNEL_CHECK();
         const int nc = h->lev[l + 1].A.n;
         const T* p = f32 ? (const T*)Lv.p32 : (const T*)Lv.p;
-        DISPATCH_CPL(cpl, ld, launch_rows((long long)Lv.A.n * k, bk_restrict<T, CPL, VEC>, grid_rows(h, nc, G), TPB, 0, st, nc, Lv.pt_ptr, Lv.pt_idx, p,
+        DISPATCH_CPL(cpl, ld, launch_rows(W, (long long)Lv.A.n * k, bk_restrict<T, CPL, VEC>, grid_rows(h, nc, G), TPB, 0, st, nc, Lv.pt_ptr, Lv.pt_idx, p,
                                                                                    lv(W.r, l), lv(W.b, l + 1), k, ld, G));
         KERNEL_CHECK();
     }
@@ -1233,11 +1236,11 @@ void block_vcycle(amg_hierarchy* h, BlockWork& W, int k, int flexible) {
         Scope sc_(&h->prof, st, l == 0 ? K_POST_L0 : K_POST,
                   (double)Lv.ap_nnz * (sizeof(T) + 4) + (double)Lv.A.n * k * (4.0 * sizeof(T) + 8));
         if (l > 0)
-            DISPATCH_CPL(cpl, ld, launch_rows((long long)Lv.ap_nnz * k, bk_post<T, T, CPL, false, VEC>, g, TPB, 0, st, 
+            DISPATCH_CPL(cpl, ld, launch_rows(W, (long long)Lv.ap_nnz * k, bk_post<T, T, CPL, false, VEC>, g, TPB, 0, st, 
                                   sv(Lv.AP), apv, minv, omega, Lv.agg, p, e, lv(W.x, l), lv(W.r, l), nullptr, nullptr,
                                   lv(W.y, l), k, ld, G, W.partial, W.ticket, W.sc, flexible));
         else
-            DISPATCH_CPL(cpl, ld, launch_rows((long long)Lv.ap_nnz * k, bk_post<T, T, CPL, true, VEC>, red_grid(h, W, G), TPB, 0, st, 
+            DISPATCH_CPL(cpl, ld, launch_rows(W, (long long)Lv.ap_nnz * k, bk_post<T, T, CPL, true, VEC>, red_grid(h, W, G), TPB, 0, st, 
                                   sv(Lv.AP), apv, minv, omega, Lv.agg, p, e, lv(W.x, 0), lv(W.r, 0), W.R,
                                   flexible ? W.Q : nullptr, (T*)W.Z, k, ld, G, W.partial, W.ticket, W.sc, flexible));
         KERNEL_CHECK();
@@ -1391,7 +1394,7 @@ void block_init_launch(amg_hierarchy* h, const double* B, double* X, int k) {
     int G, cpl;
     group_shape(W, k, &G, &cpl);
     Level& L0 = h->lev[0];
-    DISPATCH_CPL(cpl, W.K, launch_rows((long long)L0.A.nnz * k, bk_residual<CPL, VEC>, red_grid(h, W, G), TPB, 0, st, sv(L0.S), L0.S.val, X, B, W.R, r32_of(h), k, W.K, G,
+    DISPATCH_CPL(cpl, W.K, launch_rows(W, (long long)L0.A.nnz * k, bk_residual<CPL, VEC>, red_grid(h, W, G), TPB, 0, st, sv(L0.S), L0.S.val, X, B, W.R, r32_of(h), k, W.K, G,
                                                              W.partial, W.ticket, W.sc, 0));
     KERNEL_CHECK();
     bk_zero_cols<<<blocks_for((long long)L0.A.n * k, TPB, h->num_sms * 8), TPB, 0, st>>>(L0.A.n, X, k, W.K, W.sc.mode,
@@ -1418,21 +1421,21 @@ void block_step_kernels(amg_hierarchy* h, double* X, int k, bool any_active) {
         {
             Scope sc_(&h->prof, st, K_SPMV_DOT, 12.0 * nnz + (f32 ? 36.0 : 40.0) * n * k);
             if (f32 && L0.A.max_row > SPLIT_WIDE)
-                DISPATCH_CPL(cpl, ld, launch_rows((long long)L0.A.nnz * k, bk_direction<float, CPL, VEC, true>, red_grid(h, W, G), TPB, 0, st,
+                DISPATCH_CPL(cpl, ld, launch_rows(W, (long long)L0.A.nnz * k, bk_direction<float, CPL, VEC, true>, red_grid(h, W, G), TPB, 0, st,
                                           sv(L0.S), L0.S.val, (const float*)W.Z, W.P, W.Q, k, ld, G, W.partial,
                                           W.ticket, W.sc));
             else if (f32)
-                DISPATCH_CPL(cpl, ld, launch_rows((long long)L0.A.nnz * k, bk_direction<float, CPL, VEC, false>, red_grid(h, W, G), TPB, 0, st,
+                DISPATCH_CPL(cpl, ld, launch_rows(W, (long long)L0.A.nnz * k, bk_direction<float, CPL, VEC, false>, red_grid(h, W, G), TPB, 0, st,
                                           sv(L0.S), L0.S.val, (const float*)W.Z, W.P, W.Q, k, ld, G, W.partial,
                                           W.ticket, W.sc));
             else
-                DISPATCH_CPL(cpl, ld, launch_rows((long long)L0.A.nnz * k, bk_direction<double, CPL, VEC, false>, red_grid(h, W, G), TPB, 0, st, 
+                DISPATCH_CPL(cpl, ld, launch_rows(W, (long long)L0.A.nnz * k, bk_direction<double, CPL, VEC, false>, red_grid(h, W, G), TPB, 0, st, 
                                           sv(L0.S), L0.S.val, W.Z, W.P, W.Q, k, ld, G, W.partial, W.ticket, W.sc));
             KERNEL_CHECK();
         }
         {
             Scope sc_(&h->prof, st, K_UPDATE_XR, (f32 ? 52.0 : 48.0) * n * k);
-            DISPATCH_CPL(cpl, ld, launch_rows((long long)n * k, bk_update_xr<CPL, VEC>, red_grid(h, W, G), TPB, 0, st, n, W.P, W.Q, X, W.R, r32_of(h), k, ld, G,
+            DISPATCH_CPL(cpl, ld, launch_rows(W, (long long)n * k, bk_update_xr<CPL, VEC>, red_grid(h, W, G), TPB, 0, st, n, W.P, W.Q, X, W.R, r32_of(h), k, ld, G,
                                                                       W.partial, W.ticket, W.sc));
             KERNEL_CHECK();
         }
@@ -1521,7 +1524,7 @@ bool block_check_launch(amg_hierarchy* h, const double* B, double* X, int k) {
     Level& L0 = h->lev[0];
     const double nnz = (double)L0.A.nnz;
     Scope sc_(&h->prof, h->stream, K_RESIDUAL, 12.0 * nnz + 24.0 * L0.A.n * k);
-    DISPATCH_CPL(cpl, W.K, launch_rows((long long)L0.A.nnz * k, bk_residual<CPL, VEC>, red_grid(h, W, G), TPB, 0, h->stream, sv(L0.S), L0.S.val, X, B, W.R, r32_of(h), k,
+    DISPATCH_CPL(cpl, W.K, launch_rows(W, (long long)L0.A.nnz * k, bk_residual<CPL, VEC>, red_grid(h, W, G), TPB, 0, h->stream, sv(L0.S), L0.S.val, X, B, W.R, r32_of(h), k,
                                                                     W.K, G, W.partial, W.ticket, W.sc, 1));
     KERNEL_CHECK();
     copy_state_async(h, W);
@@ -1533,7 +1536,7 @@ void block_report_launch(amg_hierarchy* h, const double* B, const double* X, int
     int G, cpl;
     group_shape(W, k, &G, &cpl);
     Level& L0 = h->lev[0];
-    DISPATCH_CPL(cpl, W.K, launch_rows((long long)L0.A.nnz * k, bk_residual<CPL, VEC>, red_grid(h, W, G), TPB, 0, h->stream, sv(L0.S), L0.S.val, X, B, W.T, nullptr, k, W.K,
+    DISPATCH_CPL(cpl, W.K, launch_rows(W, (long long)L0.A.nnz * k, bk_residual<CPL, VEC>, red_grid(h, W, G), TPB, 0, h->stream, sv(L0.S), L0.S.val, X, B, W.T, nullptr, k, W.K,
                                                                     G, W.partial, W.ticket, W.sc, 2));
     KERNEL_CHECK();
     copy_state_async(h, W);
